@@ -334,3 +334,72 @@ def tolerance(case):
         return {"rel": 5e-3, "max": 0.2}
     # fp32 sums of exact products, up to 14336 of them: 1e-7 to 1.6e-6 from the same sum in 64 bits (largest entry 4.4e-6)
     return {"rel": 6e-6, "max": 2e-5}
+
+
+# ---- the same pass in 64 bits -------------------------------------------------------------------------------------
+
+def _pruned(x, m, tau):
+    """Eq. 2: the difference to the mode where it reaches the threshold (decided in binary32, as the definition says), else 0."""
+    x = x.cuda()
+    if m is None:
+        return torch.where(x.float().abs() >= tau, x.double(), 0.0)
+    return torch.where((x.float() - m).abs() >= tau, x.double() - m.double(), 0.0)
+
+
+def _block64(h, Win, Wout, m1, tau1, b1, m2, tau2, b2, gated):
+    u = _pruned(h, m1, tau1) @ Win.double()
+    if b1 is not None:
+        u = u + b1.double()
+    F = Wout.shape[0]
+    z = torch.nn.functional.silu(u[:, :F]) * u[:, F:] if gated else torch.nn.functional.gelu(u)
+    z32 = z.float()
+    kept = z32.abs() >= tau2 if m2 is None else (z32 - m2).abs() >= tau2
+    d = torch.where(kept, z if m2 is None else z - m2.double(), 0.0)
+    return d @ Wout.double() + b2.double()
+
+
+def exact(case, seed):
+    st, op = prepare(case, seed), case["op"]
+    if op == "calibrate":
+        if case["estimator"] != 0 or case["scope"] != 0:
+            return None
+        # mode: the centre of the fullest of NBINS bins between a channel's extremes, each operation rounded in binary32
+        x = st["x"].float()
+        lo, hi = x.amin(0), x.amax(0)
+        n = torch.full((), float(NBINS), device="cuda")
+        bins = torch.clamp(((x - lo) * (n / (hi - lo))).floor().long(), 0, NBINS - 1)
+        count = torch.zeros(NBINS, case["K"], dtype=torch.int64, device="cuda").scatter_add_(0, bins, torch.ones_like(bins))
+        best = (count == count.amax(0)).to(torch.uint8).argmax(0)  # the lowest of the fullest
+        m = torch.where(hi == lo, lo, lo + (best.float() + 0.5) * ((hi - lo) * (1.0 / NBINS)))
+        # threshold: the pooled quantile, between neighbours in proportion
+        v = (x - m).abs().flatten().sort().values
+        pos = case["sparsity"] * (v.numel() - 1)
+        j = min(int(pos), v.numel() - 2)
+        return [m.double(), (v[j].double() + (pos - j) * (v[j + 1].double() - v[j].double())).reshape(1)]
+    if op == "ffn":
+        return [_block64(b["h"], b["W1"], b["W2"], b["m1"], b["tau1"], b["b1"], b["m2"], b["tau2"], b["b2"], case["gated"]) for b in st["blocks"]]
+    if op == "moe":
+        p = torch.softmax(st["logits"].double(), -1)
+        top, idx = p.topk(case["top_k"], -1)
+        top = top / top.sum(-1, keepdim=True)
+        y = torch.zeros(case["B"], case["D"], dtype=torch.float64, device="cuda")
+        for e, w in enumerate(st["experts"]):
+            rows, slot = (idx == e).nonzero(as_tuple=True)
+            if rows.numel():
+                out = _block64(st["h"][rows], w["Wgu"], w["Wd"], w["m1"], w["tau1"], w["bgu_fused"], w["m2"], w["tau2"], w["bd_fused"], True)
+                y[rows] += top[rows, slot, None] * out
+        return y
+    out = []
+    for a in st["layers"]:
+        if op in ("q8", "q4"):
+            if op == "q8":
+                W = a["Wq"].double() * a["scale"].double()[:, None]
+            else:
+                q = torch.stack((a["Wq"] & 15, a["Wq"] >> 4), -1).flatten(1).double()
+                g = torch.arange(case["K"], device="cuda") // case["group"]
+                W = a["scale"].double()[g] * (q - a["zero"].double()[g])
+        else:
+            W = a["W"].double()
+        d = a["x"].double() if op == "dense" else _pruned(a["x"], a["m"], a["tau"])
+        out.append(d @ W + a["bf"].double())
+    return out
