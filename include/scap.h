@@ -197,8 +197,9 @@ scap_status scap_dense_fc(const void *x, const void *W, const float *b, float *y
  * wscale[K] fp32, one scale per input channel: W[k,n] = wscale[k] * Wq[k,n] (symmetric, no zero point).  x has
  * dtype xdt (fp16 or bf16); everything else as in scap_sparse_fc / scap_dense_fc / scap_fold_bias, with these
  * differences: N must be a multiple of 16; the bias b of the dense call and of the folding is fp32 [N] or
- * NULL; batches of more than two rows are processed two rows at a time (results per row as in scap_sparse_fc;
- * idx_out / nnz_out are only available for B <= 2, else SCAP_ERR_SHAPE).  Workspace: scap_fc_workspace(B, K, N). */
+ * NULL; idx_out / nnz_out are only available for B <= 2, else SCAP_ERR_SHAPE.  Three and more rows (and small layers)
+ * run on the tensor cores - the integers and an exact split of d into three bf16 parts, fp32 accumulation, every row of
+ * Wq read once - where K is a multiple of four; else two rows at a time (results per row as in scap_sparse_fc).  Workspace: scap_fc_workspace(B, K, N). */
 scap_status scap_sparse_fc_q8(const void *x, scap_dtype xdt, const signed char *Wq, const float *wscale, const float *m,
                               const float *tau, const float *b_fused, float *y, int B, int K, int N, uint32_t *idx_out,
                               int *nnz_out, void *ws, size_t ws_bytes, scap_stream_t stream);
@@ -213,9 +214,9 @@ scap_status scap_fold_bias_q8(const signed char *Wq, const float *wscale, const 
  * `group` consecutive INPUT channels share, per output column, scale[K/group rounded up, N] (fp32) and a zero point
  * zero[same shape] (one byte, 0..15):  W[k,n] = scale[k / group, n] * (q[k,n] - zero[k / group, n]).
  * group: a multiple of 32, 32..2048 (else SCAP_ERR_SHAPE); N a multiple of 16.  Everything else - x of dtype xdt, m, tau,
- * b_fused, y, the optional kept list, the batch rule (more than two rows run two at a time; idx_out / nnz_out only for
- * B <= 2), the workspace query - as for the 8-bit calls above.  The sum over the kept channels of one group is formed
- * on the integer codes in fp32 as sum d * q - zero * sum d, and scaled once.                                          */
+ * b_fused, y, the optional kept list, the batch rule (idx_out / nnz_out only for B <= 2), the workspace query - as for
+ * the 8-bit calls above.  The sum over the kept channels of one group is formed on the integer codes in fp32 as
+ * sum d * q - zero * sum d (tensor cores: sum d * (q - 8) - (zero - 8) * sum d), and scaled.                                          */
 scap_status scap_sparse_fc_q4(const void *x, scap_dtype xdt, const unsigned char *Wq, const float *scale,
                               const unsigned char *zero, int group, const float *m, const float *tau, const float *b_fused,
                               float *y, int B, int K, int N, uint32_t *idx_out, int *nnz_out, void *ws, size_t ws_bytes,

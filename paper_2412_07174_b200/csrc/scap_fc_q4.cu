@@ -16,6 +16,7 @@
 #include <type_traits>
 
 #include "scap_fc.cuh"
+#include "scap_qm.cuh"
 
 namespace scap {
 
@@ -386,10 +387,24 @@ static cudaError_t launch_q4_t(const Q4Args &qa, cudaStream_t st) {
     return launch_q4_pu<BT, MODE, XT, fc_pu(BT)>(qa, st);
 }
 
-// xkind: 0 fp16, 1 bf16, 2 float activations.  Batches beyond two rows run two rows at a time (row results are
-// independent; the union mask then spans two rows).
+// Calls that take the tensor-core kernel (tune "dense_stream": 0 none, 2 all it can take).  From three rows on the FMA kernel
+// needs a second launch over the codes (figures in scap_fc_qm.cu).
+// One and two rows: the FMA kernel reads the kept rows only, this one all of them, but its prologue is shorter and it needs
+// no list.  It wins whatever the sparsity while a warp has at most two blocks (K = 2048, N = 4096, one row: 6.0 us against
+// 6.7 - 7.6; at four, K = 4096, N = 4096: 8.1 against 6.7 - 9.2).
+static bool q4_on_tensor_cores(const QmArgs &a) {
+    if (g_tune.dense_stream == 0 || !qm_applicable(4, a)) return false;
+    return g_tune.dense_stream >= 2 || a.f.B >= 3 || qm_blocks_per_warp(a) <= 2;
+}
+
+// xkind: 0 fp16, 1 bf16, 2 float activations.  Batches beyond two rows that the tensor-core kernel
+// cannot take run two rows at a time (row results are independent; the union mask then spans two rows).
 static cudaError_t launch_q4(int mode, int xkind, Q4Args qa, cudaStream_t st) {
     const int B = qa.f.B;
+    QmArgs qm;
+    memset(&qm, 0, sizeof(qm));
+    qm.f = qa.f; qm.scale = qa.scale; qm.zero = qa.zero; qm.group = qa.group;
+    if (xkind != 2 && q4_on_tensor_cores(qm)) return launch_fc_qm(4, mode, xkind, qm, st);
     const size_t xsz = xkind == 2 ? 4 : 2;
     const unsigned char *x0 = static_cast<const unsigned char *>(qa.f.x);
     float *y0 = qa.f.y;

@@ -8,6 +8,7 @@
 #include <string.h>
 
 #include "scap_fc.cuh"
+#include "scap_qm.cuh"
 
 namespace scap {
 
@@ -49,10 +50,25 @@ static cudaError_t launch_q8_t(const FcArgs &a, cudaStream_t st) {
     return launch_q8_pu<BT, MODE, XT, fc_pu(BT)>(a, st);
 }
 
-// xkind: 0 fp16, 1 bf16, 2 float activations.  Batches beyond two rows run two rows at a time (row results are
-// independent; the union mask then spans two rows).
+// Calls that take the tensor-core kernel (tune "dense_stream": 0 none, 2 all it can take).  From three rows on the FMA kernel
+// needs a second launch over the codes (figures in scap_fc_qm.cu; only three or four rows with more than 85 % pruned would be
+// up to 15 % faster in two launches, and the sparsity is not known here).
+// One and two rows: the FMA kernel reads the kept rows only, this one all of them, but its prologue is shorter.  It wins
+// whatever the sparsity only while a warp has a single block (N = 1024, K = 1024, one row: 3.0 us against 3.4 - 3.7; at two
+// blocks, K = 2048, N = 4096: 5.4 against 4.4 - 5.1).
+static bool q8_on_tensor_cores(const QmArgs &a) {
+    if (g_tune.dense_stream == 0 || !qm_applicable(8, a)) return false;
+    return g_tune.dense_stream >= 2 || a.f.B >= 3 || qm_blocks_per_warp(a) <= 1;
+}
+
+// xkind: 0 fp16, 1 bf16, 2 float activations.  Batches beyond two rows that the tensor-core kernel
+// cannot take run two rows at a time (row results are independent; the union mask then spans two rows).
 static cudaError_t launch_q8(int mode, int xkind, FcArgs a, cudaStream_t st) {
     const int B = a.B;
+    QmArgs qm;
+    memset(&qm, 0, sizeof(qm));
+    qm.f = a;
+    if (xkind != 2 && q8_on_tensor_cores(qm)) return launch_fc_qm(8, mode, xkind, qm, st);
     const size_t xsz = xkind == 2 ? 4 : 2;
     const unsigned char *x0 = static_cast<const unsigned char *>(a.x);
     float *y0 = a.y;

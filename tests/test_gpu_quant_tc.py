@@ -1,0 +1,99 @@
+"""The tensor-core kernel of the quantised calls (scap_fc_qm.cu) at the edges of its tiles: remainders of the 16-channel
+blocks, of the 128-column tiles and of the scale groups, every row layout, each activation type, sparse and dense.
+
+Bound: the codes and the three parts of an activation are exact and their products are too, so what is left is the binary32
+sum of K terms: about sqrt(64) roundings of 2^-24 along a chain, against a result that is about sqrt(K) times smaller
+than the sum of the absolute values."""
+import numpy as np
+import pytest
+import torch
+
+import oracle
+import scap_inputs as si
+from scap_testlib import dev, f32, rel_l2_rows, workspace
+
+pytestmark = pytest.mark.gpu
+
+SHAPES = [  # K, N, B, group
+    (20, 16, 3, 32),        # one full and one partial block, one piece of a column tile
+    (64, 144, 1, 32),       # tile and a piece
+    (100, 272, 2, 32),      # a partial last block inside a group
+    (1000, 144, 4, 96),     # groups of an odd number of steps, partial last group
+    (1028, 528, 5, 64),
+    (2052, 400, 8, 128),
+    (516, 1040, 9, 256),    # two halves of the batch, five and four rows
+    (1504, 272, 11, 32),
+    (2304, 784, 16, 2048),  # a group longer than a rank's range
+]
+
+
+@pytest.fixture(scope="module")
+def S():
+    import paper_2412_07174_b200 as scap
+    scap.lib()
+    scap.scap_tune("dense_stream", 2)  # every quantised call that the kernel can take
+    yield scap
+    scap.scap_tune("dense_stream", 1)
+
+
+@pytest.mark.parametrize("bits", [8, 4])
+@pytest.mark.parametrize("K,N,B,group", SHAPES)
+@pytest.mark.parametrize("dt", [si.F16, si.BF16])
+def test_quantised_rows_match_the_oracle(S, bits, K, N, B, group, dt):
+    d = si.laplace_fc(4, K, N, dt, 16, B)
+    x, m, xf = dev(d["x"], dt), d["m_true"], si.to_f32(d["x"], dt)
+    bias = np.linspace(-1, 1, N).astype(np.float32)
+    ws, yg = workspace(S.scap_fc_workspace(B, K, N)), workspace(B * N * 4)
+    y = yg.view(torch.float32, (B, N))
+    if bits == 8:
+        q, scale = si.quantise_q8(d["W"], dt)
+        args = (torch.from_numpy(q).cuda(), f32(scale))
+        sparse, dense = S.scap_sparse_fc_q8, S.scap_dense_fc_q8
+        ref = lambda mm, tau: oracle.sparse_fc_q8(xf, q, scale, mm, tau, bias)  # noqa: E731
+    else:
+        q, scale, zero = si.quantise_q4(d["W"], dt, group)
+        args = (torch.from_numpy(q).cuda(), f32(scale), torch.from_numpy(zero).cuda(), group)
+        sparse, dense = S.scap_sparse_fc_q4, S.scap_dense_fc_q4
+        ref = lambda mm, tau: oracle.sparse_fc_q4(xf, q, scale, zero, group, mm, tau, bias)  # noqa: E731
+    tol = 2.0 ** -24 * 8 * np.sqrt(K)
+    for mm, tau in ((m, 0.25), (None, 0.25)):
+        y.fill_(float("nan"))
+        idx, nnz = (torch.full((n,), -1, dtype=torch.int32, device="cuda") for n in (K, 1))
+        kw = dict(idx_out=idx, nnz_out=nnz) if B <= 2 else {}
+        sparse(x, *args, None if mm is None else f32(mm), f32([tau]), f32(bias), y, ws.payload, **kw)
+        torch.cuda.synchronize()
+        assert ws.intact() and yg.intact()
+        assert rel_l2_rows(y.cpu().numpy(), ref(mm, tau)) <= tol
+        if B <= 2:
+            assert np.array_equal(idx[: int(nnz.item())].cpu().numpy().astype(np.uint32), oracle.mask(xf, mm, tau)[2])
+    y.fill_(float("nan"))
+    dense(x, *args, f32(bias), y, ws.payload)
+    torch.cuda.synchronize()
+    assert yg.intact()
+    assert rel_l2_rows(y.cpu().numpy(), ref(None, 0.0)) <= tol
+
+
+@pytest.mark.parametrize("bits", [8, 4])
+def test_an_infinite_activation_stays_in_its_row(S, bits):
+    """Row 0 holds an infinity, row 1 a NaN that the threshold drops: row 0 is non-finite, the others are as without them."""
+    K, N, B = 256, 144, 3
+    d = si.laplace_fc(4, K, N, si.BF16, 16, B)
+    if bits == 8:
+        q, scale = si.quantise_q8(d["W"], si.BF16)
+        args, fn = (torch.from_numpy(q).cuda(), f32(scale)), S.scap_sparse_fc_q8
+    else:
+        q, scale, zero = si.quantise_q4(d["W"], si.BF16, 32)
+        args, fn = (torch.from_numpy(q).cuda(), f32(scale), torch.from_numpy(zero).cuda(), 32), S.scap_sparse_fc_q4
+    x = dev(d["x"], si.BF16)
+    ws = workspace(S.scap_fc_workspace(B, K, N))
+    out = []
+    for special in (False, True):
+        xs = x.clone()
+        xs[1, 7] = float("nan") if special else 0.0
+        if special:
+            xs[0, 5] = float("inf")
+        y = torch.empty((B, N), dtype=torch.float32, device="cuda")
+        fn(xs, *args, None, f32([0.2]), None, y, ws.payload)
+        out.append(y.cpu())
+    assert torch.equal(out[0][1:], out[1][1:])
+    assert not torch.isfinite(out[1][0]).any()
