@@ -465,7 +465,7 @@ __host__ __device__ constexpr int ds_a_stage(int groups) { return 4 * 2 * groups
 constexpr int DS_OFF_W = 0;
 constexpr int DS_OFF_A = DS_OFF_W + DS_NST * DS_STAGE_W;
 constexpr int DS_OFF_GATHER = DS_OFF_A + DS_NST * ds_a_stage(6) + 2560;  // + slack: the MMA reads 128 rows of M, used or not
-constexpr int DS_OFF_MISC = DS_OFF_GATHER + 16 * TC_TN * 4;
+constexpr int DS_OFF_MISC = DS_OFF_GATHER + 16 * (TC_TN + 16) * 4;  // slices of ceil(columns / S): together up to 12 longer than the tile (GLU, S = 7)
 constexpr int DS_SMEM = DS_OFF_MISC + 512 + 1024;               // misc block + alignment slack
 static_assert(48 * TC_PART_LD * 4 <= DS_NST * DS_STAGE_W, "accumulator copy must fit in the W ring");
 static_assert(2 * (DS_SMEM + 1024) <= 233472, "two CTAs must fit in the shared memory of an SM");
