@@ -232,7 +232,8 @@ scap_status scap_fold_bias_q4(const unsigned char *Wq, const float *scale, const
  * expected to share their pattern, e.g. the beams of one prompt or the tokens of one request: group_of_row_host[b]
  * (a HOST array, read during the call only) is the group 0..15 of row b; at most 16 rows per group (else
  * SCAP_ERR_SHAPE).  Each group is pruned with the union mask of its own rows only and fetches only the weight rows
- * that mask keeps, all groups in one launch; y[b] is the same function of x[b] as in scap_sparse_fc (pruning is per
+ * that mask keeps, all groups in one launch (groups of more than four rows: where it is faster, every weight row is read
+ * once for all groups and pruning is left to the activations); y[b] is the same function of x[b] as in scap_sparse_fc (pruning is per
  * element), whatever the grouping.  No idx / nnz outputs.  Workspace: scap_grouped_workspace() bytes.              */
 size_t scap_grouped_workspace(void);
 scap_status scap_sparse_fc_grouped(const void *x, const void *W, const float *m, const float *tau, const float *b_fused,

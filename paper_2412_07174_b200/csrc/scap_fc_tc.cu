@@ -27,7 +27,7 @@
 
 #include <atomic>
 
-#include "scap_fc.cuh"
+#include "scap_ds.cuh"
 
 namespace scap {
 
@@ -456,24 +456,30 @@ __global__ void __launch_bounds__(FC_THREADS, 2) fc_tc_kernel(const FcArgs a) {
 // MN-major B operand of the MMA, no address arithmetic, one instruction per 8 KB), and pruning happens on the small
 // operand instead: a dropped channel gets a zero activation.  Roles: warp 0 issues the TMA loads, warp 1 the MMAs,
 // warps 2-7 threshold one 32-channel chunk at a time (d = x - m, |d| >= tau, ballot for the mask words, exact split into
-// parts of the weight dtype) and write it as the A operand of its stage; W ring and A ring have DS_NST stages each and
+// parts of the weight dtype) and write it as the A operand of its stage; W ring and A ring have three or four stages each and
 // share the stage's "empty" barrier.  The epilogue is that of the gather kernel.  Every wait is bounded.
 // ------------------------------------------------------------------------------------------------
-constexpr int DS_NST = 4;
+// ROWS = 8 or 16: most batch rows of a call; 32: the rows of a grouped call (scap_grouped.cu), whose operand takes more of the
+// shared memory, so the ring is one stage shorter.
 constexpr int DS_STAGE_W = 64 * TC_TN * 2;                      // 16 KB: two boxes of 64 rows x 64 columns
+__host__ __device__ constexpr int ds_nst(int ROWS) { return ROWS <= 16 ? 4 : 3; }
 __host__ __device__ constexpr int ds_a_stage(int groups) { return 4 * 2 * groups * 128; }  // A operand of 64 channels
 constexpr int DS_OFF_W = 0;
-constexpr int DS_OFF_A = DS_OFF_W + DS_NST * DS_STAGE_W;
-constexpr int DS_OFF_GATHER = DS_OFF_A + DS_NST * ds_a_stage(6) + 2560;  // + slack: the MMA reads 128 rows of M, used or not
-constexpr int DS_OFF_MISC = DS_OFF_GATHER + 16 * (TC_TN + 16) * 4;  // slices of ceil(columns / S): together up to 12 longer than the tile (GLU, S = 7)
-constexpr int DS_SMEM = DS_OFF_MISC + 512 + 1024;               // misc block + alignment slack
-static_assert(48 * TC_PART_LD * 4 <= DS_NST * DS_STAGE_W, "accumulator copy must fit in the W ring");
-static_assert(2 * (DS_SMEM + 1024) <= 233472, "two CTAs must fit in the shared memory of an SM");
+__host__ __device__ constexpr int ds_off_a(int ROWS) { return DS_OFF_W + ds_nst(ROWS) * DS_STAGE_W; }
+__host__ __device__ constexpr int ds_off_gather(int ROWS) {  // + slack: the MMA reads 128 rows of M, used or not
+    return ds_off_a(ROWS) + ds_nst(ROWS) * ds_a_stage(ROWS <= 16 ? 6 : 12) + 2560;
+}
+__host__ __device__ constexpr int ds_gather_rows(int ROWS) { return ROWS <= 16 ? 16 : 32; }
+// (a rank finishes ceil(columns / S) columns, so the slices of all ranks together are up to 12 columns longer than the tile)
+__host__ __device__ constexpr int ds_off_misc(int ROWS) { return ds_off_gather(ROWS) + ds_gather_rows(ROWS) * (TC_TN + 16) * 4; }
+__host__ __device__ constexpr int ds_smem(int ROWS) { return ds_off_misc(ROWS) + 512 + 1024; }  // misc block + alignment slack
+static_assert(48 * TC_PART_LD * 4 <= ds_off_gather(16) && 96 * TC_PART_LD * 4 <= ds_off_gather(32), "accumulator copy must fit in the rings");
+static_assert(2 * (ds_smem(16) + 1024) <= 233472 && 2 * (ds_smem(32) + 1024) <= 233472, "two CTAs must fit in the shared memory of an SM");
 
 struct DsMisc {
-    unsigned long long wfull[DS_NST];   // TMA bytes of the stage have landed
-    unsigned long long afull[DS_NST];   // both chunks of the stage's A operand are written
-    unsigned long long empty[DS_NST];   // the stage's MMAs have read W and A
+    unsigned long long wfull[4];   // TMA bytes of the stage have landed
+    unsigned long long afull[4];   // both chunks of the stage's A operand are written
+    unsigned long long empty[4];   // the stage's MMAs have read W and A
     unsigned long long done;
     unsigned long long recv;            // split-K partials of this rank's columns have landed
     uint32_t tmem_base;
@@ -492,15 +498,27 @@ __device__ __forceinline__ void tma_box_2d(uint32_t dst, const CUtensorMap *map,
                  : "memory");
 }
 
-template <bool BF16, int ROWS, int MODE, typename XT, int EPI>
+// 32 accumulator columns of this warp's 32 lanes (complete after tcgen05.wait::ld).
+__device__ __forceinline__ void tc_ld32(uint32_t (&v)[32], uint32_t addr) {
+    asm volatile(
+        "tcgen05.ld.sync.aligned.32x32b.x32.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15, "
+        "%16, %17, %18, %19, %20, %21, %22, %23, %24, %25, %26, %27, %28, %29, %30, %31}, [%32];"
+        : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]), "=r"(v[7]), "=r"(v[8]),
+          "=r"(v[9]), "=r"(v[10]), "=r"(v[11]), "=r"(v[12]), "=r"(v[13]), "=r"(v[14]), "=r"(v[15]), "=r"(v[16]),
+          "=r"(v[17]), "=r"(v[18]), "=r"(v[19]), "=r"(v[20]), "=r"(v[21]), "=r"(v[22]), "=r"(v[23]), "=r"(v[24]),
+          "=r"(v[25]), "=r"(v[26]), "=r"(v[27]), "=r"(v[28]), "=r"(v[29]), "=r"(v[30]), "=r"(v[31])
+        : "r"(addr));
+}
+
+template <bool BF16, int ROWS, int MODE, typename XT, int EPI, int NACC>
 __global__ void __launch_bounds__(FC_THREADS, 2) fc_ds_kernel(const FcArgs a, const __grid_constant__ CUtensorMap tmap) {
-    constexpr int TNT = TC_TN, HALF = TNT / 2, NSPLIT = mma_nsplit(BF16);
+    constexpr int TNT = TC_TN, HALF = TNT / 2, NSPLIT = mma_nsplit(BF16), NST = ds_nst(ROWS), GR = ds_gather_rows(ROWS);
     extern __shared__ unsigned char smem_raw[];
     unsigned char *smem = reinterpret_cast<unsigned char *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
     unsigned char *s_w = smem + DS_OFF_W;
-    unsigned char *s_a = smem + DS_OFF_A;
-    float *s_gather = reinterpret_cast<float *>(smem + DS_OFF_GATHER);
-    DsMisc *misc = reinterpret_cast<DsMisc *>(smem + DS_OFF_MISC);
+    unsigned char *s_a = smem + ds_off_a(ROWS);
+    float *s_gather = reinterpret_cast<float *>(smem + ds_off_gather(ROWS));
+    DsMisc *misc = reinterpret_cast<DsMisc *>(smem + ds_off_misc(ROWS));
     float *s_part = reinterpret_cast<float *>(s_w);  // accumulator rows, after the stream
     volatile int *abort_flag = &misc->abort;
     const uint32_t spin = a.spin ? (uint32_t)a.spin : TC_SPIN;
@@ -518,7 +536,7 @@ __global__ void __launch_bounds__(FC_THREADS, 2) fc_ds_kernel(const FcArgs a, co
     const int per = ((EPI == EPI_GLU ? HALF : TNT) + S - 1) / S;   // columns (gate/up pairs) a rank finishes
     const uint32_t recv_bar = smem_addr(&misc->recv);
     if (tid == 0) {
-        for (int i = 0; i < DS_NST; ++i) {
+        for (int i = 0; i < NST; ++i) {
             mbar_init(&misc->wfull[i], 1);
             mbar_init(&misc->afull[i], 2);
             mbar_init(&misc->empty[i], 1);
@@ -568,7 +586,7 @@ __global__ void __launch_bounds__(FC_THREADS, 2) fc_ds_kernel(const FcArgs a, co
     // calls.  Everything else (x, m, tau, biases, row maps) is read after the wait.
     const int x0 = EPI == EPI_GLU ? tile * HALF : tile * TNT;
     const int x1 = EPI == EPI_GLU ? a.Nh + tile * HALF : tile * TNT + HALF;
-    const int nq_first = nq < DS_NST ? nq : DS_NST;
+    const int nq_first = nq < NST ? nq : NST;
     if (tid == 0) {
         for (int q = 0; q < nq_first; ++q) {
             mbar_arrive_expect_tx(&misc->wfull[q], DS_STAGE_W);
@@ -578,7 +596,7 @@ __global__ void __launch_bounds__(FC_THREADS, 2) fc_ds_kernel(const FcArgs a, co
         }
     }
     if (warp == 0) {
-        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&misc->tmem_base)), "r"(TNT) : "memory");
+        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&misc->tmem_base)), "r"(NACC * TNT) : "memory");
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
     }
     float bias0[2], bias1[2];
@@ -607,8 +625,8 @@ __global__ void __launch_bounds__(FC_THREADS, 2) fc_ds_kernel(const FcArgs a, co
         if (lane == 0) {
             int q = nq_first;  // the first ring went out above
             for (; q < nq; ++q) {
-                const uint32_t st = (uint32_t)q % DS_NST;
-                if (!mbar_wait(&misc->empty[st], (((uint32_t)q / DS_NST) & 1u) ^ 1u, 1, abort_flag, spin)) break;
+                const uint32_t st = (uint32_t)q % NST;
+                if (!mbar_wait(&misc->empty[st], (((uint32_t)q / NST) & 1u) ^ 1u, 1, abort_flag, spin)) break;
                 mbar_arrive_expect_tx(&misc->wfull[st], DS_STAGE_W);
                 const int row0 = (q * S + s) * 64;
                 const uint32_t dst = smem_u32(s_w) + st * DS_STAGE_W;
@@ -619,8 +637,8 @@ __global__ void __launch_bounds__(FC_THREADS, 2) fc_ds_kernel(const FcArgs a, co
             // this CTA's shared memory: wait for them (fixed limit; they land within microseconds) before anyone leaves.
             if (*abort_flag) {
                 int drain_abort = 0;
-                for (int qq = q > DS_NST ? q - DS_NST : 0; qq < q; ++qq)
-                    mbar_wait(&misc->wfull[(uint32_t)qq % DS_NST], ((uint32_t)qq / DS_NST) & 1u, 5, &drain_abort, TC_SPIN);
+                for (int qq = q > NST ? q - NST : 0; qq < q; ++qq)
+                    mbar_wait(&misc->wfull[(uint32_t)qq % NST], ((uint32_t)qq / NST) & 1u, 5, &drain_abort, TC_SPIN);
             }
         }
         __syncwarp();
@@ -628,7 +646,7 @@ __global__ void __launch_bounds__(FC_THREADS, 2) fc_ds_kernel(const FcArgs a, co
         // ---- MMA issuer: per stage four MMAs of 16 rows
         if (lane == 0) {
             for (int q = 0; q < nq; ++q) {
-                const uint32_t st = (uint32_t)q % DS_NST, par = ((uint32_t)q / DS_NST) & 1u;
+                const uint32_t st = (uint32_t)q % NST, par = ((uint32_t)q / NST) & 1u;
                 if (!mbar_wait(&misc->afull[st], par, 2, abort_flag, spin)) break;
                 if (!mbar_wait(&misc->wfull[st], par, 2, abort_flag, spin)) break;
                 tc_fence_after();
@@ -637,7 +655,10 @@ __global__ void __launch_bounds__(FC_THREADS, 2) fc_ds_kernel(const FcArgs a, co
                 for (uint32_t kb = 0; kb < 4; ++kb) {
                     const uint64_t da = tc_desc(smem_u32(s_a) + st * ASTG + kb * BLK, LBO, 128, 0);
                     const uint64_t db = tc_desc(smem_u32(s_w) + st * DS_STAGE_W + kb * 2048, DS_STAGE_W / 2, 1024, 2);
-                    tc_mma(tmem, da, db, idesc, (q > 0 || kb > 0) ? 1u : 0u);
+                    // NACC = 2: stages alternate between two accumulators.  The tensor core truncates where it adds to one, so half
+                    // the chain is half the error (K = 14336 in eight ranks: 9.5e-7 -> 4.2e-7); plain calls keep to one,
+                    // which is 1 % faster.
+                    tc_mma(tmem + (uint32_t)(q & (NACC - 1)) * TNT, da, db, idesc, (q >= NACC || kb > 0) ? 1u : 0u);
                 }
                 tc_commit(&misc->empty[st]);
             }
@@ -651,60 +672,84 @@ __global__ void __launch_bounds__(FC_THREADS, 2) fc_ds_kernel(const FcArgs a, co
         // activations are one or two 16-byte loads, and the eight positions of a row inside a K half are one 16-byte
         // store per part.  (Rows of x that are not 16-byte aligned - K not a multiple of 8 - take scalar loads.)
         const int pw = warp - 2;
-        constexpr int CPL = ROWS;                   // channels per lane
-        constexpr int XV = CPL * (int)sizeof(XT) / 16;  // 16-byte loads of x per lane
-        const int b = lane % ROWS, cgp = lane / ROWS, ch0 = cgp * CPL;
+        // (32 rows: a lane keeps its row and takes the chunk in four pieces of eight channels, in a rolled loop - unrolled, the
+        // code of a chunk is 16 KB, which the instruction cache does not hold: 72 us a call instead of 36 for 32 rows of 11008 x 4096.)
+        constexpr int CPL = ROWS <= 16 ? ROWS : 8;      // channels per lane and piece
+        constexpr int SUB = ROWS <= 16 ? 1 : 4;         // pieces of a chunk
+        constexpr int XV = CPL * (int)sizeof(XT) / 16;  // 16-byte loads of x per lane and piece
+        const int b = lane % ROWS, ch0 = ROWS <= 16 ? (lane / ROWS) * CPL : 0;
         const bool vec_ok = ((size_t)a.x_ld * sizeof(XT)) % 16 == 0;
         const int xrow = a.in_rows ? misc->rows[b < B ? b : 0] : (b < B ? b : 0);
-        for (int jc = pw; jc < 2 * nq; jc += FC_WARPS - 2) {
-            const int q = jc >> 1, h = jc & 1;
-            const uint32_t st = (uint32_t)q % DS_NST;
-            const int c = 2 * (q * S + s) + h;  // global 32-channel chunk
-            const int k0 = c * 32 + ch0;        // this lane's first channel
-            float xv[CPL], mv[CPL];
+        struct Piece {
+            uint4 raw[XV];
+            float m[CPL];
+        };
+        auto load_piece = [&](Piece &pc, int jc, int u) {
+            const int k0 = (2 * ((jc >> 1) * S + s) + (jc & 1)) * 32 + ch0 + u * CPL;
             if (vec_ok) {
-                uint4 raw[XV];
 #pragma unroll
                 for (int v = 0; v < XV; ++v) {
                     const int kk = k0 + v * (16 / (int)sizeof(XT));
-                    raw[v] = ld_act16_if(reinterpret_cast<const unsigned char *>(xg + (size_t)xrow * a.x_ld + kk), b < B && kk < K, pol_keep);
+                    pc.raw[v] = ld_act16_if(reinterpret_cast<const unsigned char *>(xg + (size_t)xrow * a.x_ld + kk), b < B && kk < K, pol_keep);
                 }
-                const XT *xe = reinterpret_cast<const XT *>(raw);
-#pragma unroll
-                for (int i = 0; i < CPL; ++i) xv[i] = widen1(xe[i]);
             } else {
+                XT e[CPL];
 #pragma unroll
-                for (int i = 0; i < CPL; ++i) xv[i] = widen1(ld_act_if(xg + (size_t)xrow * a.x_ld + k0 + i, b < B && k0 + i < K));
+                for (int i = 0; i < CPL; ++i) e[i] = ld_act_if(xg + (size_t)xrow * a.x_ld + k0 + i, b < B && k0 + i < K);
+                memcpy(pc.raw, e, sizeof(e));
             }
             if (K % 4 == 0) {
 #pragma unroll
                 for (int v = 0; v < CPL / 4; ++v) {
                     uint4 r4 = make_uint4(0, 0, 0, 0);
                     if (MODE == MODE_GATHER && a.m) r4 = ld_act16_if(reinterpret_cast<const unsigned char *>(a.m + k0 + 4 * v), b < B && k0 + 4 * v < K, pol_keep);
-                    mv[4 * v] = __uint_as_float(r4.x); mv[4 * v + 1] = __uint_as_float(r4.y);
-                    mv[4 * v + 2] = __uint_as_float(r4.z); mv[4 * v + 3] = __uint_as_float(r4.w);
+                    pc.m[4 * v] = __uint_as_float(r4.x); pc.m[4 * v + 1] = __uint_as_float(r4.y);
+                    pc.m[4 * v + 2] = __uint_as_float(r4.z); pc.m[4 * v + 3] = __uint_as_float(r4.w);
                 }
             } else {
 #pragma unroll
-                for (int i = 0; i < CPL; ++i) mv[i] = (MODE == MODE_GATHER && a.m) ? ld_act_if(a.m + k0 + i, b < B && k0 + i < K) : 0.0f;
+                for (int i = 0; i < CPL; ++i) pc.m[i] = (MODE == MODE_GATHER && a.m) ? ld_act_if(a.m + k0 + i, b < B && k0 + i < K) : 0.0f;
             }
-            bool go = true;
-            if (lane == 0) go = mbar_wait(&misc->empty[st], (((uint32_t)q / DS_NST) & 1u) ^ 1u, 1, abort_flag, spin);
-            go = __shfl_sync(0xffffffffu, go ? 1 : 0, 0) != 0;
-            if (!go) break;
-            uint32_t mine = 0;
+        };
+        Piece cur, next;
+        if (SUB > 1 && pw < 2 * nq) load_piece(next, pw, 0);
+        uint32_t mine = 0;
+#pragma unroll 1
+        for (int jc = pw, u = 0; jc < 2 * nq;) {
+            const int q = jc >> 1, h = jc & 1;
+            const uint32_t st = (uint32_t)q % NST;
+            const int c = 2 * (q * S + s) + h;  // global 32-channel chunk
+            const int nu = u + 1 == SUB ? 0 : u + 1, nj = u + 1 == SUB ? jc + FC_WARPS - 2 : jc;
+            if constexpr (SUB > 1) {  // a piece ahead: a request takes 1 - 2 us under the weight stream
+                cur = next;
+                if (nj < 2 * nq) load_piece(next, nj, nu);
+            } else {
+                load_piece(cur, jc, 0);
+            }
+            if (u == 0) {
+                bool go = true;
+                if (lane == 0) go = mbar_wait(&misc->empty[st], (((uint32_t)q / NST) & 1u) ^ 1u, 1, abort_flag, spin);
+                go = __shfl_sync(0xffffffffu, go ? 1 : 0, 0) != 0;
+                if (!go) break;
+                mine = 0;
+            }
+            const int chu = ch0 + u * CPL, k0 = c * 32 + chu;  // this lane's first channel of the piece
+            const XT *xe = reinterpret_cast<const XT *>(cur.raw);
             unsigned short part[CPL][3];
+            uint32_t kept_bits = 0;
 #pragma unroll
             for (int i = 0; i < CPL; ++i) {
-                const float dv = (MODE == MODE_GATHER && a.m) ? __fsub_rn(xv[i], mv[i]) : xv[i];
+                const float xv = widen1(xe[i]);
+                const float dv = (MODE == MODE_GATHER && a.m) ? __fsub_rn(xv, cur.m[i]) : xv;
                 const bool kept = b < B && k0 + i < K && (MODE == MODE_DENSE || fabsf(dv) >= tau);
-                mine |= kept ? (1u << i) : 0u;
+                kept_bits |= kept ? (1u << i) : 0u;
                 split_parts<BF16>(kept ? dv : 0.0f, part[i]);
             }
+            mine |= kept_bits << chu;
             if (b < B) {
 #pragma unroll
                 for (int v = 0; v < CPL / 8; ++v) {
-                    const int pos = h * 32 + ch0 + 8 * v;   // first of eight consecutive positions: one K half of one block
+                    const int pos = h * 32 + chu + 8 * v;   // first of eight consecutive positions: one K half of one block
                     unsigned char *dst = s_a + st * ASTG + (size_t)(pos >> 4) * BLK + ((pos >> 3) & 1) * LBO;
 #pragma unroll
                     for (int p = 0; p < NSPLIT; ++p) {
@@ -718,11 +763,17 @@ __global__ void __launch_bounds__(FC_THREADS, 2) fc_ds_kernel(const FcArgs a, co
                     }
                 }
             }
-            const unsigned bal = __reduce_or_sync(0xffffffffu, mine << ch0);   // union over the rows, all 32 channels
-            if (MODE == MODE_GATHER && a.bits && tile == 0 && lane == 0 && c * 32 < K) a.bits[c] = bal;
-            asm volatile("fence.proxy.async.shared::cta;" ::: "memory");  // generic-proxy writes -> visible to the tensor core
-            __syncwarp();
-            if (lane == 0) mbar_arrive(&misc->afull[st]);
+            if (u + 1 == SUB) {
+                if (MODE == MODE_GATHER && a.bits && tile == 0) {
+                    const unsigned bal = __reduce_or_sync(0xffffffffu, mine);   // union over the rows, all 32 channels
+                    if (lane == 0 && c * 32 < K) a.bits[c] = bal;
+                }
+                asm volatile("fence.proxy.async.shared::cta;" ::: "memory");  // generic-proxy writes -> visible to the tensor core
+                __syncwarp();
+                if (lane == 0) mbar_arrive(&misc->afull[st]);
+            }
+            jc = nj;
+            u = nu;
         }
     }
     // ---- all threads: wait until the last MMA has finished
@@ -736,34 +787,28 @@ __global__ void __launch_bounds__(FC_THREADS, 2) fc_ds_kernel(const FcArgs a, co
         int drain_abort = 0;
         mbar_wait(&misc->done, 0, 4, &drain_abort, TC_SPIN);
     }
-    const bool have_acc = nq > 0 && !*abort_flag;
+    const bool have_acc = nq > 0 && !*abort_flag, two = NACC == 2 && nq > 1;
     // Accumulator rows (part p of batch row b = row p B + b = TMEM lane) to shared memory.  A warp reaches the 32 lanes
-    // of its quarter (warp mod 4), so warps 0 and 4 share lanes 0-31 and warps 1 and 5 lanes 32-63, half the columns each.
-    if (have_acc && (warp & 3) * 32 < racc && (warp & 3) < 2) {
+    // of its quarter (warp mod 4), so warps 0 and 4 share lanes 0-31, warps 1 and 5 lanes 32-63 (and so on), half the columns each.
+    if (have_acc && (warp & 3) * 32 < racc) {
         const int lq = warp & 3;
 #pragma unroll 1
         for (int c0 = (warp >> 2) * 64; c0 < (warp >> 2) * 64 + 64; c0 += 32) {
-            uint32_t v[32];
-            asm volatile(
-                "tcgen05.ld.sync.aligned.32x32b.x32.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15, "
-                "%16, %17, %18, %19, %20, %21, %22, %23, %24, %25, %26, %27, %28, %29, %30, %31}, [%32];"
-                : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]), "=r"(v[7]), "=r"(v[8]),
-                  "=r"(v[9]), "=r"(v[10]), "=r"(v[11]), "=r"(v[12]), "=r"(v[13]), "=r"(v[14]), "=r"(v[15]), "=r"(v[16]),
-                  "=r"(v[17]), "=r"(v[18]), "=r"(v[19]), "=r"(v[20]), "=r"(v[21]), "=r"(v[22]), "=r"(v[23]), "=r"(v[24]),
-                  "=r"(v[25]), "=r"(v[26]), "=r"(v[27]), "=r"(v[28]), "=r"(v[29]), "=r"(v[30]), "=r"(v[31])
-                : "r"(tmem + ((uint32_t)(lq * 32) << 16) + (uint32_t)c0));
+            uint32_t v[32], w[32];
+            tc_ld32(v, tmem + ((uint32_t)(lq * 32) << 16) + (uint32_t)c0);
+            if (two) tc_ld32(w, tmem + ((uint32_t)(lq * 32) << 16) + (uint32_t)(TNT + c0));
             asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
             const int r = lq * 32 + lane;
             if (r < racc) {
 #pragma unroll
-                for (int j = 0; j < 32; ++j) s_part[r * TC_PART_LD + c0 + j] = __uint_as_float(v[j]);
+                for (int j = 0; j < 32; ++j) s_part[r * TC_PART_LD + c0 + j] = two ? __uint_as_float(v[j]) + __uint_as_float(w[j]) : __uint_as_float(v[j]);
             }
         }
     }
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
-    if (warp == 0) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(TNT) : "memory");
+    if (warp == 0) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(NACC * TNT) : "memory");
     // ---- cluster exchange, push form: the parts of an element are added (smallest first) and the sum goes straight to
     // the cluster rank that finishes its column - slot (this rank, row) of that rank's gather buffer - as an asynchronous
     // store that counts down the owner's barrier.  No cluster-wide barrier after the prologue: a rank finishes its columns
@@ -777,11 +822,11 @@ __global__ void __launch_bounds__(FC_THREADS, 2) fc_ds_kernel(const FcArgs a, co
         if constexpr (EPI == EPI_GLU) {
             const int j = c % HALF, hf = c / HALF;
             r = j / per;
-            slot0 = (s * 16 * 2 + hf) * per + (j - r * per);
+            slot0 = (s * GR * 2 + hf) * per + (j - r * per);
             bstride = 2 * per;
         } else {
             r = c / per;
-            slot0 = s * 16 * per + (c - r * per);
+            slot0 = s * GR * per + (c - r * per);
             bstride = per;
         }
         const uint32_t dst0 = S > 1 ? cluster_addr(smem_addr(s_gather) + 4u * (uint32_t)slot0, (uint32_t)r) : 0u;
@@ -803,7 +848,7 @@ __global__ void __launch_bounds__(FC_THREADS, 2) fc_ds_kernel(const FcArgs a, co
     } else {
         __syncthreads();
     }
-    finish_columns<BF16, 16, EPI, TNT>(a, tile, s, per, s_gather, bias0, bias1);
+    finish_columns<BF16, GR, EPI, TNT>(a, tile, s, per, s_gather, bias0, bias1);
 }
 
 // ---- host side ------------------------------------------------------------------------------------------------
@@ -913,13 +958,13 @@ static bool ds_tensor_map(CUtensorMap *map, const void *W, int K, int ldw, bool 
               CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
-template <bool BF16, int ROWS, int MODE, typename XT, int EPI>
+template <bool BF16, int ROWS, int MODE, typename XT, int EPI, int NACC = 1>
 static cudaError_t launch_ds_r(const FcArgs &a, const CUtensorMap &map, cudaStream_t st) {
     static SmemOptIn opt_in;
-    auto kern = fc_ds_kernel<BF16, ROWS, MODE, XT, EPI>;
-    cudaError_t e0 = ensure_dynamic_smem(kern, DS_SMEM, opt_in);
+    auto kern = fc_ds_kernel<BF16, ROWS, MODE, XT, EPI, NACC>;
+    cudaError_t e0 = ensure_dynamic_smem(kern, ds_smem(ROWS), opt_in);
     if (e0 != cudaSuccess) return e0;
-    return launch_cluster(kern, dim3(fc_tiles(a.Nh, EPI, TC_TN), a.S), dim3(FC_THREADS), DS_SMEM, a.S, st, g_tune.pdl != 0, a, map);
+    return launch_cluster(kern, dim3(fc_tiles(a.Nh, EPI, TC_TN), a.S), dim3(FC_THREADS), ds_smem(ROWS), a.S, st, g_tune.pdl != 0, a, map);
 }
 template <bool BF16, int MODE, typename XT, int EPI>
 static cudaError_t launch_ds_t(const FcArgs &a, const CUtensorMap &map, cudaStream_t st) {
@@ -965,6 +1010,20 @@ cudaError_t launch_fc_ds(bool bf16, int mode, int xkind, int epi, const FcArgs &
     CUtensorMap map;
     if (!ds_tensor_map(&map, a.W, a.K, a.ldw, bf16)) return cudaErrorNotSupported;
     return bf16 ? launch_ds_w<true>(mode, xkind, epi, a, map, st) : launch_ds_w<false>(mode, xkind, epi, a, map, st);
+}
+
+// The rows of a grouped call, up to 32 of them, in one pass over the weight.
+cudaError_t launch_fc_ds_grouped(bool bf16, const FcArgs &a, cudaStream_t st) {
+    CUtensorMap map;
+    if (!ds_tensor_map(&map, a.W, a.K, a.ldw, bf16)) return cudaErrorNotSupported;
+    if (bf16) {
+        if (a.B <= 8) return launch_ds_r<true, 8, MODE_GATHER, __nv_bfloat16, EPI_BIAS, 2>(a, map, st);
+        if (a.B <= 16) return launch_ds_r<true, 16, MODE_GATHER, __nv_bfloat16, EPI_BIAS, 2>(a, map, st);
+        return launch_ds_r<true, 32, MODE_GATHER, __nv_bfloat16, EPI_BIAS, 2>(a, map, st);
+    }
+    if (a.B <= 8) return launch_ds_r<false, 8, MODE_GATHER, __half, EPI_BIAS, 2>(a, map, st);
+    if (a.B <= 16) return launch_ds_r<false, 16, MODE_GATHER, __half, EPI_BIAS, 2>(a, map, st);
+    return launch_ds_r<false, 32, MODE_GATHER, __half, EPI_BIAS, 2>(a, map, st);
 }
 
 cudaError_t launch_fc_tc(bool bf16, int mode, int xkind, int epi, const FcArgs &a, cudaStream_t st) {

@@ -5,7 +5,7 @@
 // fetches only the weight rows its own rows keep.  Up to 64 rows in up to 16 groups of at most 16 rows.
 #include <string.h>
 
-#include "scap_fc.cuh"
+#include "scap_ds.cuh"
 
 namespace scap {
 
@@ -112,6 +112,35 @@ scap_status scap_sparse_fc_grouped(const void *x, const void *W, const float *m,
     if (stt != SCAP_OK) return stt;
 
     cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
+    // Groups of more than four rows would take the mma.sync body, one gather per group: the weight crosses the chip once per
+    // group.  The dense-stream kernel reads every row once per 32 rows of the batch, prunes on the activations (which is per
+    // element, so the grouping changes nothing in y), and its time does not depend on the masks.  (Groups of up to four rows
+    // stay on the FMA bodies, whose sums round to nearest.)  Gather -> stream, overlap 0.9, 50 % / 80 % pruned, us:
+    //   11008 x 4096   2 x 6 rows 40 / 32 -> 22   4 x 8 rows 73 / 58 -> 36   8 x 8 rows 135 / 104 -> 71
+    //    2048 x 1024   2 x 6 rows 12 / 12 ->  8   4 x 8 rows 14 / 12 -> 11   8 x 8 rows  16 /  14 -> 21
+    //   14336 x 2048   2 x 6 rows 35 / 30 -> 24   4 x 8 rows 53 / 43 -> 42   8 x 8 rows  92 /  71 -> 82
+    // Above 16 rows it is bound by the preparation of the activations, which takes two CTAs on most SMs to hide, while the
+    // groups of a gather fill an empty chip themselves: there it needs a full grid, or a short layer and one pass.
+    const int s_ds = ds_choose_split(K, N, EPI_BIAS);
+    const bool full_grid = 2 * fc_tiles(N, EPI_BIAS, 128) * s_ds >= 3 * sm_count();
+    if (max_nb > 4 && g_tune.dense_stream != 0 && K >= 64 && (B <= 16 || full_grid || (B <= 32 && K <= 4096))) {
+        FcArgs f;
+        memset(&f, 0, sizeof(f));
+        f.W = W; f.K = K; f.ldw = N; f.Nh = N; f.tn = 128; f.x_ld = K; f.m = m; f.tau = tau; f.bias = b_fused; f.y_ld = N;
+        f.S = s_ds;
+        f.spin = g_tune.tc_spin;
+        f.status = tc_status_ptr();
+        const int passes = (B + 31) / 32;
+        for (int p = 0, b0 = 0; p < passes; ++p) {
+            f.B = (B - b0 + passes - p - 1) / (passes - p);
+            f.x = static_cast<const unsigned char *>(x) + (size_t)b0 * K * 2;
+            f.y = y + (size_t)b0 * N;
+            const cudaError_t e = launch_fc_ds_grouped(dt == SCAP_BF16, f, st);
+            if (e != cudaSuccess) return cuda_status(e);
+            b0 += f.B;
+        }
+        return SCAP_OK;
+    }
     GroupedArgs a;
     memset(&a, 0, sizeof(a));
     a.f.W = W; a.f.K = K; a.f.ldw = N; a.f.Nh = N;
