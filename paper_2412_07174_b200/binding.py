@@ -1,4 +1,7 @@
-"""ctypes binding of libscap_b200.so: same names as the C ABI, marshalling only."""
+"""Binding of libscap_b200.so: same names as the C ABI, marshalling only.
+
+The decode calls go through a small native helper (csrc/scap_pycall.c), the others through ctypes: at one token the host
+bounds a call, and marshalling was most of it (scap_sparse_fc, K = N = 1024, one row: 10.5 -> 5.3 us a call, 4.1 us on the device)."""
 from __future__ import annotations
 
 import ctypes as C
@@ -46,6 +49,8 @@ def lib_path() -> str:
 
 
 _lib = None
+_call = None    # call(address, arg, ...) of the native helper
+_entry = {}     # name -> address of the entry point
 
 
 def lib():
@@ -118,8 +123,21 @@ def lib():
     L.scap_moe_workspace.restype = sz
     L.scap_moe_ffn.argtypes = [vp, vp, C.POINTER(ScapExpert), i, i, vp, i, i, i, i, vp, vp, vp, sz, vp]
     L.scap_moe_ffn.restype = i
+    from ._scap_call import call
+    _entry.update({n: C.cast(getattr(L, n), C.c_void_p).value for n in EXPORTS})
+    global _call
+    _call = call
     _lib = L
     return L
+
+
+def _invoke(name: str, *args) -> None:
+    """Calls the entry point `name`; an argument is a tensor (its address), an address, an integer or None."""
+    if _lib is None:
+        lib()
+    code = _call(_entry[name], *args)
+    if code != 0:
+        raise ScapError(code, name)
 
 
 def status_string(code: int) -> str:
@@ -155,22 +173,26 @@ def _ptr(t):
 
 def _stream(stream):
     if stream is None:
+        if torch.cuda.is_initialized():  # the current stream of the current device, without a Stream object
+            return torch._C._cuda_getCurrentRawStream(torch._C._cuda_getDevice())
         return torch.cuda.current_stream().cuda_stream
     if isinstance(stream, int):
         return stream
     return stream.cuda_stream
 
 
+_DTYPES = {torch.float16: SCAP_F16, torch.bfloat16: SCAP_BF16}
+
+
 def dtype_of(t: torch.Tensor) -> int:
-    if t.dtype == torch.float16:
-        return SCAP_F16
-    if t.dtype == torch.bfloat16:
-        return SCAP_BF16
+    code = _DTYPES.get(t.dtype)
+    if code is not None:
+        return code
     raise TypeError("weights/activations must be float16 or bfloat16, got %s" % t.dtype)
 
 
 def _ws(ws):
-    return (_ptr(ws), ws.numel() * ws.element_size()) if ws is not None else (None, 0)
+    return (ws.data_ptr(), ws.nbytes) if ws is not None else (None, 0)
 
 
 def scap_calibrate_workspace(T: int, K: int, nbins: int) -> int:
@@ -214,16 +236,14 @@ def scap_sparse_fc(x, W, m, tau, b_fused, y, ws, idx_out=None, nnz_out=None, str
     B, K = x.shape
     N = W.shape[1]
     p, n = _ws(ws)
-    _check(lib().scap_sparse_fc(_ptr(x), _ptr(W), _ptr(m), _ptr(tau), _ptr(b_fused), _ptr(y), B, K, N, dtype_of(W),
-                                _ptr(idx_out), _ptr(nnz_out), p, n, _stream(stream)), "scap_sparse_fc")
+    _invoke("scap_sparse_fc", x, W, m, tau, b_fused, y, B, K, N, dtype_of(W), idx_out, nnz_out, p, n, _stream(stream))
 
 
 def scap_dense_fc(x, W, b, y, ws, stream=None) -> None:
     B, K = x.shape
     N = W.shape[1]
     p, n = _ws(ws)
-    _check(lib().scap_dense_fc(_ptr(x), _ptr(W), _ptr(b), _ptr(y), B, K, N, dtype_of(W), p, n, _stream(stream)),
-           "scap_dense_fc")
+    _invoke("scap_dense_fc", x, W, b, y, B, K, N, dtype_of(W), p, n, _stream(stream))
 
 
 def scap_sparse_fc_q8(x, Wq, wscale, m, tau, b_fused, y, ws, idx_out=None, nnz_out=None, stream=None) -> None:
@@ -231,16 +251,14 @@ def scap_sparse_fc_q8(x, Wq, wscale, m, tau, b_fused, y, ws, idx_out=None, nnz_o
     B, K = x.shape
     N = Wq.shape[1]
     p, n = _ws(ws)
-    _check(lib().scap_sparse_fc_q8(_ptr(x), dtype_of(x), _ptr(Wq), _ptr(wscale), _ptr(m), _ptr(tau), _ptr(b_fused), _ptr(y), B, K, N,
-                                   _ptr(idx_out), _ptr(nnz_out), p, n, _stream(stream)), "scap_sparse_fc_q8")
+    _invoke("scap_sparse_fc_q8", x, dtype_of(x), Wq, wscale, m, tau, b_fused, y, B, K, N, idx_out, nnz_out, p, n, _stream(stream))
 
 
 def scap_dense_fc_q8(x, Wq, wscale, b, y, ws, stream=None) -> None:
     B, K = x.shape
     N = Wq.shape[1]
     p, n = _ws(ws)
-    _check(lib().scap_dense_fc_q8(_ptr(x), dtype_of(x), _ptr(Wq), _ptr(wscale), _ptr(b), _ptr(y), B, K, N, p, n, _stream(stream)),
-           "scap_dense_fc_q8")
+    _invoke("scap_dense_fc_q8", x, dtype_of(x), Wq, wscale, b, y, B, K, N, p, n, _stream(stream))
 
 
 def scap_fold_bias_q8(Wq, wscale, m, b, b_fused, ws, stream=None) -> None:
@@ -255,16 +273,15 @@ def scap_sparse_fc_q4(x, Wq, scale, zero, group, m, tau, b_fused, y, ws, idx_out
     B, K = x.shape
     N = Wq.shape[1] * 2
     p, n = _ws(ws)
-    _check(lib().scap_sparse_fc_q4(_ptr(x), dtype_of(x), _ptr(Wq), _ptr(scale), _ptr(zero), int(group), _ptr(m), _ptr(tau), _ptr(b_fused),
-                                   _ptr(y), B, K, N, _ptr(idx_out), _ptr(nnz_out), p, n, _stream(stream)), "scap_sparse_fc_q4")
+    _invoke("scap_sparse_fc_q4", x, dtype_of(x), Wq, scale, zero, int(group), m, tau, b_fused, y, B, K, N, idx_out, nnz_out, p, n,
+            _stream(stream))
 
 
 def scap_dense_fc_q4(x, Wq, scale, zero, group, b, y, ws, stream=None) -> None:
     B, K = x.shape
     N = Wq.shape[1] * 2
     p, n = _ws(ws)
-    _check(lib().scap_dense_fc_q4(_ptr(x), dtype_of(x), _ptr(Wq), _ptr(scale), _ptr(zero), int(group), _ptr(b), _ptr(y), B, K, N, p, n,
-                                  _stream(stream)), "scap_dense_fc_q4")
+    _invoke("scap_dense_fc_q4", x, dtype_of(x), Wq, scale, zero, int(group), b, y, B, K, N, p, n, _stream(stream))
 
 
 def scap_fold_bias_q4(Wq, scale, zero, group, m, b, b_fused, ws, stream=None) -> None:
@@ -284,8 +301,7 @@ def scap_sparse_fc_grouped(x, W, m, tau, b_fused, y, groups, ws, stream=None) ->
     N = W.shape[1]
     p, n = _ws(ws)
     arr = (C.c_int * B)(*[int(g) for g in groups])
-    _check(lib().scap_sparse_fc_grouped(_ptr(x), _ptr(W), _ptr(m), _ptr(tau), _ptr(b_fused), _ptr(y), B, K, N, dtype_of(W), arr, p, n,
-                                        _stream(stream)), "scap_sparse_fc_grouped")
+    _invoke("scap_sparse_fc_grouped", x, W, m, tau, b_fused, y, B, K, N, dtype_of(W), C.addressof(arr), p, n, _stream(stream))
 
 
 def scap_fc_host_workspace(B: int, K: int, N: int) -> int:
@@ -297,8 +313,7 @@ def scap_sparse_fc_host(x_host, W, m, tau, b_fused, y_host, ws, stream=None) -> 
     B, K = x_host.shape
     N = W.shape[1]
     p, n = _ws(ws)
-    _check(lib().scap_sparse_fc_host(_ptr(x_host), _ptr(W), _ptr(m), _ptr(tau), _ptr(b_fused), _ptr(y_host), B, K, N,
-                                     dtype_of(W), p, n, _stream(stream)), "scap_sparse_fc_host")
+    _invoke("scap_sparse_fc_host", x_host, W, m, tau, b_fused, y_host, B, K, N, dtype_of(W), p, n, _stream(stream))
 
 
 def scap_glu_workspace(B: int, D: int, F: int) -> int:
@@ -310,9 +325,8 @@ def scap_glu_ffn(h, Wgu, Wd, m1, tau1, bgu_fused, m2, tau2, bd_fused, y, ws, z_o
     B, D = h.shape
     F = Wd.shape[0]
     p, n = _ws(ws)
-    _check(lib().scap_glu_ffn(_ptr(h), _ptr(Wgu), _ptr(Wd), _ptr(m1), _ptr(tau1), _ptr(bgu_fused), _ptr(m2), _ptr(tau2),
-                              _ptr(bd_fused), _ptr(y), B, D, F, dtype_of(Wgu), _ptr(z_out), _ptr(idx1_out), _ptr(nnz1_out),
-                              _ptr(idx2_out), _ptr(nnz2_out), p, n, _stream(stream)), "scap_glu_ffn")
+    _invoke("scap_glu_ffn", h, Wgu, Wd, m1, tau1, bgu_fused, m2, tau2, bd_fused, y, B, D, F, dtype_of(Wgu), z_out, idx1_out, nnz1_out,
+            idx2_out, nnz2_out, p, n, _stream(stream))
 
 
 def scap_gelu_ffn_workspace(B: int, D: int, F: int) -> int:
@@ -324,9 +338,8 @@ def scap_gelu_ffn(h, Wu, Wd, m1, tau1, bu_fused, m2, tau2, bd_fused, y, ws, z_ou
     B, D = h.shape
     F = Wd.shape[0]
     p, n = _ws(ws)
-    _check(lib().scap_gelu_ffn(_ptr(h), _ptr(Wu), _ptr(Wd), _ptr(m1), _ptr(tau1), _ptr(bu_fused), _ptr(m2), _ptr(tau2),
-                               _ptr(bd_fused), _ptr(y), B, D, F, dtype_of(Wu), _ptr(z_out), _ptr(idx1_out), _ptr(nnz1_out),
-                               _ptr(idx2_out), _ptr(nnz2_out), p, n, _stream(stream)), "scap_gelu_ffn")
+    _invoke("scap_gelu_ffn", h, Wu, Wd, m1, tau1, bu_fused, m2, tau2, bd_fused, y, B, D, F, dtype_of(Wu), z_out, idx1_out, nnz1_out,
+            idx2_out, nnz2_out, p, n, _stream(stream))
 
 
 def scap_glu_static_capacity() -> int:
@@ -337,9 +350,7 @@ def scap_glu_ffn_static(h, Wgu, Wd, m1, tau1, bgu_fused, m2, tau2, bd_fused, y, 
     """scap_glu_ffn for callers that may not allocate: the scratch is a fixed array inside the library (see scap.h)."""
     B, D = h.shape
     F = Wd.shape[0]
-    _check(lib().scap_glu_ffn_static(_ptr(h), _ptr(Wgu), _ptr(Wd), _ptr(m1), _ptr(tau1), _ptr(bgu_fused), _ptr(m2),
-                                     _ptr(tau2), _ptr(bd_fused), _ptr(y), B, D, F, dtype_of(Wgu), _ptr(z_out),
-                                     _stream(stream)), "scap_glu_ffn_static")
+    _invoke("scap_glu_ffn_static", h, Wgu, Wd, m1, tau1, bgu_fused, m2, tau2, bd_fused, y, B, D, F, dtype_of(Wgu), z_out, _stream(stream))
 
 
 def scap_moe_workspace(B: int, D: int, F: int, E: int, top_k: int) -> int:

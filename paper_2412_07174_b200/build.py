@@ -6,12 +6,14 @@ import glob
 import os
 import subprocess
 import sys
+import sysconfig
 
 HERE = os.path.dirname(os.path.abspath(__file__))
 ROOT = os.path.dirname(HERE)
 CSRC = os.path.join(HERE, "csrc")
 OBJ = os.path.join(HERE, "_build")
 LIB = os.path.join(HERE, "libscap_b200.so")
+CALL = os.path.join(HERE, "_scap_call.so")  # the binding's call helper
 
 # no --use_fast_math: the mask arithmetic must round exactly as documented
 NVCC_FLAGS = ["-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo", "-O3", "-std=c++17", "-Xcompiler", "-fPIC"]
@@ -57,6 +59,11 @@ def build(force: bool = False, verbose: bool = False) -> str:
         subprocess.check_call([nvcc, "-gencode", "arch=compute_100a,code=sm_100a", "--shared", "-cudart", "static",
                                "-o", tmp, *objs])
         os.replace(tmp, LIB)
+    src = os.path.join(CSRC, "scap_pycall.c")
+    if force or _newer(CALL, [src]):
+        tmp = CALL + ".tmp.%d" % os.getpid()
+        subprocess.check_call([os.environ.get("CC", "gcc"), "-O2", "-shared", "-fPIC", "-I", sysconfig.get_paths()["include"], src, "-o", tmp])
+        os.replace(tmp, CALL)
     return LIB
 
 
