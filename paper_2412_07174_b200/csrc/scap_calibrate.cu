@@ -29,6 +29,7 @@ __device__ __forceinline__ void widen8(const uint4 &v, float (&f)[8]) {
 // Rows t0, t0 + CAL_ROWS, ... (CAL_U of them) of this thread's 8 channels, all loads in flight together; rows at or
 // beyond T are skipped (their slots keep zeros and `valid` says how many are real).
 constexpr int CAL_U = 16;  // with 128 rows per sweep: 2048 rows of a strip live in registers at once
+template <int CAL_U>
 __device__ __forceinline__ int load_rows(const uint16_t *xp, int K, int T, int t0, uint4 (&v)[CAL_U]) {
     const uint64_t pol = l2_policy_keep();  // the radix passes read the tensor again: it fits in L2, ask for it to stay
     int valid = 0;
@@ -76,7 +77,12 @@ __device__ __forceinline__ uint4 rotate_channels(const uint4 &v, int r) {
 // pieces (16 rows x 2 pieces) of 8 channels; each lane rotates its 8 channels by its row number, so that in every
 // step of the unrolled loop the lanes of a warp update CWT different channels: with 32 channels no two lanes ever
 // meet in a bank, whatever the bins; with 16 channels two lanes can.
-template <bool BF16, int CWT>
+//
+// U = 16-byte loads per thread that the passes are unrolled for (128 U rows live in registers).  The code of a pass grows
+// with U whether or not there are that many rows, and one CTA runs it once, straight through the instruction cache: up to
+// 1024 rows eight are faster (whole call, us, 16 -> 8: 128 x 1024 20.5 -> 17.1, 512 x 4096 34.9 -> 33.5), beyond they would
+// read the strip again in every pass (2048 x 14336: 127 -> 141).
+template <bool BF16, int CWT, int U>
 __global__ void __launch_bounds__(CWT * 16, CWT == 16 ? 2 : 1) mode_kernel(const uint16_t *__restrict__ x, int T, int K, int nbins,
                                                            float *__restrict__ m_out, uint32_t *__restrict__ hist_a,
                                                            int want_hist, const float *__restrict__ m_given) {
@@ -94,10 +100,10 @@ __global__ void __launch_bounds__(CWT * 16, CWT == 16 ? 2 : 1) mode_kernel(const
     const int kc = k0 + q * 8;
     const bool ok = kc < K;  // K is a multiple of 8
     const uint16_t *xp = x + kc;
-    // Up to CAL_ROWS * CAL_U = 2048 rows: the strip is read once, all loads in flight together, and the three
+    // Up to CAL_ROWS * U = 2048 rows: the strip is read once, all loads in flight together, and the three
     // passes below run from registers; longer inputs are re-read per pass (from L2 when they fit).
-    const bool resident = T <= CAL_ROWS * CAL_U;
-    uint4 v[CAL_U];
+    const bool resident = T <= CAL_ROWS * U;
+    uint4 v[U];
     int nv = 0;
     if (resident && ok) nv = load_rows(xp, K, T, rl, v);
 
@@ -110,10 +116,10 @@ __global__ void __launch_bounds__(CWT * 16, CWT == 16 ? 2 : 1) mode_kernel(const
 #pragma unroll
         for (int j = 0; j < 8; ++j) { lo[j] = INFINITY; hi[j] = -INFINITY; }
         if (ok)
-            for (int t0 = rl; t0 < T; t0 += CAL_ROWS * CAL_U) {
+            for (int t0 = rl; t0 < T; t0 += CAL_ROWS * U) {
                 if (!resident) nv = load_rows(xp, K, T, t0, v);
 #pragma unroll
-                for (int u = 0; u < CAL_U; ++u) {
+                for (int u = 0; u < U; ++u) {
                     if (u < nv) {
                         float f[8];
                         widen8<BF16>(v[u], f);
@@ -159,10 +165,10 @@ __global__ void __launch_bounds__(CWT * 16, CWT == 16 ? 2 : 1) mode_kernel(const
             scale[i] = hi[i] != lo[i] ? __fdiv_rn((float)nbins, __fsub_rn(hi[i], lo[i])) : 0.0f;
         }
         if (ok)
-            for (int t0 = rl; t0 < T; t0 += CAL_ROWS * CAL_U) {
+            for (int t0 = rl; t0 < T; t0 += CAL_ROWS * U) {
                 if (!resident) nv = load_rows(xp, K, T, t0, v);
 #pragma unroll
-                for (int u = 0; u < CAL_U; ++u) {
+                for (int u = 0; u < U; ++u) {
                     if (u < nv) {
                         float f[8];
                         widen8<BF16>(rotate_channels(v[u], r), f);
@@ -249,10 +255,10 @@ __global__ void __launch_bounds__(CWT * 16, CWT == 16 ? 2 : 1) mode_kernel(const
     const int cp = lane & 3;  // copy of this lane
     uint32_t *hq = smem + cp * RADIX_BINS;
     if (ok)
-        for (int t0 = rl; t0 < T; t0 += CAL_ROWS * CAL_U) {
+        for (int t0 = rl; t0 < T; t0 += CAL_ROWS * U) {
             if (!resident) nv = load_rows(xp, K, T, t0, v);
 #pragma unroll
-            for (int u = 0; u < CAL_U; ++u) {
+            for (int u = 0; u < U; ++u) {
                 if (u < nv) {
                     float f[8];
                     widen8<BF16>(v[u], f);
@@ -536,7 +542,10 @@ __device__ __forceinline__ void find_rank256(const uint32_t *h, uint32_t r, int 
 }
 
 // Median per channel: two 8-bit radix passes over the 16-bit keys of a strip of CW channels, from registers.
+// Eight loads per thread: longer inputs are read again for the second pass, but the unrolled passes stay in the instruction
+// cache (median and threshold of 2048 x 14336: 208 us with sixteen, 166 with eight).
 // Shared memory: hi[CW][256] | lo[2][CW][256] counters | per-channel bucket state.
+constexpr int MED_U = 8;
 template <bool BF16>
 __global__ void __launch_bounds__(CAL_THREADS) median_kernel(const uint16_t *__restrict__ x, int T, int K, float *__restrict__ m_out) {
     extern __shared__ __align__(16) uint32_t smem[];
@@ -546,18 +555,18 @@ __global__ void __launch_bounds__(CAL_THREADS) median_kernel(const uint16_t *__r
     const int k0 = blockIdx.x * CW, kc = k0 + q * 8;
     const bool ok = kc < K;
     const uint16_t *xp = x + kc;
-    const bool resident = T <= CAL_ROWS * CAL_U;
-    uint4 v[CAL_U];
+    const bool resident = T <= CAL_ROWS * MED_U;
+    uint4 v[MED_U];
     int nv = 0;
     if (resident && ok) nv = load_rows(xp, K, T, rl, v);
     for (int i = tid; i < 3 * CW * 256; i += CAL_THREADS) smem[i] = 0;
     __syncthreads();
     // pass A: high byte
     if (ok)
-        for (int t0 = rl; t0 < T; t0 += CAL_ROWS * CAL_U) {
+        for (int t0 = rl; t0 < T; t0 += CAL_ROWS * MED_U) {
             if (!resident) nv = load_rows(xp, K, T, t0, v);
 #pragma unroll
-            for (int u = 0; u < CAL_U; ++u) {
+            for (int u = 0; u < MED_U; ++u) {
                 if (u < nv) {
                     const uint32_t w[4] = {v[u].x, v[u].y, v[u].z, v[u].w};
 #pragma unroll
@@ -580,10 +589,10 @@ __global__ void __launch_bounds__(CAL_THREADS) median_kernel(const uint16_t *__r
     __syncthreads();
     // pass B: low byte inside the two buckets
     if (ok)
-        for (int t0 = rl; t0 < T; t0 += CAL_ROWS * CAL_U) {
+        for (int t0 = rl; t0 < T; t0 += CAL_ROWS * MED_U) {
             if (!resident) nv = load_rows(xp, K, T, t0, v);
 #pragma unroll
-            for (int u = 0; u < CAL_U; ++u) {
+            for (int u = 0; u < MED_U; ++u) {
                 if (u < nv) {
                     const uint32_t w[4] = {v[u].x, v[u].y, v[u].z, v[u].w};
 #pragma unroll
@@ -943,17 +952,22 @@ static scap_status calibrate_t(const uint16_t *x, int T, int K, double sparsity,
     const int cw = g_tune.cal_strip;  // 16 or 32 channels per CTA
     size_t smem = (size_t)cw * HW * 4;
     if (smem < (size_t)4 * RADIX_BINS * 4) smem = (size_t)4 * RADIX_BINS * 4;  // the four copies of the first radix histogram
-    static SmemOptIn opt_in32, opt_in16;
+    static SmemOptIn opt_in32, opt_in16, opt_in16s;
     const float *given = own_mode ? (const float *)nullptr : (const float *)m_out;
-    if (cw == 16) {
-        e = ensure_dynamic_smem(mode_kernel<BF16, 16>, 2048 / 2 * 16 * 4, opt_in16);
+    if (cw == 16 && T <= CAL_ROWS * 8) {
+        e = ensure_dynamic_smem(mode_kernel<BF16, 16, 8>, 2048 / 2 * 16 * 4, opt_in16s);
         if (e != cudaSuccess) return cuda_status(e);
-        e = launch(mode_kernel<BF16, 16>, dim3((K + 15) / 16), dim3(256), smem, st, pdl, x, T, K, nbins, m_out, hist,
+        e = launch(mode_kernel<BF16, 16, 8>, dim3((K + 15) / 16), dim3(256), smem, st, pdl, x, T, K, nbins, m_out, hist,
+                   want_tau ? 1 : 0, given);
+    } else if (cw == 16) {
+        e = ensure_dynamic_smem(mode_kernel<BF16, 16, CAL_U>, 2048 / 2 * 16 * 4, opt_in16);
+        if (e != cudaSuccess) return cuda_status(e);
+        e = launch(mode_kernel<BF16, 16, CAL_U>, dim3((K + 15) / 16), dim3(256), smem, st, pdl, x, T, K, nbins, m_out, hist,
                    want_tau ? 1 : 0, given);
     } else {
-        e = ensure_dynamic_smem(mode_kernel<BF16, 32>, 2048 / 2 * 32 * 4, opt_in32);
+        e = ensure_dynamic_smem(mode_kernel<BF16, 32, CAL_U>, 2048 / 2 * 32 * 4, opt_in32);
         if (e != cudaSuccess) return cuda_status(e);
-        e = launch(mode_kernel<BF16, 32>, dim3((K + 31) / 32), dim3(512), smem, st, pdl, x, T, K, nbins, m_out, hist,
+        e = launch(mode_kernel<BF16, 32, CAL_U>, dim3((K + 31) / 32), dim3(512), smem, st, pdl, x, T, K, nbins, m_out, hist,
                    want_tau ? 1 : 0, given);
     }
     if (e != cudaSuccess) return cuda_status(e);
