@@ -672,108 +672,179 @@ __global__ void __launch_bounds__(FC_THREADS, 2) fc_ds_kernel(const FcArgs a, co
         // activations are one or two 16-byte loads, and the eight positions of a row inside a K half are one 16-byte
         // store per part.  (Rows of x that are not 16-byte aligned - K not a multiple of 8 - take scalar loads.)
         const int pw = warp - 2;
-        // (32 rows: a lane keeps its row and takes the chunk in four pieces of eight channels, in a rolled loop - unrolled, the
-        // code of a chunk is 16 KB, which the instruction cache does not hold: 72 us a call instead of 36 for 32 rows of 11008 x 4096.)
-        constexpr int CPL = ROWS <= 16 ? ROWS : 8;      // channels per lane and piece
-        constexpr int SUB = ROWS <= 16 ? 1 : 4;         // pieces of a chunk
-        constexpr int XV = CPL * (int)sizeof(XT) / 16;  // 16-byte loads of x per lane and piece
-        const int b = lane % ROWS, ch0 = ROWS <= 16 ? (lane / ROWS) * CPL : 0;
-        const bool vec_ok = ((size_t)a.x_ld * sizeof(XT)) % 16 == 0;
-        const int xrow = a.in_rows ? misc->rows[b < B ? b : 0] : (b < B ? b : 0);
-        struct Piece {
-            uint4 raw[XV];
-            float m[CPL];
-        };
-        auto load_piece = [&](Piece &pc, int jc, int u) {
-            const int k0 = (2 * ((jc >> 1) * S + s) + (jc & 1)) * 32 + ch0 + u * CPL;
-            if (vec_ok) {
+        if constexpr (ROWS <= 16) {
+            constexpr int CPL = ROWS;                   // channels per lane
+            constexpr int XV = CPL * (int)sizeof(XT) / 16;  // 16-byte loads of x per lane
+            const int b = lane % ROWS, cgp = lane / ROWS, ch0 = cgp * CPL;
+            const bool vec_ok = ((size_t)a.x_ld * sizeof(XT)) % 16 == 0;
+            const int xrow = a.in_rows ? misc->rows[b < B ? b : 0] : (b < B ? b : 0);
+            for (int jc = pw; jc < 2 * nq; jc += FC_WARPS - 2) {
+                const int q = jc >> 1, h = jc & 1;
+                const uint32_t st = (uint32_t)q % NST;
+                const int c = 2 * (q * S + s) + h;  // global 32-channel chunk
+                const int k0 = c * 32 + ch0;        // this lane's first channel
+                float xv[CPL], mv[CPL];
+                if (vec_ok) {
+                    uint4 raw[XV];
 #pragma unroll
-                for (int v = 0; v < XV; ++v) {
-                    const int kk = k0 + v * (16 / (int)sizeof(XT));
-                    pc.raw[v] = ld_act16_if(reinterpret_cast<const unsigned char *>(xg + (size_t)xrow * a.x_ld + kk), b < B && kk < K, pol_keep);
+                    for (int v = 0; v < XV; ++v) {
+                        const int kk = k0 + v * (16 / (int)sizeof(XT));
+                        raw[v] = ld_act16_if(reinterpret_cast<const unsigned char *>(xg + (size_t)xrow * a.x_ld + kk), b < B && kk < K, pol_keep);
+                    }
+                    const XT *xe = reinterpret_cast<const XT *>(raw);
+#pragma unroll
+                    for (int i = 0; i < CPL; ++i) xv[i] = widen1(xe[i]);
+                } else {
+#pragma unroll
+                    for (int i = 0; i < CPL; ++i) xv[i] = widen1(ld_act_if(xg + (size_t)xrow * a.x_ld + k0 + i, b < B && k0 + i < K));
                 }
-            } else {
-                XT e[CPL];
+                if (K % 4 == 0) {
 #pragma unroll
-                for (int i = 0; i < CPL; ++i) e[i] = ld_act_if(xg + (size_t)xrow * a.x_ld + k0 + i, b < B && k0 + i < K);
-                memcpy(pc.raw, e, sizeof(e));
-            }
-            if (K % 4 == 0) {
+                    for (int v = 0; v < CPL / 4; ++v) {
+                        uint4 r4 = make_uint4(0, 0, 0, 0);
+                        if (MODE == MODE_GATHER && a.m) r4 = ld_act16_if(reinterpret_cast<const unsigned char *>(a.m + k0 + 4 * v), b < B && k0 + 4 * v < K, pol_keep);
+                        mv[4 * v] = __uint_as_float(r4.x); mv[4 * v + 1] = __uint_as_float(r4.y);
+                        mv[4 * v + 2] = __uint_as_float(r4.z); mv[4 * v + 3] = __uint_as_float(r4.w);
+                    }
+                } else {
 #pragma unroll
-                for (int v = 0; v < CPL / 4; ++v) {
-                    uint4 r4 = make_uint4(0, 0, 0, 0);
-                    if (MODE == MODE_GATHER && a.m) r4 = ld_act16_if(reinterpret_cast<const unsigned char *>(a.m + k0 + 4 * v), b < B && k0 + 4 * v < K, pol_keep);
-                    pc.m[4 * v] = __uint_as_float(r4.x); pc.m[4 * v + 1] = __uint_as_float(r4.y);
-                    pc.m[4 * v + 2] = __uint_as_float(r4.z); pc.m[4 * v + 3] = __uint_as_float(r4.w);
+                    for (int i = 0; i < CPL; ++i) mv[i] = (MODE == MODE_GATHER && a.m) ? ld_act_if(a.m + k0 + i, b < B && k0 + i < K) : 0.0f;
                 }
-            } else {
-#pragma unroll
-                for (int i = 0; i < CPL; ++i) pc.m[i] = (MODE == MODE_GATHER && a.m) ? ld_act_if(a.m + k0 + i, b < B && k0 + i < K) : 0.0f;
-            }
-        };
-        Piece cur, next;
-        if (SUB > 1 && pw < 2 * nq) load_piece(next, pw, 0);
-        uint32_t mine = 0;
-#pragma unroll 1
-        for (int jc = pw, u = 0; jc < 2 * nq;) {
-            const int q = jc >> 1, h = jc & 1;
-            const uint32_t st = (uint32_t)q % NST;
-            const int c = 2 * (q * S + s) + h;  // global 32-channel chunk
-            const int nu = u + 1 == SUB ? 0 : u + 1, nj = u + 1 == SUB ? jc + FC_WARPS - 2 : jc;
-            if constexpr (SUB > 1) {  // a piece ahead: a request takes 1 - 2 us under the weight stream
-                cur = next;
-                if (nj < 2 * nq) load_piece(next, nj, nu);
-            } else {
-                load_piece(cur, jc, 0);
-            }
-            if (u == 0) {
                 bool go = true;
                 if (lane == 0) go = mbar_wait(&misc->empty[st], (((uint32_t)q / NST) & 1u) ^ 1u, 1, abort_flag, spin);
                 go = __shfl_sync(0xffffffffu, go ? 1 : 0, 0) != 0;
                 if (!go) break;
-                mine = 0;
-            }
-            const int chu = ch0 + u * CPL, k0 = c * 32 + chu;  // this lane's first channel of the piece
-            const XT *xe = reinterpret_cast<const XT *>(cur.raw);
-            unsigned short part[CPL][3];
-            uint32_t kept_bits = 0;
+                uint32_t mine = 0;
+                unsigned short part[CPL][3];
 #pragma unroll
-            for (int i = 0; i < CPL; ++i) {
-                const float xv = widen1(xe[i]);
-                const float dv = (MODE == MODE_GATHER && a.m) ? __fsub_rn(xv, cur.m[i]) : xv;
-                const bool kept = b < B && k0 + i < K && (MODE == MODE_DENSE || fabsf(dv) >= tau);
-                kept_bits |= kept ? (1u << i) : 0u;
-                split_parts<BF16>(kept ? dv : 0.0f, part[i]);
-            }
-            mine |= kept_bits << chu;
-            if (b < B) {
+                for (int i = 0; i < CPL; ++i) {
+                    const float dv = (MODE == MODE_GATHER && a.m) ? __fsub_rn(xv[i], mv[i]) : xv[i];
+                    const bool kept = b < B && k0 + i < K && (MODE == MODE_DENSE || fabsf(dv) >= tau);
+                    mine |= kept ? (1u << i) : 0u;
+                    split_parts<BF16>(kept ? dv : 0.0f, part[i]);
+                }
+                if (b < B) {
 #pragma unroll
-                for (int v = 0; v < CPL / 8; ++v) {
-                    const int pos = h * 32 + chu + 8 * v;   // first of eight consecutive positions: one K half of one block
-                    unsigned char *dst = s_a + st * ASTG + (size_t)(pos >> 4) * BLK + ((pos >> 3) & 1) * LBO;
+                    for (int v = 0; v < CPL / 8; ++v) {
+                        const int pos = h * 32 + ch0 + 8 * v;   // first of eight consecutive positions: one K half of one block
+                        unsigned char *dst = s_a + st * ASTG + (size_t)(pos >> 4) * BLK + ((pos >> 3) & 1) * LBO;
 #pragma unroll
-                    for (int p = 0; p < NSPLIT; ++p) {
-                        const int r = p * B + b;
-                        uint4 w;
-                        w.x = (uint32_t)part[8 * v + 0][p] | ((uint32_t)part[8 * v + 1][p] << 16);
-                        w.y = (uint32_t)part[8 * v + 2][p] | ((uint32_t)part[8 * v + 3][p] << 16);
-                        w.z = (uint32_t)part[8 * v + 4][p] | ((uint32_t)part[8 * v + 5][p] << 16);
-                        w.w = (uint32_t)part[8 * v + 6][p] | ((uint32_t)part[8 * v + 7][p] << 16);
-                        *reinterpret_cast<uint4 *>(dst + (r >> 3) * 128 + (r & 7) * 16) = w;
+                        for (int p = 0; p < NSPLIT; ++p) {
+                            const int r = p * B + b;
+                            uint4 w;
+                            w.x = (uint32_t)part[8 * v + 0][p] | ((uint32_t)part[8 * v + 1][p] << 16);
+                            w.y = (uint32_t)part[8 * v + 2][p] | ((uint32_t)part[8 * v + 3][p] << 16);
+                            w.z = (uint32_t)part[8 * v + 4][p] | ((uint32_t)part[8 * v + 5][p] << 16);
+                            w.w = (uint32_t)part[8 * v + 6][p] | ((uint32_t)part[8 * v + 7][p] << 16);
+                            *reinterpret_cast<uint4 *>(dst + (r >> 3) * 128 + (r & 7) * 16) = w;
+                        }
                     }
                 }
-            }
-            if (u + 1 == SUB) {
-                if (MODE == MODE_GATHER && a.bits && tile == 0) {
-                    const unsigned bal = __reduce_or_sync(0xffffffffu, mine);   // union over the rows, all 32 channels
-                    if (lane == 0 && c * 32 < K) a.bits[c] = bal;
-                }
+                const unsigned bal = __reduce_or_sync(0xffffffffu, mine << ch0);   // union over the rows, all 32 channels
+                if (MODE == MODE_GATHER && a.bits && tile == 0 && lane == 0 && c * 32 < K) a.bits[c] = bal;
                 asm volatile("fence.proxy.async.shared::cta;" ::: "memory");  // generic-proxy writes -> visible to the tensor core
                 __syncwarp();
                 if (lane == 0) mbar_arrive(&misc->afull[st]);
             }
-            jc = nj;
-            u = nu;
+        } else {
+            // 32 rows: a lane keeps its row and takes the chunk in four pieces of eight channels, in a rolled loop - unrolled, the
+            // code of a chunk is 16 KB, which the instruction cache does not hold: 72 us a call instead of 36 for 32 rows of 11008 x 4096.
+            constexpr int CPL = 8, SUB = 4;                 // channels per piece, pieces per chunk
+            constexpr int XV = CPL * (int)sizeof(XT) / 16;  // 16-byte loads of x per lane and piece
+            const int b = lane;
+            const bool vec_ok = ((size_t)a.x_ld * sizeof(XT)) % 16 == 0;
+            const int xrow = a.in_rows ? misc->rows[b < B ? b : 0] : (b < B ? b : 0);
+            struct Piece {
+                uint4 raw[XV];
+                float m[CPL];
+            };
+            auto load_piece = [&](Piece &pc, int jc, int u) {
+                const int k0 = (2 * ((jc >> 1) * S + s) + (jc & 1)) * 32 + u * CPL;
+                if (vec_ok) {
+#pragma unroll
+                    for (int v = 0; v < XV; ++v) {
+                        const int kk = k0 + v * (16 / (int)sizeof(XT));
+                        pc.raw[v] = ld_act16_if(reinterpret_cast<const unsigned char *>(xg + (size_t)xrow * a.x_ld + kk), b < B && kk < K, pol_keep);
+                    }
+                } else {
+                    XT e[CPL];
+#pragma unroll
+                    for (int i = 0; i < CPL; ++i) e[i] = ld_act_if(xg + (size_t)xrow * a.x_ld + k0 + i, b < B && k0 + i < K);
+                    memcpy(pc.raw, e, sizeof(e));
+                }
+                if (K % 4 == 0) {
+#pragma unroll
+                    for (int v = 0; v < CPL / 4; ++v) {
+                        uint4 r4 = make_uint4(0, 0, 0, 0);
+                        if (MODE == MODE_GATHER && a.m) r4 = ld_act16_if(reinterpret_cast<const unsigned char *>(a.m + k0 + 4 * v), b < B && k0 + 4 * v < K, pol_keep);
+                        pc.m[4 * v] = __uint_as_float(r4.x); pc.m[4 * v + 1] = __uint_as_float(r4.y);
+                        pc.m[4 * v + 2] = __uint_as_float(r4.z); pc.m[4 * v + 3] = __uint_as_float(r4.w);
+                    }
+                } else {
+#pragma unroll
+                    for (int i = 0; i < CPL; ++i) pc.m[i] = (MODE == MODE_GATHER && a.m) ? ld_act_if(a.m + k0 + i, b < B && k0 + i < K) : 0.0f;
+                }
+            };
+            Piece cur, next;
+            if (pw < 2 * nq) load_piece(next, pw, 0);
+            uint32_t mine = 0;
+#pragma unroll 1
+            for (int jc = pw, u = 0; jc < 2 * nq;) {
+                const int q = jc >> 1, h = jc & 1;
+                const uint32_t st = (uint32_t)q % NST;
+                const int c = 2 * (q * S + s) + h;  // global 32-channel chunk
+                const int nu = u + 1 == SUB ? 0 : u + 1, nj = u + 1 == SUB ? jc + FC_WARPS - 2 : jc;
+                cur = next;  // asked for a piece ahead: a request takes 1 - 2 us under the weight stream
+                if (nj < 2 * nq) load_piece(next, nj, nu);
+                if (u == 0) {
+                    bool go = true;
+                    if (lane == 0) go = mbar_wait(&misc->empty[st], (((uint32_t)q / NST) & 1u) ^ 1u, 1, abort_flag, spin);
+                    go = __shfl_sync(0xffffffffu, go ? 1 : 0, 0) != 0;
+                    if (!go) break;
+                    mine = 0;
+                }
+                const int chu = u * CPL, k0 = c * 32 + chu;  // this lane's first channel of the piece
+                const XT *xe = reinterpret_cast<const XT *>(cur.raw);
+                unsigned short part[CPL][3];
+                uint32_t kept_bits = 0;
+#pragma unroll
+                for (int i = 0; i < CPL; ++i) {
+                    const float xv = widen1(xe[i]);
+                    const float dv = (MODE == MODE_GATHER && a.m) ? __fsub_rn(xv, cur.m[i]) : xv;
+                    const bool kept = b < B && k0 + i < K && (MODE == MODE_DENSE || fabsf(dv) >= tau);
+                    kept_bits |= kept ? (1u << i) : 0u;
+                    split_parts<BF16>(kept ? dv : 0.0f, part[i]);
+                }
+                mine |= kept_bits << chu;
+                if (b < B) {
+#pragma unroll
+                    for (int v = 0; v < CPL / 8; ++v) {
+                        const int pos = h * 32 + chu + 8 * v;   // first of eight consecutive positions: one K half of one block
+                        unsigned char *dst = s_a + st * ASTG + (size_t)(pos >> 4) * BLK + ((pos >> 3) & 1) * LBO;
+#pragma unroll
+                        for (int p = 0; p < NSPLIT; ++p) {
+                            const int r = p * B + b;
+                            uint4 w;
+                            w.x = (uint32_t)part[8 * v + 0][p] | ((uint32_t)part[8 * v + 1][p] << 16);
+                            w.y = (uint32_t)part[8 * v + 2][p] | ((uint32_t)part[8 * v + 3][p] << 16);
+                            w.z = (uint32_t)part[8 * v + 4][p] | ((uint32_t)part[8 * v + 5][p] << 16);
+                            w.w = (uint32_t)part[8 * v + 6][p] | ((uint32_t)part[8 * v + 7][p] << 16);
+                            *reinterpret_cast<uint4 *>(dst + (r >> 3) * 128 + (r & 7) * 16) = w;
+                        }
+                    }
+                }
+                if (u + 1 == SUB) {
+                    if (MODE == MODE_GATHER && a.bits && tile == 0) {
+                        const unsigned bal = __reduce_or_sync(0xffffffffu, mine);   // union over the rows, all 32 channels
+                        if (lane == 0 && c * 32 < K) a.bits[c] = bal;
+                    }
+                    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");  // generic-proxy writes -> visible to the tensor core
+                    __syncwarp();
+                    if (lane == 0) mbar_arrive(&misc->afull[st]);
+                }
+                jc = nj;
+                u = nu;
+            }
         }
     }
     // ---- all threads: wait until the last MMA has finished
