@@ -36,8 +36,9 @@
  *     scap_fold_bias, or any kernel or copy of the caller's), with no further synchronisation.  The weight matrix W
  *     is the exception: it is a constant of the layer and must be complete in device memory when the call is
  *     ISSUED (not written by work still pending on the stream), because kernels that know their first weight rows
- *     without looking at the activations (the batch 5..16 kernel, the dense calls, a sparse call with "head_rows"
- *     set) request them before that wait, so that the memory system does not idle between consecutive calls.  Consecutive calls overlap where they can: a kernel may
+ *     without looking at the activations (the batch 5..16 kernel, also on 8- and 4-bit codes and on the rows of a
+ *     grouped call; the dense calls, a sparse call with "head_rows" set) request them before that wait, so that the
+ *     memory system does not idle between consecutive calls.  Consecutive calls overlap where they can: a kernel may
  *     become resident and set up its shared memory while its predecessor drains (programmatic dependent launch,
  *     "pdl" below).
  */
@@ -199,7 +200,8 @@ scap_status scap_dense_fc(const void *x, const void *W, const float *b, float *y
  * differences: N must be a multiple of 16; the bias b of the dense call and of the folding is fp32 [N] or
  * NULL; idx_out / nnz_out are only available for B <= 2, else SCAP_ERR_SHAPE.  Three and more rows (and small layers)
  * run on the tensor cores - the integers and an exact split of d into three bf16 parts, fp32 accumulation, every row of
- * Wq read once - where K is a multiple of four; else two rows at a time (results per row as in scap_sparse_fc).  Workspace: scap_fc_workspace(B, K, N). */
+ * Wq read once - where K is a multiple of four; else two rows at a time (results per row as in scap_sparse_fc).
+ * Workspace: scap_fc_workspace(B, K, N). */
 scap_status scap_sparse_fc_q8(const void *x, scap_dtype xdt, const signed char *Wq, const float *wscale, const float *m,
                               const float *tau, const float *b_fused, float *y, int B, int K, int N, uint32_t *idx_out,
                               int *nnz_out, void *ws, size_t ws_bytes, scap_stream_t stream);
