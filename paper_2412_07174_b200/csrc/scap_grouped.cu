@@ -96,7 +96,7 @@ scap_status scap_sparse_fc_grouped(const void *x, const void *W, const float *m,
     if (ws_bytes < scap_grouped_workspace()) return SCAP_ERR_WORKSPACE;
     GroupTable t;
     memset(&t, 0, sizeof(t));
-    int groups = 0, max_nb = 0, active = 0;
+    int groups = 0, max_nb = 0, min_nb = SCAP_MAX_BATCH, active = 0;
     for (int b = 0; b < B; ++b) {
         const int g = group_of_row_host[b];
         if (g < 0 || g >= GR_MAX_GROUPS) return SCAP_ERR_INVALID_ARG;
@@ -106,6 +106,7 @@ scap_status scap_sparse_fc_grouped(const void *x, const void *W, const float *m,
     }
     for (int g = 0; g < groups; ++g) {
         if (t.nb[g] > max_nb) max_nb = t.nb[g];
+        if (t.nb[g] > 0 && t.nb[g] < min_nb) min_nb = t.nb[g];
         active += t.nb[g] > 0;
     }
     scap_status stt = check_device();
@@ -114,8 +115,9 @@ scap_status scap_sparse_fc_grouped(const void *x, const void *W, const float *m,
     cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
     // Groups of more than four rows would take the mma.sync body, one gather per group: the weight crosses the chip once per
     // group.  The dense-stream kernel reads every row once per 32 rows of the batch, prunes on the activations (which is per
-    // element, so the grouping changes nothing in y), and its time does not depend on the masks.  (Groups of up to four rows
-    // stay on the FMA bodies, whose sums round to nearest.)  Gather -> stream, overlap 0.9, 50 % / 80 % pruned, us:
+    // element, so the grouping changes nothing in y), and its time does not depend on the masks.  (A call with a group of up
+    // to four rows stays on the gather: such a group runs on the FMA bodies there, in binary32 and rounded to nearest, and
+    // what a row gets does not depend on the size of another row's group.)  Gather -> stream, overlap 0.9, 50 % / 80 % pruned, us:
     //   11008 x 4096   2 x 6 rows 40 / 32 -> 22   4 x 8 rows 73 / 58 -> 36   8 x 8 rows 135 / 104 -> 71
     //    2048 x 1024   2 x 6 rows 12 / 12 ->  8   4 x 8 rows 14 / 12 -> 11   8 x 8 rows  16 /  14 -> 21
     //   14336 x 2048   2 x 6 rows 35 / 30 -> 24   4 x 8 rows 53 / 43 -> 42   8 x 8 rows  92 /  71 -> 82
@@ -123,7 +125,7 @@ scap_status scap_sparse_fc_grouped(const void *x, const void *W, const float *m,
     // groups of a gather fill an empty chip themselves: there it needs a full grid, or a short layer and one pass.
     const int s_ds = ds_choose_split(K, N, EPI_BIAS);
     const bool full_grid = 2 * fc_tiles(N, EPI_BIAS, 128) * s_ds >= 3 * sm_count();
-    if (max_nb > 4 && g_tune.dense_stream != 0 && K >= 64 && (B <= 16 || full_grid || (B <= 32 && K <= 4096))) {
+    if (min_nb > 4 && g_tune.dense_stream != 0 && K >= 64 && (B <= 16 || full_grid || (B <= 32 && K <= 4096))) {
         FcArgs f;
         memset(&f, 0, sizeof(f));
         f.W = W; f.K = K; f.ldw = N; f.Nh = N; f.tn = 128; f.x_ld = K; f.m = m; f.tau = tau; f.bias = b_fused; f.y_ld = N;

@@ -36,3 +36,40 @@ def test_large_groups_match_the_oracle(K, N, B, n_ctx, dt):
     S.scap_device_status()
     assert ws.intact() and yg.intact()
     assert rel_l2_rows(y.cpu().numpy(), y64) <= 2.0 ** -23 * 8 * np.sqrt(K)
+
+
+@pytest.mark.parametrize("dt", [si.F16, si.BF16])
+@pytest.mark.parametrize("sizes", [(1, 3, 8), (2, 16, 4, 4), (5, 1)])
+def test_groups_of_up_to_four_rows_keep_binary32_beside_larger_ones(dt, sizes):
+    """A row's arithmetic does not depend on the size of another row's group.  Up to four rows a group is multiplied in binary32:
+    |x - m| beyond the range of fp16 is no overflow, and entries far below 1 keep all their bits.
+
+    Bound: a sum goes through at most about 40 roundings (rows of a row group, row groups, ranks), each 2^-24 / sqrt(3) rms of a
+    partial sum that has on average half the variance of the whole: 2^-24 sqrt(40 / 6), twice that for the worst row."""
+    import paper_2412_07174_b200 as S
+    K, N, B = 1024, 264, sum(sizes)
+    BOUND = 2.0 ** -24 * 2 * np.sqrt(40 / 6)
+    rng = np.random.default_rng(3)
+    groups = rng.permutation(np.repeat(np.arange(len(sizes)), sizes))
+    small = np.array([sizes[g] <= 4 for g in groups])
+    m = rng.uniform(-0.01, 0.01, K).astype(np.float32)
+    x = m + rng.laplace(0.0, 0.01, (B, K))
+    x[:, ::7] = m[::7]                                 # pruned
+    m[3] = si.to_f32(si.to_bits(np.array([-60000.0]), dt), dt)[0]
+    x[:, 3] = np.where(small, 60000.0, m[3])           # |x - m| = 120000 where the group is small
+    d = si.laplace_fc(4, K, N, dt, 16, 1)
+    bits = si.to_bits(x, dt)
+    xf = si.to_f32(bits, dt)
+    W, tau = d["W"], 0.001
+    y64 = oracle.sparse_fc(xf, W, dt, m, tau, None, threads=8)
+    ws, y = workspace(S.scap_grouped_workspace()), torch.full((B, N), float("nan"), device="cuda")
+    S.scap_sparse_fc_grouped(dev(bits, dt), dev(W, dt), f32(m), f32([tau]), None, y, groups.tolist(), ws.payload)
+    torch.cuda.synchronize()
+    assert ws.intact() and np.isfinite(y.cpu().numpy()[small]).all()
+    assert rel_l2_rows(y.cpu().numpy()[small], y64[small]) <= BOUND
+    # the same without the one large channel, beside which the others do not count
+    bits[:, 3] = bits[~small][0, 3]
+    y64 = oracle.sparse_fc(si.to_f32(bits, dt), W, dt, m, tau, None, threads=8)
+    S.scap_sparse_fc_grouped(dev(bits, dt), dev(W, dt), f32(m), f32([tau]), None, y, groups.tolist(), ws.payload)
+    torch.cuda.synchronize()
+    assert rel_l2_rows(y.cpu().numpy()[small], y64[small]) <= BOUND
