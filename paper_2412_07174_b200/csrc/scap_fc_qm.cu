@@ -165,7 +165,9 @@ __global__ void __launch_bounds__(FC_THREADS, 2) fc_qm_kernel(const QmArgs qa) {
     prefetch_bias<true, EPI_BIAS, QM_TN>(a, tile, s, per, bias0, bias1);
     const int gb = WB == 4 ? qa.group >> 4 : 1;  // blocks per scale group
     const int g_lo = r_lo / gb;                  // first group of the rank
+    bool careful = false;                        // a scale of the rank is not finite
     if constexpr (WB == 4) {
+        bool odd = false;
         const int ng = r_n > 0 ? (r_lo + r_n - 1) / gb - g_lo + 1 : 0;
         for (int i = tid; i < ng * 40; i += FC_THREADS) {
             const int gi = i / 40, p = i - gi * 40;
@@ -174,8 +176,10 @@ __global__ void __launch_bounds__(FC_THREADS, 2) fc_qm_kernel(const QmArgs qa) {
             const size_t at = (size_t)(g_lo + gi) * N + tile * QM_TN + c;
             const uint4 v = ld_act16_if(p < 32 ? (const void *)(qa.scale + at) : (const void *)(qa.zero + at), on);
             *reinterpret_cast<uint4 *>(p < 32 ? s_scale + (size_t)(gi * QM_TN + c) * 4 : s_zero + (size_t)(gi * QM_TN + c)) = v;
+            const uint32_t top = max(max(v.x << 1, v.y << 1), max(v.z << 1, v.w << 1));
+            odd |= p < 32 && top >= 0xff000000u;
         }
-        __syncthreads();
+        careful = __syncthreads_or(odd) != 0;
     }
 
     float acc[NS][NP][4], ds[NS][4], y[WB == 4 ? NS : 1][WB == 4 ? NP : 1][4];
@@ -204,8 +208,8 @@ __global__ void __launch_bounds__(FC_THREADS, 2) fc_qm_kernel(const QmArgs qa) {
             if constexpr (MODE == MODE_GATHER) v = __fsub_rn(v, mv[i]);  // (m == NULL: zeros)
             const bool on = k_ok && (MODE == MODE_DENSE || fabsf(v) >= tau);
             kept |= on ? 1u << i : 0u;
-            v = on ? v : 0.0f;
             if constexpr (WB == 8) v = __fmul_rn(v, cv[i]);
+            v = on ? v : 0.0f;  // (after the scale: that of a dropped channel has no part in y, whatever it is)
             // three consecutive 8-bit fields of the significand; an infinity stays one part (its rest would be NaN)
             hi[i] = __float_as_uint(v) & 0xffff0000u;
             float rest = v - __uint_as_float(hi[i]);
@@ -266,8 +270,9 @@ __global__ void __launch_bounds__(FC_THREADS, 2) fc_qm_kernel(const QmArgs qa) {
             mma_all(ds[0], ds[NS - 1], ones);
         }
     };
-    // 4-bit: y += scale (sum d (q - 8) - (zero - 8) sum d), once per group (and warp)
-    auto flush = [&](int blk) {
+    // 4-bit: y += scale (sum d (q - 8) - (zero - 8) sum d), once per group (and warp).  The scale of a group that a row has dropped
+    // has no part in y, whatever it is: where a scale is not finite, sums of zero are left out (checking always: 2 % at groups of 32).
+    auto flush_as = [&](int blk, auto careful_tag) {
         const int gi = blk / gb - g_lo;
         const float *sc = reinterpret_cast<const float *>(s_scale) + gi * QM_TN + lcol;
         const unsigned char *zp = s_zero + gi * QM_TN + lcol;
@@ -280,7 +285,8 @@ __global__ void __launch_bounds__(FC_THREADS, 2) fc_qm_kernel(const QmArgs qa) {
             for (int q = 0; q < NS; ++q)
 #pragma unroll
                 for (int i = 0; i < 4; ++i) {
-                    y[q][j][i] = fmaf(i < 2 ? sv.x : sv.y, fmaf(i < 2 ? z0 : z1, ds[q][i & 1], acc[q][j][i]), y[q][j][i]);
+                    const float sum = fmaf(i < 2 ? z0 : z1, ds[q][i & 1], acc[q][j][i]);
+                    if (!decltype(careful_tag)::value || sum != 0.0f) y[q][j][i] = fmaf(i < 2 ? sv.x : sv.y, sum, y[q][j][i]);
                     acc[q][j][i] = 0.0f;
                 }
         }
@@ -288,6 +294,10 @@ __global__ void __launch_bounds__(FC_THREADS, 2) fc_qm_kernel(const QmArgs qa) {
         for (int q = 0; q < NS; ++q)
 #pragma unroll
             for (int i = 0; i < 4; ++i) ds[q][i] = 0.0f;
+    };
+    auto flush = [&](int blk) {
+        if (careful) flush_as(blk, std::true_type{});
+        else flush_as(blk, std::false_type{});
     };
     int left = WB == 4 ? gb - b_lo % gb : 0;  // blocks until the group ends
 #pragma unroll 1

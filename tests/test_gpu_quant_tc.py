@@ -97,3 +97,29 @@ def test_an_infinite_activation_stays_in_its_row(S, bits):
         out.append(y.cpu())
     assert torch.equal(out[0][1:], out[1][1:])
     assert not torch.isfinite(out[1][0]).any()
+
+
+@pytest.mark.parametrize("bits", [8, 4])
+@pytest.mark.parametrize("B", [1, 2, 3, 5])
+@pytest.mark.parametrize("special", [float("inf"), float("nan")])
+def test_a_scale_that_no_kept_channel_uses_has_no_effect(S, bits, B, special):
+    """Channels 64..95 (one scale group of 32) are dropped by every row: their scales are not part of any sum, whatever they hold."""
+    K, N = 256, 144
+    d = si.laplace_fc(4, K, N, si.BF16, 16, B)
+    x = dev(d["x"], si.BF16)
+    x[:, 64:96] = 0.0
+    ws = workspace(S.scap_fc_workspace(B, K, N))
+    out = []
+    for value in (1.0, special):
+        if bits == 8:
+            q, scale = si.quantise_q8(d["W"], si.BF16)
+            scale[64:96] = value
+            args, fn = (torch.from_numpy(q).cuda(), f32(scale)), S.scap_sparse_fc_q8
+        else:
+            q, scale, zero = si.quantise_q4(d["W"], si.BF16, 32)
+            scale[2] = value
+            args, fn = (torch.from_numpy(q).cuda(), f32(scale), torch.from_numpy(zero).cuda(), 32), S.scap_sparse_fc_q4
+        y = torch.empty((B, N), dtype=torch.float32, device="cuda")
+        fn(x, *args, None, f32([0.2]), None, y, ws.payload)
+        out.append(y.cpu())
+    assert torch.isfinite(out[0]).all() and torch.equal(out[0], out[1])
