@@ -6,6 +6,7 @@ from __future__ import annotations
 
 import ctypes as C
 import os
+import warnings
 
 import torch
 
@@ -49,8 +50,8 @@ def lib_path() -> str:
 
 
 _lib = None
-_call = None    # call(address, arg, ...) of the native helper
-_entry = {}     # name -> address of the entry point
+_call = None    # call(entry, arg, ...) -> status: the native helper, or ctypes where it is not built
+_entry = {}     # name -> what `_call` takes as the entry point: its address, or the ctypes function
 
 
 def lib():
@@ -101,7 +102,7 @@ def lib():
     L.scap_fold_bias_q4.restype = i
     L.scap_grouped_workspace.argtypes = []
     L.scap_grouped_workspace.restype = sz
-    L.scap_sparse_fc_grouped.argtypes = [vp, vp, vp, vp, vp, vp, i, i, i, i, C.POINTER(C.c_int), vp, sz, vp]
+    L.scap_sparse_fc_grouped.argtypes = [vp, vp, vp, vp, vp, vp, i, i, i, i, vp, vp, sz, vp]
     L.scap_sparse_fc_grouped.restype = i
     L.scap_fc_host_workspace.argtypes = [i, i, i]
     L.scap_fc_host_workspace.restype = sz
@@ -123,12 +124,22 @@ def lib():
     L.scap_moe_workspace.restype = sz
     L.scap_moe_ffn.argtypes = [vp, vp, C.POINTER(ScapExpert), i, i, vp, i, i, i, i, vp, vp, vp, sz, vp]
     L.scap_moe_ffn.restype = i
-    from ._scap_call import call
-    _entry.update({n: C.cast(getattr(L, n), C.c_void_p).value for n in EXPORTS})
     global _call
+    try:
+        from ._scap_call import call
+        _entry.update({n: C.cast(getattr(L, n), C.c_void_p).value for n in EXPORTS})
+    except ImportError as e:
+        warnings.warn("%s: calls go through ctypes, about 5 us slower each; `python -m paper_2412_07174_b200.build` builds the helper" % e)
+        call = _ctypes_call
+        _entry.update({n: getattr(L, n) for n in EXPORTS})
     _call = call
     _lib = L
     return L
+
+
+def _ctypes_call(entry, *args) -> int:
+    """What the native helper does, by ctypes."""
+    return entry(*[_ptr(a) for a in args])
 
 
 def _invoke(name: str, *args) -> None:

@@ -13,7 +13,8 @@ ROOT = os.path.dirname(HERE)
 CSRC = os.path.join(HERE, "csrc")
 OBJ = os.path.join(HERE, "_build")
 LIB = os.path.join(HERE, "libscap_b200.so")
-CALL = os.path.join(HERE, "_scap_call.so")  # the binding's call helper
+# the binding's call helper, named for the interpreter it is built against: another one does not load it
+CALL = os.path.join(HERE, "_scap_call" + sysconfig.get_config_var("EXT_SUFFIX"))
 
 # no --use_fast_math: the mask arithmetic must round exactly as documented
 NVCC_FLAGS = ["-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo", "-O3", "-std=c++17", "-Xcompiler", "-fPIC"]
@@ -59,12 +60,25 @@ def build(force: bool = False, verbose: bool = False) -> str:
         subprocess.check_call([nvcc, "-gencode", "arch=compute_100a,code=sm_100a", "--shared", "-cudart", "static",
                                "-o", tmp, *objs])
         os.replace(tmp, LIB)
-    src = os.path.join(CSRC, "scap_pycall.c")
-    if force or _newer(CALL, [src]):
-        tmp = CALL + ".tmp.%d" % os.getpid()
-        subprocess.check_call([os.environ.get("CC", "gcc"), "-O2", "-shared", "-fPIC", "-I", sysconfig.get_paths()["include"], src, "-o", tmp])
-        os.replace(tmp, CALL)
+    build_call_helper(force)
     return LIB
+
+
+def build_call_helper(force: bool = False, target: str = CALL) -> bool:
+    """The binding's call helper.  It needs a C compiler and the Python headers; without them the CUDA library is complete all the
+    same and the binding calls it through ctypes, so a failure here is reported and no more."""
+    src = os.path.join(CSRC, "scap_pycall.c")
+    if not force and not _newer(target, [src]):
+        return True
+    tmp = target + ".tmp.%d" % os.getpid()
+    cmd = [os.environ.get("CC", "gcc"), "-O2", "-shared", "-fPIC", "-I", sysconfig.get_paths()["include"], src, "-o", tmp]
+    try:
+        subprocess.check_call(cmd)
+    except (OSError, subprocess.CalledProcessError) as e:
+        print("the call helper was not built (%s): calls go through ctypes, about 5 us slower each" % e, file=sys.stderr)
+        return False
+    os.replace(tmp, target)
+    return True
 
 
 if __name__ == "__main__":
