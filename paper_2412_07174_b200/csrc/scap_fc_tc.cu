@@ -512,6 +512,7 @@ __device__ __forceinline__ void tc_ld32(uint32_t (&v)[32], uint32_t addr) {
 
 template <bool BF16, int ROWS, int MODE, typename XT, int EPI, int NACC>
 __global__ void __launch_bounds__(FC_THREADS, 2) fc_ds_kernel(const FcArgs a, const __grid_constant__ CUtensorMap tmap) {
+    static_assert(ROWS <= 16 || MODE == MODE_GATHER, "the 32-row form is for grouped calls: sparse, no row map, no mask output");
     constexpr int TNT = TC_TN, HALF = TNT / 2, NSPLIT = mma_nsplit(BF16), NST = ds_nst(ROWS), GR = ds_gather_rows(ROWS);
     extern __shared__ unsigned char smem_raw[];
     unsigned char *smem = reinterpret_cast<unsigned char *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
@@ -570,7 +571,7 @@ __global__ void __launch_bounds__(FC_THREADS, 2) fc_ds_kernel(const FcArgs a, co
                 if (k < K) prefetch_l2_keep(a.m + k);
             }
         }
-        if (!a.in_rows) {  // (with a row map the rows are not known yet)
+        if (ROWS > 16 || !a.in_rows) {  // (with a row map the rows are not known yet)
             constexpr int XL = (64 * (int)sizeof(XT) + 127) / 128;  // lines per row and block
             for (int i = t; i < nq * B * XL; i += FC_THREADS - 64) {
                 const int l = i % XL, rb = i / XL, b = rb % B, q = rb / B;
@@ -612,7 +613,7 @@ __global__ void __launch_bounds__(FC_THREADS, 2) fc_ds_kernel(const FcArgs a, co
         if (warp >= 2) tau = ld_act(a.tau);
     }
     prefetch_bias<BF16, EPI, TNT>(a, tile, s, per, bias0, bias1);
-    if (a.in_rows && tid < 16) misc->rows[tid] = __ldcg(a.in_rows + (tid < B ? tid : 0));
+    if (ROWS <= 16 && a.in_rows && tid < 16) misc->rows[tid] = __ldcg(a.in_rows + (tid < B ? tid : 0));
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
@@ -753,7 +754,7 @@ __global__ void __launch_bounds__(FC_THREADS, 2) fc_ds_kernel(const FcArgs a, co
             constexpr int XV = CPL * (int)sizeof(XT) / 16;  // 16-byte loads of x per lane and piece
             const int b = lane;
             const bool vec_ok = ((size_t)a.x_ld * sizeof(XT)) % 16 == 0;
-            const int xrow = a.in_rows ? misc->rows[b < B ? b : 0] : (b < B ? b : 0);
+            const int xrow = b < B ? b : 0;
             struct Piece {
                 uint4 raw[XV];
                 float m[CPL];
@@ -776,18 +777,17 @@ __global__ void __launch_bounds__(FC_THREADS, 2) fc_ds_kernel(const FcArgs a, co
 #pragma unroll
                     for (int v = 0; v < CPL / 4; ++v) {
                         uint4 r4 = make_uint4(0, 0, 0, 0);
-                        if (MODE == MODE_GATHER && a.m) r4 = ld_act16_if(reinterpret_cast<const unsigned char *>(a.m + k0 + 4 * v), b < B && k0 + 4 * v < K, pol_keep);
+                        if (a.m) r4 = ld_act16_if(reinterpret_cast<const unsigned char *>(a.m + k0 + 4 * v), b < B && k0 + 4 * v < K, pol_keep);
                         pc.m[4 * v] = __uint_as_float(r4.x); pc.m[4 * v + 1] = __uint_as_float(r4.y);
                         pc.m[4 * v + 2] = __uint_as_float(r4.z); pc.m[4 * v + 3] = __uint_as_float(r4.w);
                     }
                 } else {
 #pragma unroll
-                    for (int i = 0; i < CPL; ++i) pc.m[i] = (MODE == MODE_GATHER && a.m) ? ld_act_if(a.m + k0 + i, b < B && k0 + i < K) : 0.0f;
+                    for (int i = 0; i < CPL; ++i) pc.m[i] = a.m ? ld_act_if(a.m + k0 + i, b < B && k0 + i < K) : 0.0f;
                 }
             };
             Piece cur, next;
             if (pw < 2 * nq) load_piece(next, pw, 0);
-            uint32_t mine = 0;
 #pragma unroll 1
             for (int jc = pw, u = 0; jc < 2 * nq;) {
                 const int q = jc >> 1, h = jc & 1;
@@ -801,21 +801,17 @@ __global__ void __launch_bounds__(FC_THREADS, 2) fc_ds_kernel(const FcArgs a, co
                     if (lane == 0) go = mbar_wait(&misc->empty[st], (((uint32_t)q / NST) & 1u) ^ 1u, 1, abort_flag, spin);
                     go = __shfl_sync(0xffffffffu, go ? 1 : 0, 0) != 0;
                     if (!go) break;
-                    mine = 0;
                 }
                 const int chu = u * CPL, k0 = c * 32 + chu;  // this lane's first channel of the piece
                 const XT *xe = reinterpret_cast<const XT *>(cur.raw);
                 unsigned short part[CPL][3];
-                uint32_t kept_bits = 0;
 #pragma unroll
                 for (int i = 0; i < CPL; ++i) {
                     const float xv = widen1(xe[i]);
-                    const float dv = (MODE == MODE_GATHER && a.m) ? __fsub_rn(xv, cur.m[i]) : xv;
-                    const bool kept = b < B && k0 + i < K && (MODE == MODE_DENSE || fabsf(dv) >= tau);
-                    kept_bits |= kept ? (1u << i) : 0u;
+                    const float dv = a.m ? __fsub_rn(xv, cur.m[i]) : xv;
+                    const bool kept = b < B && k0 + i < K && fabsf(dv) >= tau;
                     split_parts<BF16>(kept ? dv : 0.0f, part[i]);
                 }
-                mine |= kept_bits << chu;
                 if (b < B) {
 #pragma unroll
                     for (int v = 0; v < CPL / 8; ++v) {
@@ -834,10 +830,6 @@ __global__ void __launch_bounds__(FC_THREADS, 2) fc_ds_kernel(const FcArgs a, co
                     }
                 }
                 if (u + 1 == SUB) {
-                    if (MODE == MODE_GATHER && a.bits && tile == 0) {
-                        const unsigned bal = __reduce_or_sync(0xffffffffu, mine);   // union over the rows, all 32 channels
-                        if (lane == 0 && c * 32 < K) a.bits[c] = bal;
-                    }
                     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");  // generic-proxy writes -> visible to the tensor core
                     __syncwarp();
                     if (lane == 0) mbar_arrive(&misc->afull[st]);
