@@ -72,7 +72,7 @@ def test_q8_batches_beyond_two_rows_and_the_dense_and_folding_calls(S):
     torch.cuda.synchronize()
     bf64 = oracle.fold_bias_q8(d["Wq"], d["wscale"], m, bias)
     assert rel_l2_rows(bfg.cpu().numpy(), bf64) <= 1e-6
-    # five rows (two + two + one launches): every row equals its own batch-1 result definition
+    # five rows: every row equals its own batch-1 result definition
     y64 = oracle.sparse_fc_q8(xf, d["Wq"], d["wscale"], m, 0.3, bf64.astype(np.float32))
     y, _ = run_q8(S, d, m, 0.3, bf64.astype(np.float32), want_idx=False)
     assert rel_l2_rows(y, y64) <= REL_L2_TOL
