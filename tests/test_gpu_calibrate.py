@@ -138,6 +138,18 @@ def test_estimators_and_scopes_bit_exact(S, estimator, scope, T, K, dt, nbins, s
     assert tau_g.view(np.uint32) == np.float32(tau_o).view(np.uint32)
 
 
+@pytest.mark.parametrize("estimator", [oracle.HISTOGRAM, oracle.MEDIAN])
+@pytest.mark.parametrize("T", [1023, 1024, 1025, 2047, 2048, 2049])
+def test_rows_at_the_limits_of_what_a_strip_keeps_in_registers(S, estimator, T):
+    """The passes over a strip are unrolled for eight (1024 rows) or sixteen (2048 rows) loads per thread; beyond, they re-read."""
+    K, nbins, s = 72, 512, 0.6
+    d = si.laplace_fc(4, K, 8, si.BF16, T, 1)
+    m_o, tau_o = oracle.calibrate_ex(si.to_f32(d["x_calib"], si.BF16), s, estimator, oracle.PER_CHANNEL, nbins)
+    m_g, tau_g = run_calibrate_ex(S, d["x_calib"], si.BF16, s, estimator, oracle.PER_CHANNEL, nbins)
+    assert np.array_equal(m_g.view(np.uint32), m_o.view(np.uint32))
+    assert tau_g.view(np.uint32) == np.float32(tau_o).view(np.uint32)
+
+
 @pytest.mark.parametrize("T,K,dt,G,s", [
     (256, 64, si.F16, 129, 0.5),
     (300, 40, si.BF16, 64, 0.3),

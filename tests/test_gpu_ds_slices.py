@@ -9,7 +9,7 @@ pytestmark = pytest.mark.gpu
 
 
 @pytest.mark.parametrize("split", [3, 5, 6, 7])
-def test_sixteen_rows_equal_two_times_eight(split):
+def test_sixteen_rows_equal_two_times_eight_and_the_sum_in_64_bits(split):
     import paper_2412_07174_b200 as S
     g = torch.Generator(device="cuda").manual_seed(7)
     D, F, B = 512, 1032, 16
@@ -40,5 +40,9 @@ def test_sixteen_rows_equal_two_times_eight(split):
             whole, halves = fn(h), torch.cat([fn(h[:8].contiguous()), fn(h[8:].contiguous())])
             S.scap_device_status()
             assert float((whole - halves).norm() / halves.norm()) < 1e-5  # binary32 sums of at most 1032 terms
+            u = h.double() @ Wgu.double()
+            if fn is block:
+                u = (torch.nn.functional.silu(u[:, :F]) * u[:, F:]) @ Wd.double()
+            assert float((whole - u).norm() / u.norm()) < 1e-5
     finally:
         S.scap_tune("split_k", 0)
