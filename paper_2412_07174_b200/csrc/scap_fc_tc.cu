@@ -776,8 +776,7 @@ __global__ void __launch_bounds__(FC_THREADS, 2) fc_ds_kernel(const FcArgs a, co
                 if (K % 4 == 0) {
 #pragma unroll
                     for (int v = 0; v < CPL / 4; ++v) {
-                        uint4 r4 = make_uint4(0, 0, 0, 0);
-                        if (a.m) r4 = ld_act16_if(reinterpret_cast<const unsigned char *>(a.m + k0 + 4 * v), b < B && k0 + 4 * v < K, pol_keep);
+                        const uint4 r4 = ld_act16_if(reinterpret_cast<const unsigned char *>(a.m + k0 + 4 * v), a.m != nullptr && b < B && k0 + 4 * v < K, pol_keep);
                         pc.m[4 * v] = __uint_as_float(r4.x); pc.m[4 * v + 1] = __uint_as_float(r4.y);
                         pc.m[4 * v + 2] = __uint_as_float(r4.z); pc.m[4 * v + 3] = __uint_as_float(r4.w);
                     }
@@ -808,7 +807,7 @@ __global__ void __launch_bounds__(FC_THREADS, 2) fc_ds_kernel(const FcArgs a, co
 #pragma unroll
                 for (int i = 0; i < CPL; ++i) {
                     const float xv = widen1(xe[i]);
-                    const float dv = a.m ? __fsub_rn(xv, cur.m[i]) : xv;
+                    const float dv = __fsub_rn(xv, cur.m[i]);  // (m == NULL: zeros)
                     const bool kept = b < B && k0 + i < K && fabsf(dv) >= tau;
                     split_parts<BF16>(kept ? dv : 0.0f, part[i]);
                 }

@@ -30,18 +30,19 @@ def test_large_groups_match_the_oracle(K, N, B, n_ctx, stream, dt):
     xf, m = si.to_f32(d["x"], dt), d["m_true"]
     tau = oracle.tau(si.to_f32(d["x_calib"], dt), m, 0.6)
     bias = np.linspace(-1, 1, N).astype(np.float32)
-    y64 = oracle.sparse_fc(xf, d["W"], dt, m, tau, None, threads=8) + bias[None, :]
     ws, yg = workspace(S.scap_grouped_workspace()), workspace(B * N * 4)
     y = yg.view(torch.float32, (B, N))
-    y.fill_(float("nan"))
-    S.scap_sparse_fc_grouped(dev(d["x"], dt), dev(d["W"], dt), f32(m), f32([tau]), f32(bias), y, d["ctx"].tolist(), ws.payload)
-    torch.cuda.synchronize()
-    S.scap_device_status()
-    assert ws.intact() and yg.intact()
-    assert bool((ws.payload == CANARY).all().item()) == stream  # only the gather writes its row table there
     ranks = min(8, -(-K // 64))
     bound = 2.0 ** -23 * (4 + K / (32 * ranks)) if stream else 2.0 ** -23 * 8 * np.sqrt(K)
-    assert rel_l2_rows(y.cpu().numpy(), y64) <= bound
+    for mm in (m, None):
+        y64 = oracle.sparse_fc(xf, d["W"], dt, mm, tau, None, threads=8) + bias[None, :]
+        y.fill_(float("nan"))
+        S.scap_sparse_fc_grouped(dev(d["x"], dt), dev(d["W"], dt), None if mm is None else f32(mm), f32([tau]), f32(bias), y, d["ctx"].tolist(), ws.payload)
+        torch.cuda.synchronize()
+        S.scap_device_status()
+        assert ws.intact() and yg.intact()
+        assert bool((ws.payload == CANARY).all().item()) == stream  # only the gather writes its row table there
+        assert rel_l2_rows(y.cpu().numpy(), y64) <= bound
 
 
 @pytest.mark.parametrize("dt", [si.F16, si.BF16])
