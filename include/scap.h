@@ -36,9 +36,9 @@
  *     scap_fold_bias, or any kernel or copy of the caller's), with no further synchronisation.  The weight matrix W
  *     is the exception: it is a constant of the layer and must be complete in device memory when the call is
  *     ISSUED (not written by work still pending on the stream), because kernels that know their first weight rows
- *     without looking at the activations (the batch 5..16 kernel, also on 8- and 4-bit codes and on the rows of a
- *     grouped call; the dense calls, a sparse call with "head_rows" set) request them before that wait, so that the
- *     memory system does not idle between consecutive calls.  Consecutive calls overlap where they can: a kernel may
+ *     without looking at the activations (the batch 5..16 kernel, also on the rows of a grouped call; the tensor-core
+ *     kernel of 8- and 4-bit weights at any batch; the dense calls, a sparse call with "head_rows" set) request them
+ *     before that wait, so that the memory system does not idle between consecutive calls.  Consecutive calls overlap where they can: a kernel may
  *     become resident and set up its shared memory while its predecessor drains (programmatic dependent launch,
  *     "pdl" below).
  */
@@ -92,7 +92,13 @@ int scap_version(void);
  *              its weight tile with TMA box loads and prunes on the activation operand (with that many rows the union
  *              mask of unrelated rows keeps nearly every channel anyway); 0 = the gather kernels, which fetch kept rows
  *              only (better when the rows of a batch share their pattern and the union keeps less than about half);
- *              2 = the dense-stream kernel from batch 3 on
+ *              2 = the dense-stream kernel from batch 3 on.
+ *              8- and 4-bit weights: 1 = the tensor-core kernel, which reads every row of codes, from batch 3 on and for
+ *              small layers at batch 1 and 2; 0 = the FMA kernels, which fetch kept rows only and take two rows at a time
+ *              (better for 8-bit calls of three or four rows that prune more than about 80 %); 2 = the tensor-core
+ *              kernel wherever it can run.
+ *              Grouped calls: 0 = always one gather per group (better when the rows of a group keep the very same
+ *              channels, and less than about a fifth of them); else see scap_sparse_fc_grouped
  *   "tc_spin"  tcgen05 kernels: how often a wait on one of its shared-memory barriers polls before it gives up
  *              (0 = the built-in limit of about a million polls, the default).  A limit of 1 makes the waits of
  *              the next call run out at once, which is how the error path of scap_device_status() is exercised
@@ -199,8 +205,9 @@ scap_status scap_dense_fc(const void *x, const void *W, const float *b, float *y
  * dtype xdt (fp16 or bf16); everything else as in scap_sparse_fc / scap_dense_fc / scap_fold_bias, with these
  * differences: N must be a multiple of 16; the bias b of the dense call and of the folding is fp32 [N] or
  * NULL; idx_out / nnz_out are only available for B <= 2, else SCAP_ERR_SHAPE.  Three and more rows (and small layers)
- * run on the tensor cores - the integers and an exact split of d into three bf16 parts, fp32 accumulation, every row of
- * Wq read once - where K is a multiple of four; else two rows at a time (results per row as in scap_sparse_fc).
+ * run on the tensor cores - the integers and an exact split of d * wscale into three bf16 parts, fp32 accumulation, every
+ * row of Wq requested once, by 9..16 rows twice - where K is a multiple of four and wscale 16-byte aligned; else two rows
+ * at a time (results per row as in scap_sparse_fc).  The scale of a channel that a row drops has no part in that row of y.
  * Workspace: scap_fc_workspace(B, K, N). */
 scap_status scap_sparse_fc_q8(const void *x, scap_dtype xdt, const signed char *Wq, const float *wscale, const float *m,
                               const float *tau, const float *b_fused, float *y, int B, int K, int N, uint32_t *idx_out,
@@ -217,7 +224,9 @@ scap_status scap_fold_bias_q8(const signed char *Wq, const float *wscale, const 
  * zero[same shape] (one byte, 0..15):  W[k,n] = scale[k / group, n] * (q[k,n] - zero[k / group, n]).
  * group: a multiple of 32, 32..2048 (else SCAP_ERR_SHAPE); N a multiple of 16.  Everything else - x of dtype xdt, m, tau,
  * b_fused, y, the optional kept list, the batch rule (idx_out / nnz_out only for B <= 2), the workspace query - as for
- * the 8-bit calls above.  The sum over the kept channels of one group is formed on the integer codes in fp32 as
+ * the 8-bit calls above; the tensor-core route wants, instead of an aligned wscale, that no rank of a cluster meets more
+ * than 96 groups (their scales stay in shared memory), which leaves out K above about 3000 S channels at group 32 and
+ * 12000 S at group 128, S = 1..8 being the split-K factor.  The sum over the kept channels of one group is formed on the integer codes in fp32 as
  * sum d * q - zero * sum d (tensor cores: sum d * (q - 8) - (zero - 8) * sum d), and scaled.                                          */
 scap_status scap_sparse_fc_q4(const void *x, scap_dtype xdt, const unsigned char *Wq, const float *scale,
                               const unsigned char *zero, int group, const float *m, const float *tau, const float *b_fused,
@@ -234,8 +243,9 @@ scap_status scap_fold_bias_q4(const unsigned char *Wq, const float *scale, const
  * expected to share their pattern, e.g. the beams of one prompt or the tokens of one request: group_of_row_host[b]
  * (a HOST array, read during the call only) is the group 0..15 of row b; at most 16 rows per group (else
  * SCAP_ERR_SHAPE).  Each group is pruned with the union mask of its own rows only and fetches only the weight rows
- * that mask keeps, all groups in one launch (groups of more than four rows: where it is faster, every weight row is read
- * once for all groups and pruning is left to the activations); y[b] is the same function of x[b] as in scap_sparse_fc (pruning is per
+ * that mask keeps, all groups in one launch.  Where every group has more than four rows and the layer fills the device,
+ * the call takes the dense-stream kernel of scap_sparse_fc instead: every weight row is read once per 32 rows of the batch
+ * (one launch each) and pruning is left to the activations ("dense_stream" 0 turns that off).  y[b] is the same function of x[b] as in scap_sparse_fc (pruning is per
  * element), whatever the grouping.  No idx / nnz outputs.  Workspace: scap_grouped_workspace() bytes.              */
 size_t scap_grouped_workspace(void);
 scap_status scap_sparse_fc_grouped(const void *x, const void *W, const float *m, const float *tau, const float *b_fused,

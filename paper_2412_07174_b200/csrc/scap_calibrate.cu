@@ -26,15 +26,15 @@ __device__ __forceinline__ void widen8(const uint4 &v, float (&f)[8]) {
     widen2<BF16>(v.w, f[6], f[7]);
 }
 
-// Rows t0, t0 + CAL_ROWS, ... (CAL_U of them) of this thread's 8 channels, all loads in flight together; rows at or
+// Rows t0, t0 + CAL_ROWS, ... (U of them) of this thread's 8 channels, all loads in flight together; rows at or
 // beyond T are skipped (their slots keep zeros and `valid` says how many are real).
 constexpr int CAL_U = 16;  // with 128 rows per sweep: 2048 rows of a strip live in registers at once
-template <int CAL_U>
-__device__ __forceinline__ int load_rows(const uint16_t *xp, int K, int T, int t0, uint4 (&v)[CAL_U]) {
+template <int U>
+__device__ __forceinline__ int load_rows(const uint16_t *xp, int K, int T, int t0, uint4 (&v)[U]) {
     const uint64_t pol = l2_policy_keep();  // the radix passes read the tensor again: it fits in L2, ask for it to stay
     int valid = 0;
 #pragma unroll
-    for (int u = 0; u < CAL_U; ++u) {
+    for (int u = 0; u < U; ++u) {
         const int t = t0 + u * CAL_ROWS;
         v[u] = make_uint4(0, 0, 0, 0);
         if (t < T) {
@@ -80,7 +80,7 @@ __device__ __forceinline__ uint4 rotate_channels(const uint4 &v, int r) {
 //
 // U = 16-byte loads per thread that the passes are unrolled for (128 U rows live in registers).  The code of a pass grows
 // with U whether or not there are that many rows, and one CTA runs it once, straight through the instruction cache: up to
-// 1024 rows eight are faster (whole call, us, 16 -> 8: 128 x 1024 20.5 -> 17.1, 512 x 4096 34.9 -> 33.5), beyond they would
+// 1024 rows eight are faster (whole call, us, 16 -> 8: 128 x 1024 20.0 -> 17.1, 512 x 4096 32.8 -> 31.5), beyond they would
 // read the strip again in every pass (2048 x 14336: 127 -> 141).
 template <bool BF16, int CWT, int U>
 __global__ void __launch_bounds__(CWT * 16, CWT == 16 ? 2 : 1) mode_kernel(const uint16_t *__restrict__ x, int T, int K, int nbins,
@@ -100,7 +100,7 @@ __global__ void __launch_bounds__(CWT * 16, CWT == 16 ? 2 : 1) mode_kernel(const
     const int kc = k0 + q * 8;
     const bool ok = kc < K;  // K is a multiple of 8
     const uint16_t *xp = x + kc;
-    // Up to CAL_ROWS * U = 2048 rows: the strip is read once, all loads in flight together, and the three
+    // Up to CAL_ROWS * U rows (1024 at U = 8, 2048 at 16): the strip is read once, all loads in flight together, and the three
     // passes below run from registers; longer inputs are re-read per pass (from L2 when they fit).
     const bool resident = T <= CAL_ROWS * U;
     uint4 v[U];
@@ -543,7 +543,7 @@ __device__ __forceinline__ void find_rank256(const uint32_t *h, uint32_t r, int 
 
 // Median per channel: two 8-bit radix passes over the 16-bit keys of a strip of CW channels, from registers.
 // Eight loads per thread: longer inputs are read again for the second pass, but the unrolled passes stay in the instruction
-// cache (median and threshold of 2048 x 14336: 208 us with sixteen, 166 with eight).
+// cache (median and threshold, us, sixteen -> eight: 2048 x 14336 208 -> 166, 2048 x 1024 58.2 -> 55.4, 1100 x 4096 47.8 -> 46.5).
 // Shared memory: hi[CW][256] | lo[2][CW][256] counters | per-channel bucket state.
 constexpr int MED_U = 8;
 template <bool BF16>

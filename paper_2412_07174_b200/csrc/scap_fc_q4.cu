@@ -391,7 +391,8 @@ static cudaError_t launch_q4_t(const Q4Args &qa, cudaStream_t st) {
 // needs a second launch over the codes (figures in scap_fc_qm.cu).
 // One and two rows: the FMA kernel reads the kept rows only, this one all of them, but its prologue is shorter and it needs
 // no list.  It wins whatever the sparsity while a warp has at most two blocks (K = 2048, N = 4096, one row: 6.0 us against
-// 6.7 - 7.6; at four, K = 4096, N = 4096: 8.1 against 6.7 - 9.2).
+// 6.8 - 7.4; at four, K = 4096, N = 4096: 7.9 against 7.0 - 9.2).  From three rows on it wins up to 95 % pruned (11008 x 4096, three
+// rows: 17.8 us against 31.1 at 50 %, 18.1 at 95 %).  Calls whose scale groups do not fit (qm_applicable) stay on the FMA kernel.
 static bool q4_on_tensor_cores(const QmArgs &a) {
     if (g_tune.dense_stream == 0 || !qm_applicable(4, a)) return false;
     return g_tune.dense_stream >= 2 || a.f.B >= 3 || qm_blocks_per_warp(a) <= 2;

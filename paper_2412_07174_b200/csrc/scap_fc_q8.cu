@@ -51,11 +51,13 @@ static cudaError_t launch_q8_t(const FcArgs &a, cudaStream_t st) {
 }
 
 // Calls that take the tensor-core kernel (tune "dense_stream": 0 none, 2 all it can take).  From three rows on the FMA kernel
-// needs a second launch over the codes (figures in scap_fc_qm.cu; only three or four rows with more than 85 % pruned would be
-// up to 15 % faster in two launches, and the sparsity is not known here).
+// needs a second launch over the codes (figures in scap_fc_qm.cu).  Two launches over the kept rows only are the faster form for three
+// and four rows of a large layer that prune a lot, and the sparsity is not known here (11008 x 4096, us, FMA -> this one at
+// 50 / 80 / 85 / 90 / 95 %: three rows 21.7 / 16.8 / 15.1 / 13.9 / 12.7 -> 18.0, four rows 24.9 / 18.9 / 16.5 / 14.7 / 12.0 -> 18.1;
+// five rows 33.1 / 26.1 / 24.0 / 22.0 / 19.5 -> 23.7): a caller who knows sets "dense_stream" 0.
 // One and two rows: the FMA kernel reads the kept rows only, this one all of them, but its prologue is shorter.  It wins
-// whatever the sparsity only while a warp has a single block (N = 1024, K = 1024, one row: 3.0 us against 3.4 - 3.7; at two
-// blocks, K = 2048, N = 4096: 5.4 against 4.4 - 5.1).
+// whatever the sparsity only while a warp has a single block (K = N = 1024, one row: 2.7 us against 3.3 - 3.4, two rows 3.1 against
+// 3.9 - 4.2; at two blocks, K = 2048, N = 4096: 5.2 against 4.2 - 5.3).
 static bool q8_on_tensor_cores(const QmArgs &a) {
     if (g_tune.dense_stream == 0 || !qm_applicable(8, a)) return false;
     return g_tune.dense_stream >= 2 || a.f.B >= 3 || qm_blocks_per_warp(a) <= 1;

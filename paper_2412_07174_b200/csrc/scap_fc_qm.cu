@@ -13,14 +13,17 @@
 //   instruction streams on every scheduler and a dozen hand-overs per stage cost more than the tensor core saves.)
 //
 // Why it is here: beyond two rows the fp32-FMA kernels run two rows per launch, so the codes cross the chip B / 2 times.
-// K = 11008, N = 4096, half of the entries pruned, weights from DRAM, FMA kernel -> this one, us per call:
-//   8-bit   4 rows 24.4 -> 16.8   8 rows 47.5 -> 20.0   16 rows 93.8 -> 34
-//   4-bit   4 rows 35.7 -> 16.2   8 rows 71   -> 21.4   16 rows 141  -> 37
-// The codes are 45 (22.5) MB, 7 (3.5) us at copy speed; what is left is about 300 instructions per 16 channels x 128 columns
-// and warp (half of them on the half-rate integer pipe) and the fixed 3 us of a call.
+// K = 11008, N = 4096, half of the entries pruned, weights from DRAM, FMA kernel -> this one, device us per call:
+//   8-bit            4 rows 24.6 -> 17.9   8 rows 48.0 -> 23.9   16 rows  94.6 -> 41.1
+//   4-bit, group 128 4 rows 36.1 -> 16.8   8 rows 71.6 -> 21.3   16 rows 142   -> 37.0
+// The codes are 45 (22.5) MB, 7 (3.5) us at copy speed.  What is left, by counters at eight rows: 9.3 M (10.7 M) warp instructions,
+// 421 (485) per 16 channels x 128 columns with everything included, 56 % (48 %) of them on the half-rate integer pipe, at 0.38
+// (0.48) a cycle and scheduler; a warp waits for its loads more than half (a quarter) of the time, since with 128 registers a
+// thread there are 16 warps on an SM with two blocks each in flight.
 //
-// Precision: the codes are small integers and the leading part has 8 significant bits, so a chain of leading products is exact
-// in binary32 (the tensor core truncates what does not fit); the two smaller parts never share an accumulator with it.
+// Precision: codes, parts and products (16 bits at most) are exact; the sum of a chain is truncated by the tensor core where the
+// exponents of its terms lie too far apart.  The two smaller parts never share an accumulator with the leading one.  Error against
+// 64 bits 8e-8 (8-bit FMA kernel 1.3e-7).
 // A rank's channels are spread over 4 or 8 warps and S ranks, added at the end in fixed order in binary32.
 //
 //   grid = (128-column tiles, S, 1 or 2), cluster (1, S, 1), 256 threads, two CTAs per SM

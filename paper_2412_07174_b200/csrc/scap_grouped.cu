@@ -3,6 +3,8 @@
 // one prompt, the tokens of one request - keep it).  The caller names the group of every row; each group is one
 // z-slice of the grid and runs the ordinary FC body on its own rows (read and written through a row map), so a group
 // fetches only the weight rows its own rows keep.  Up to 64 rows in up to 16 groups of at most 16 rows.
+// Calls whose groups all have more than four rows leave the gather for the dense-stream kernel (scap_fc_tc.cu) where that is
+// the faster way to the same y; the rule is at the entry point.
 #include <string.h>
 
 #include "scap_ds.cuh"
@@ -117,10 +119,18 @@ scap_status scap_sparse_fc_grouped(const void *x, const void *W, const float *m,
     // group.  The dense-stream kernel reads every row once per 32 rows of the batch, prunes on the activations (which is per
     // element, so the grouping changes nothing in y), and its time does not depend on the masks.  (A call with a group of up
     // to four rows stays on the gather: such a group runs on the FMA bodies there, in binary32 and rounded to nearest, and
-    // what a row gets does not depend on the size of another row's group.)  Gather -> stream, overlap 0.9, 50 % / 80 % pruned, us:
-    //   11008 x 4096   2 x 6 rows 40 / 32 -> 22   4 x 8 rows 73 / 58 -> 36   8 x 8 rows 135 / 104 -> 71
-    //    2048 x 1024   2 x 6 rows 12 / 12 ->  8   4 x 8 rows 14 / 12 -> 11   8 x 8 rows  16 /  14 -> 21
-    //   14336 x 2048   2 x 6 rows 35 / 30 -> 24   4 x 8 rows 53 / 43 -> 42   8 x 8 rows  92 /  71 -> 82
+    // what a row gets does not depend on the size of another row's group.)  Device time, us, gather -> stream,
+    // rows of a group with nine tenths of their pattern in common, 50 % / 80 % pruned | with all of it, 65 / 80 / 90 %:
+    //   11008 x 4096   2 x 6 rows  40 /  33 -> 22 | 27 / 21 / 17 -> 22
+    //                  4 x 8 rows  73 /  58 -> 35 | 46 / 36 / 28 -> 35
+    //                  8 x 8 rows 136 / 104 -> 67 | 79 / 61 / 48 -> 67
+    //    4096 x 4096   2 x 6 rows  23 /  20 -> 14 | 18 / 15 / 13 -> 13
+    //                  4 x 8 rows  33 /  28 -> 19 | 23 / 19 / 16 -> 19
+    //                  8 x 8 rows  58 /  47 -> 36 | 37 / 30 / 25 -> 36
+    //    2048 x 1024   2 x 6 rows  12 /  12 ->  7   4 x 8 rows 13 / 13 -> 10   8 x 8 rows 16 / 14 -> 19
+    //   14336 x 2048   2 x 6 rows  35 /  30 -> 24   4 x 8 rows 53 / 43 -> 40   8 x 8 rows 93 / 71 -> 78
+    // The masks are not known here.  Rows that keep exactly the same channels, fewer than a fifth of them, are the one kind of
+    // call that loses by the stream (at 90 % pruned up to 1.4 times the time); a caller who has them sets "dense_stream" 0.
     // Above 16 rows it is bound by the preparation of the activations, which takes two CTAs on most SMs to hide, while the
     // groups of a gather fill an empty chip themselves: there it needs a full grid, or a short layer and one pass.
     const int s_ds = ds_choose_split(K, N, EPI_BIAS);
