@@ -14,7 +14,7 @@
 //
 // Why it is here: beyond two rows the fp32-FMA kernels run two rows per launch, so the codes cross the chip B / 2 times.
 // K = 11008, N = 4096, half of the entries pruned, weights from DRAM, FMA kernel -> this one, device us per call:
-//   8-bit            4 rows 24.6 -> 17.9   8 rows 48.0 -> 23.9   16 rows  94.6 -> 41.1
+//   8-bit            4 rows 24.6 -> 18.3   8 rows 48.0 -> 23.9   16 rows  94.6 -> 41.2
 //   4-bit, group 128 4 rows 36.1 -> 16.8   8 rows 71.6 -> 21.3   16 rows 142   -> 37.0
 // The codes are 45 (22.5) MB, 7 (3.5) us at copy speed.  What is left, by counters at eight rows: 9.3 M (10.7 M) warp instructions,
 // 421 (485) per 16 channels x 128 columns with everything included, 56 % (48 %) of them on the half-rate integer pipe, at 0.38
@@ -42,6 +42,14 @@ constexpr int QM_GROUP_BYTES = QM_TN * 5;  // 128 scales and 128 zero points
 __host__ __device__ constexpr int qm_cw(int BT) { return BT <= 4 ? 128 : 64; }     // columns per warp
 __host__ __device__ constexpr int qm_nkg(int BT) { return FC_WARPS * qm_cw(BT) / QM_TN; }  // ranges of channels per rank
 __host__ __device__ constexpr int qm_red_bytes(int BT) { return qm_nkg(BT) * BT * QM_TN * 4; }
+// 8-bit weights: the leading sums leave the tensor core's accumulators every 16 QM_CHAIN channels, for slots of the thread in shared
+// memory.  A truncating accumulator that holds a large value (one activation a thousand times the others) loses up to 2^-23 of it with
+// every product: a chain of 224 (14336 x 11008, 16 rows, one rank) was off by 6.3e-6 of the result, the FMA kernel by 2.4e-7; in chains of eight it is
+// 3.1e-7, and 7e-8 (FMA 1.9e-7) where the large ones are thirty times the others.  11008 x 4096, us: four rows 17.8 -> 18.3, eight rows
+// 23.8 -> 23.9, sixteen 41.0 -> 41.2.  (The 4-bit sums are closed once per group.)
+constexpr int QM_CHAIN = 8;
+__host__ __device__ constexpr int qm_slot_quads(int BT) { return qm_cw(BT) / 16; }  // float4 per thread
+__host__ __device__ constexpr int qm_slot_bytes(int WB, int BT) { return WB == 8 ? FC_THREADS * qm_slot_quads(BT) * 16 : 0; }
 __host__ __device__ constexpr int qm_smem(int BT) { return qm_red_bytes(BT) + BT * GATHER_LD * 4 + 16; }  // partials | gather | barrier
 static_assert(2 * (qm_smem(4) + QM_SCALE_MAX + 1024) <= 233472 && 2 * (qm_smem(8) + QM_SCALE_MAX + 1024) <= 233472, "two CTAs must fit in the shared memory of an SM");
 
@@ -302,6 +310,26 @@ __global__ void __launch_bounds__(FC_THREADS, 2) fc_qm_kernel(const QmArgs qa) {
         if (careful) flush_as(blk, std::true_type{});
         else flush_as(blk, std::false_type{});
     };
+    bool promoted = false;
+    auto add_slots = [&]() {
+        const float4 *s_slot = reinterpret_cast<const float4 *>(smem + qm_smem(BT)) + threadIdx.x;  // [quad][thread]
+#pragma unroll
+        for (int j = 0; j < NP; ++j) {
+            const float4 p = s_slot[j * FC_THREADS];
+            acc[0][j][0] += p.x; acc[0][j][1] += p.y; acc[0][j][2] += p.z; acc[0][j][3] += p.w;
+        }
+    };
+    auto promote = [&]() {
+        if (promoted) add_slots();
+        promoted = true;
+        float4 *s_slot = reinterpret_cast<float4 *>(smem + qm_smem(BT)) + threadIdx.x;
+#pragma unroll
+        for (int j = 0; j < NP; ++j) {
+            s_slot[j * FC_THREADS] = make_float4(acc[0][j][0], acc[0][j][1], acc[0][j][2], acc[0][j][3]);
+#pragma unroll
+            for (int i = 0; i < 4; ++i) acc[0][j][i] = 0.0f;
+        }
+    };
     int left = WB == 4 ? gb - b_lo % gb : 0;  // blocks until the group ends
 #pragma unroll 1
     for (int blk = b_lo; blk < b_hi; blk += PX) {
@@ -314,7 +342,9 @@ __global__ void __launch_bounds__(FC_THREADS, 2) fc_qm_kernel(const QmArgs qa) {
                 if (WB == 4 && (--left == 0 || blk + i + 1 == b_hi)) { flush(blk + i); left = gb; }
             }
         }
+        if (WB == 8 && (blk + PX - b_lo) % QM_CHAIN == 0 && blk + PX < b_hi) promote();
     }
+    if (WB == 8 && promoted) add_slots();
 
     // ---- parts of a batch row added smallest first, and the factor 64; this warp's partial tile -> shared memory
 #pragma unroll
@@ -367,10 +397,13 @@ template <int WB, int BT, int MODE, typename XT>
 static cudaError_t launch_qm_b(const QmArgs &qa, cudaStream_t st) {
     static SmemOptIn opt_in;
     auto kern = fc_qm_kernel<WB, BT, MODE, XT>;
-    cudaError_t e0 = ensure_dynamic_smem(kern, qm_smem(BT) + (WB == 4 ? QM_SCALE_MAX : 0), opt_in);
+    cudaError_t e0 = ensure_dynamic_smem(kern, qm_smem(BT) + (WB == 4 ? QM_SCALE_MAX : qm_slot_bytes(WB, BT)), opt_in);
     if (e0 != cudaSuccess) return e0;
-    return launch_cluster(kern, dim3((qa.f.ldw + QM_TN - 1) / QM_TN, qa.f.S, qa.f.B > 8 ? 2 : 1), dim3(FC_THREADS),
-                          qm_smem(BT) + (WB == 4 ? qa.sg * QM_GROUP_BYTES : 0), qa.f.S, st, g_tune.pdl != 0, qa);
+    // (the slots are there where a warp has more than one chain)
+    const int blocks = (qa.f.K + 15) / 16, warps = qm_nkg(BT) * qa.f.S;
+    const int extra = WB == 4 ? qa.sg * QM_GROUP_BYTES : (blocks + warps - 1) / warps > QM_CHAIN ? qm_slot_bytes(WB, BT) : 0;
+    return launch_cluster(kern, dim3((qa.f.ldw + QM_TN - 1) / QM_TN, qa.f.S, qa.f.B > 8 ? 2 : 1), dim3(FC_THREADS), qm_smem(BT) + extra,
+                          qa.f.S, st, g_tune.pdl != 0, qa);
 }
 template <int WB, int MODE, typename XT>
 static cudaError_t launch_qm_x(const QmArgs &qa, cudaStream_t st) {

@@ -91,6 +91,18 @@ def test_every_cluster_size(S, bits, split, B):
         S.scap_tune("split_k", 0)
 
 
+@pytest.mark.parametrize("blocks", [8, 9, 10, 16, 17, 25])
+@pytest.mark.parametrize("B", [1, 2, 4, 8])
+def test_lengths_of_the_8_bit_chains(S, blocks, B):
+    """Up to eight blocks of 16 channels stay in the accumulator of a warp, longer stretches leave it every eight blocks."""
+    warps = 4 if B > 4 else 8
+    try:
+        S.scap_tune("split_k", 1)
+        check(S, 8, 16 * (blocks * warps - 1) + 4, 144, B, 32, si.BF16)  # the last warp's stretch ends in a partial block
+    finally:
+        S.scap_tune("split_k", 0)
+
+
 @pytest.mark.parametrize("bits", [8, 4])
 @pytest.mark.parametrize("K,B,stream", [(1001, 3, 1), (1002, 5, 1), (1003, 16, 1), (1000, 5, 0), (1000, 16, 0)])
 def test_calls_that_run_two_rows_at_a_time(S, bits, K, B, stream):
@@ -110,6 +122,35 @@ def test_either_side_of_the_limit_of_scale_groups(S, K):
         check(S, 4, K, 144, 3, 32, si.F16)
     finally:
         S.scap_tune("split_k", 0)
+
+
+@pytest.mark.parametrize("bits", [8, 4])
+@pytest.mark.parametrize("B", [1, 4, 16])
+def test_a_few_large_activations_do_not_cost_the_others_their_bits(S, bits, B):
+    """A truncating accumulator that holds a large value early loses up to 2^-23 of it with every further product, so its chain has to be
+    short: eight products (8-bit) or a scale group of 128 channels (4-bit), and a handful of additions after it."""
+    K, N = 14336, 144
+    d = si.laplace_fc(4, K, N, si.BF16, 16, B)
+    x = si.to_f32(d["x"], si.BF16).astype(np.float64)
+    x[:, ::K // 8] = 300.0 * (1 + np.arange(B))[:, None]  # the first channel of every warp's stretch
+    bits_x = si.to_bits(x, si.BF16)
+    xf, m = si.to_f32(bits_x, si.BF16), d["m_true"]
+    if bits == 8:
+        q, scale = si.quantise_q8(d["W"], si.BF16)
+        args, fn = (torch.from_numpy(q).cuda(), f32(scale)), S.scap_sparse_fc_q8
+        y64 = oracle.sparse_fc_q8(xf, q, scale, m, 0.1, None)
+    else:
+        q, scale, zero = si.quantise_q4(d["W"], si.BF16, 128)
+        args, fn = (torch.from_numpy(q).cuda(), f32(scale), torch.from_numpy(zero).cuda(), 128), S.scap_sparse_fc_q4
+        y64 = oracle.sparse_fc_q4(xf, q, scale, zero, 128, m, 0.1, None)
+    y = torch.empty((B, N), dtype=torch.float32, device="cuda")
+    try:
+        S.scap_tune("split_k", 1)
+        fn(dev(bits_x, si.BF16), *args, f32(m), f32([0.1]), None, y, workspace(S.scap_fc_workspace(B, K, N)).payload)
+        torch.cuda.synchronize()
+    finally:
+        S.scap_tune("split_k", 0)
+    assert rel_l2_rows(y.cpu().numpy(), y64) <= 2.0 ** -23 * (8 + 2)
 
 
 @pytest.mark.parametrize("bits", [8, 4])
