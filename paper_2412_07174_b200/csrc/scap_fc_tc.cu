@@ -510,10 +510,32 @@ __device__ __forceinline__ void tc_ld32(uint32_t (&v)[32], uint32_t addr) {
         : "r"(addr));
 }
 
+// Parts of an activation.  fp16 rows of a grouped call (NACC = 2) take three parts of 4, 9 and 11 bits instead of two of 11: the
+// products with the leading part are 15 bits, so its accumulator has bits to spare and truncates next to nothing, and what the
+// others lose is small.  The gather, whose chains are shorter, is the measure: of 240 fp16 calls of 1024 .. 14336 channels the
+// two parts were further off than it in 151 (up to 3.4 times: 14336 x 520, 12 rows, 7.8e-7 against 2.3e-7), 5 + 8 + 11 bits in 21
+// (up to 1.3 times), these in none.  fp16, us: 11008 x 4096 12 rows 21.2 -> 22.0, 32 rows 32.2 -> 36.8; 4096 x 4096 32 rows
+// 17.8 -> 19.9.
+__host__ __device__ constexpr bool ds_fine_split(bool bf16, int NACC) { return !bf16 && NACC == 2; }
+__host__ __device__ constexpr int ds_nsplit(bool bf16, int NACC) { return ds_fine_split(bf16, NACC) ? 3 : mma_nsplit(bf16); }
+template <bool BF16, int NACC>
+__device__ __forceinline__ void ds_split(float v, unsigned short (&part)[3]) {
+    if constexpr (ds_fine_split(BF16, NACC)) {
+        const __half hi = __float2half_rn(__uint_as_float(__float_as_uint(v) & 0xfff00000u));
+        const float r1 = v - __half2float(hi);
+        const __half mid = __float2half_rn(__uint_as_float(__float_as_uint(r1) & 0xffff8000u));
+        part[0] = __half_as_ushort(hi);
+        part[1] = __half_as_ushort(mid);
+        part[2] = __half_as_ushort(__float2half_rn(r1 - __half2float(mid)));
+    } else {
+        split_parts<BF16>(v, part);
+    }
+}
+
 template <bool BF16, int ROWS, int MODE, typename XT, int EPI, int NACC>
 __global__ void __launch_bounds__(FC_THREADS, 2) fc_ds_kernel(const FcArgs a, const __grid_constant__ CUtensorMap tmap) {
     static_assert(ROWS <= 16 || MODE == MODE_GATHER, "the 32-row form is for grouped calls: sparse, no row map, no mask output");
-    constexpr int TNT = TC_TN, HALF = TNT / 2, NSPLIT = mma_nsplit(BF16), NST = ds_nst(ROWS), GR = ds_gather_rows(ROWS);
+    constexpr int TNT = TC_TN, HALF = TNT / 2, NSPLIT = ds_nsplit(BF16, NACC), NST = ds_nst(ROWS), GR = ds_gather_rows(ROWS);
     extern __shared__ unsigned char smem_raw[];
     unsigned char *smem = reinterpret_cast<unsigned char *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
     unsigned char *s_w = smem + DS_OFF_W;
@@ -722,7 +744,7 @@ __global__ void __launch_bounds__(FC_THREADS, 2) fc_ds_kernel(const FcArgs a, co
                     const float dv = (MODE == MODE_GATHER && a.m) ? __fsub_rn(xv[i], mv[i]) : xv[i];
                     const bool kept = b < B && k0 + i < K && (MODE == MODE_DENSE || fabsf(dv) >= tau);
                     mine |= kept ? (1u << i) : 0u;
-                    split_parts<BF16>(kept ? dv : 0.0f, part[i]);
+                    ds_split<BF16, NACC>(kept ? dv : 0.0f, part[i]);
                 }
                 if (b < B) {
 #pragma unroll
@@ -809,7 +831,7 @@ __global__ void __launch_bounds__(FC_THREADS, 2) fc_ds_kernel(const FcArgs a, co
                     const float xv = widen1(xe[i]);
                     const float dv = __fsub_rn(xv, cur.m[i]);  // (m == NULL: zeros)
                     const bool kept = b < B && k0 + i < K && fabsf(dv) >= tau;
-                    split_parts<BF16>(kept ? dv : 0.0f, part[i]);
+                    ds_split<BF16, NACC>(kept ? dv : 0.0f, part[i]);
                 }
                 if (b < B) {
 #pragma unroll

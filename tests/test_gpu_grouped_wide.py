@@ -3,8 +3,7 @@ the faster route: the edges of its row counts, 64-channel blocks, 128-column til
 paths (K a multiple of eight or not), and the rows and results of the second pass.
 
 Bound of the stream: an accumulator takes K / (32 S) products of 16 channels (S ranks, two accumulators), each of which truncates
-it by at most 2^-23 of its value, and a handful of binary32 additions follow; fp16 splits d into two parts, 2^-23 of it at most
-for entries of this size.  The gather kernel rounds once per 16 channels of a warp's list and is held to the looser bound of random
+it by at most 2^-23 of its value, and a handful of binary32 additions follow; the three parts of d hold all of it.  The gather kernel rounds once per 16 channels of a warp's list and is held to the looser bound of random
 roundings, 2^-23 8 sqrt(K)."""
 import numpy as np
 import pytest
@@ -33,7 +32,7 @@ def test_large_groups_match_the_oracle(K, N, B, n_ctx, stream, dt):
     ws, yg = workspace(S.scap_grouped_workspace()), workspace(B * N * 4)
     y = yg.view(torch.float32, (B, N))
     ranks = min(8, -(-K // 64))
-    bound = 2.0 ** -23 * (4 + K / (32 * ranks)) if stream else 2.0 ** -23 * 8 * np.sqrt(K)
+    bound = 2.0 ** -23 * (2 + K / (32 * ranks)) if stream else 2.0 ** -23 * 8 * np.sqrt(K)
     for mm in (m, None):
         y64 = oracle.sparse_fc(xf, d["W"], dt, mm, tau, None, threads=8) + bias[None, :]
         y.fill_(float("nan"))
@@ -43,6 +42,28 @@ def test_large_groups_match_the_oracle(K, N, B, n_ctx, stream, dt):
         assert ws.intact() and yg.intact()
         assert bool((ws.payload == CANARY).all().item()) == stream  # only the gather writes its row table there
         assert rel_l2_rows(y.cpu().numpy(), y64) <= bound
+
+
+@pytest.mark.parametrize("dt", [si.F16, si.BF16])
+@pytest.mark.parametrize("K,N,B,n_ctx", [(14336, 520, 12, 2), (11008, 264, 5, 1), (3000, 2048, 24, 3), (1024, 1024, 32, 4)])
+def test_the_stream_is_no_further_off_than_the_gather(K, N, B, n_ctx, dt):
+    import paper_2412_07174_b200 as S
+    d = si.context_batch(4, K, N, dt, 64, B, n_ctx, 0.9)
+    xf, m = si.to_f32(d["x"], dt), d["m_true"]
+    tau = oracle.tau(si.to_f32(d["x_calib"], dt), m, 0.6)
+    y64 = oracle.sparse_fc(xf, d["W"], dt, m, tau, None, threads=8)
+    err = {}
+    try:
+        for route in (1, 0):
+            S.scap_tune("dense_stream", route)
+            y, ws = torch.empty((B, N), device="cuda"), workspace(S.scap_grouped_workspace())
+            S.scap_sparse_fc_grouped(dev(d["x"], dt), dev(d["W"], dt), f32(m), f32([tau]), None, y, d["ctx"].tolist(), ws.payload)
+            torch.cuda.synchronize()
+            assert bool((ws.payload == CANARY).all().item()) == (route == 1)
+            err[route] = float(np.linalg.norm(y.cpu().numpy() - y64) / np.linalg.norm(y64))
+    finally:
+        S.scap_tune("dense_stream", 1)
+    assert err[1] <= err[0]
 
 
 @pytest.mark.parametrize("dt", [si.F16, si.BF16])
