@@ -452,34 +452,44 @@ __global__ void __launch_bounds__(FC_THREADS, 2) fc_tc_kernel(const FcArgs a) {
 // Dense-stream variant (batch 5..16).  With that many rows the union mask of independent rows keeps nearly every channel
 // (Appendix C), so gathering kept rows buys nothing and costs the memory-level parallelism of the copy engine.  Here
 // the CTA streams ALL rows of its share of the tile - blocks of 64 consecutive rows, block q of rank s = rows
-// (q S + s) 64 .. + 63 - with two TMA box loads per block (64 columns x 64 rows each, 128-byte swizzle: exactly the
-// MN-major B operand of the MMA, no address arithmetic, one instruction per 8 KB), and pruning happens on the small
+// (q S + s) 64 .. + 63 - with two TMA box loads per block (64 columns x 64 rows each, 128-byte swizzle: exactly an
+// MN-major operand of the MMA, no address arithmetic, one instruction per 8 KB), and pruning happens on the small
 // operand instead: a dropped channel gets a zero activation.  Roles: warp 0 issues the TMA loads, warp 1 the MMAs,
 // warps 2-7 threshold one 32-channel chunk at a time (d = x - m, |d| >= tau, ballot for the mask words, exact split into
-// parts of the weight dtype) and write it as the A operand of its stage; W ring and A ring have three or four stages each and
-// share the stage's "empty" barrier.  The epilogue is that of the gather kernel.  Every wait is bounded.
+// parts of the weight dtype) and write it as the activation operand of its stage; both rings have as many stages and
+// share the stage's "empty" barrier.  Every wait is bounded.
+//
+// The 128 columns of the tile are the M rows of the MMA and the activations its N columns: N = 16 .. 96, just what the parts
+// of the batch rows need.  With the roles the other way round M was 128 whatever the batch, and the tensor core multiplied
+// 128 x 128 for 24 or 48 rows of use: back to back the calls then ran into the power limit (1000 W, 1.55 - 1.66 GHz instead of
+// 1.96) and slowed down with the clock.  A column is a TMEM lane now, so a thread of the epilogue finds all parts of its column's
+// results in its own lane and sends them on without a pass through shared memory.  Us per call, back to back for 0.3 s, before -> now:
+// 14336 x 4096, 16 rows 27.3 - 29.3 -> 23.7; 11008 x 4096 dense, 8 rows 19.1 -> 17.6; 4096 x 4096 fp16, 5 rows 10.7 -> 10.2;
+// GELU block of MPT-7B, fp16, 8 rows 57 - 62 -> 48.5; 32 grouped rows of 11008 x 4096 33.3 -> 31.3.
 // ------------------------------------------------------------------------------------------------
 // ROWS = 8 or 16: most batch rows of a call; 32: the rows of a grouped call (scap_grouped.cu), whose operand takes more of the
-// shared memory, so the ring is one stage shorter.
+// shared memory, so the ring is shorter.
 constexpr int DS_STAGE_W = 64 * TC_TN * 2;                      // 16 KB: two boxes of 64 rows x 64 columns
-__host__ __device__ constexpr int ds_nst(int ROWS) { return ROWS <= 16 ? 4 : 3; }
-__host__ __device__ constexpr int ds_a_stage(int groups) { return 4 * 2 * groups * 128; }  // A operand of 64 channels
+constexpr int DS_MAX_NST = 5;
+__host__ __device__ constexpr int ds_nst(int ROWS) { return ROWS == 8 ? 5 : ROWS == 16 ? 4 : 3; }
+__host__ __device__ constexpr int ds_a_stage(int ROWS) { return 4 * 2 * 3 * ROWS * 16; }  // activations of 64 channels, three parts at most
 constexpr int DS_OFF_W = 0;
 __host__ __device__ constexpr int ds_off_a(int ROWS) { return DS_OFF_W + ds_nst(ROWS) * DS_STAGE_W; }
-__host__ __device__ constexpr int ds_off_gather(int ROWS) {  // + slack: the MMA reads 128 rows of M, used or not
-    return ds_off_a(ROWS) + ds_nst(ROWS) * ds_a_stage(ROWS <= 16 ? 6 : 12) + 2560;
+__host__ __device__ constexpr int ds_off_gather(int ROWS) {  // + slack: an odd number of 8-row groups is completed with what follows
+    return ds_off_a(ROWS) + ds_nst(ROWS) * ds_a_stage(ROWS) + 128;
 }
-__host__ __device__ constexpr int ds_gather_rows(int ROWS) { return ROWS <= 16 ? 16 : 32; }
 // (a rank finishes ceil(columns / S) columns, so the slices of all ranks together are up to 12 columns longer than the tile)
-__host__ __device__ constexpr int ds_off_misc(int ROWS) { return ds_off_gather(ROWS) + ds_gather_rows(ROWS) * (TC_TN + 16) * 4; }
+__host__ __device__ constexpr int ds_off_misc(int ROWS) { return ds_off_gather(ROWS) + ROWS * (TC_TN + 16) * 4; }
 __host__ __device__ constexpr int ds_smem(int ROWS) { return ds_off_misc(ROWS) + 512 + 1024; }  // misc block + alignment slack
-static_assert(48 * TC_PART_LD * 4 <= ds_off_gather(16) && 96 * TC_PART_LD * 4 <= ds_off_gather(32), "accumulator copy must fit in the rings");
-static_assert(2 * (ds_smem(16) + 1024) <= 233472 && 2 * (ds_smem(32) + 1024) <= 233472, "two CTAs must fit in the shared memory of an SM");
+static_assert(2 * (ds_smem(8) + 1024) <= 233472 && 2 * (ds_smem(16) + 1024) <= 233472 && 2 * (ds_smem(32) + 1024) <= 233472, "two CTAs must fit in the shared memory of an SM");
+// N columns of the MMA (a multiple of 16 at M = 128) and the TMEM columns of a CTA (a power of two from 32 on)
+__host__ __device__ constexpr int ds_ncols(int ROWS, int nsplit) { return (nsplit * ROWS + 15) / 16 * 16; }
+__host__ __device__ constexpr int ds_tmem_cols(int n) { return n <= 32 ? 32 : n <= 64 ? 64 : n <= 128 ? 128 : 256; }
 
 struct DsMisc {
-    unsigned long long wfull[4];   // TMA bytes of the stage have landed
-    unsigned long long afull[4];   // both chunks of the stage's A operand are written
-    unsigned long long empty[4];   // the stage's MMAs have read W and A
+    unsigned long long wfull[DS_MAX_NST];   // TMA bytes of the stage have landed
+    unsigned long long afull[DS_MAX_NST];   // both chunks of the stage's activation operand are written
+    unsigned long long empty[DS_MAX_NST];   // the stage's MMAs have read both operands
     unsigned long long done;
     unsigned long long recv;            // split-K partials of this rank's columns have landed
     uint32_t tmem_base;
@@ -498,18 +508,14 @@ __device__ __forceinline__ void tma_box_2d(uint32_t dst, const CUtensorMap *map,
                  : "memory");
 }
 
-// 32 accumulator columns of this warp's 32 lanes (complete after tcgen05.wait::ld).
-__device__ __forceinline__ void tc_ld32(uint32_t (&v)[32], uint32_t addr) {
-    asm volatile(
-        "tcgen05.ld.sync.aligned.32x32b.x32.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15, "
-        "%16, %17, %18, %19, %20, %21, %22, %23, %24, %25, %26, %27, %28, %29, %30, %31}, [%32];"
-        : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]), "=r"(v[7]), "=r"(v[8]),
-          "=r"(v[9]), "=r"(v[10]), "=r"(v[11]), "=r"(v[12]), "=r"(v[13]), "=r"(v[14]), "=r"(v[15]), "=r"(v[16]),
-          "=r"(v[17]), "=r"(v[18]), "=r"(v[19]), "=r"(v[20]), "=r"(v[21]), "=r"(v[22]), "=r"(v[23]), "=r"(v[24]),
-          "=r"(v[25]), "=r"(v[26]), "=r"(v[27]), "=r"(v[28]), "=r"(v[29]), "=r"(v[30]), "=r"(v[31])
-        : "r"(addr));
+// 4 or 8 accumulator columns of this warp's 32 lanes (complete after tcgen05.wait::ld).
+__device__ __forceinline__ void tc_ldn(uint32_t (&v)[4], uint32_t addr) {
+    asm volatile("tcgen05.ld.sync.aligned.32x32b.x4.b32 {%0, %1, %2, %3}, [%4];" : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]) : "r"(addr));
 }
-
+__device__ __forceinline__ void tc_ldn(uint32_t (&v)[8], uint32_t addr) {
+    asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+                 : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]), "=r"(v[7]) : "r"(addr));
+}
 // Parts of an activation.  fp16 rows of a grouped call (NACC = 2) take three parts of 4, 9 and 11 bits instead of two of 11: the
 // products with the leading part are 15 bits, so its accumulator has bits to spare and truncates next to nothing, and what the
 // others lose is small.  The gather, whose chains are shorter, is the measure: of 240 fp16 calls of 1024 .. 14336 channels the
@@ -535,23 +541,22 @@ __device__ __forceinline__ void ds_split(float v, unsigned short (&part)[3]) {
 template <bool BF16, int ROWS, int MODE, typename XT, int EPI, int NACC>
 __global__ void __launch_bounds__(FC_THREADS, 2) fc_ds_kernel(const FcArgs a, const __grid_constant__ CUtensorMap tmap) {
     static_assert(ROWS <= 16 || MODE == MODE_GATHER, "the 32-row form is for grouped calls: sparse, no row map, no mask output");
-    constexpr int TNT = TC_TN, HALF = TNT / 2, NSPLIT = ds_nsplit(BF16, NACC), NST = ds_nst(ROWS), GR = ds_gather_rows(ROWS);
+    constexpr int TNT = TC_TN, HALF = TNT / 2, NSPLIT = ds_nsplit(BF16, NACC), NST = ds_nst(ROWS), GR = ROWS;
+    constexpr int NCOLS = ds_ncols(ROWS, NSPLIT), TCOLS = ds_tmem_cols(NACC * NCOLS);
     extern __shared__ unsigned char smem_raw[];
     unsigned char *smem = reinterpret_cast<unsigned char *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
     unsigned char *s_w = smem + DS_OFF_W;
     unsigned char *s_a = smem + ds_off_a(ROWS);
     float *s_gather = reinterpret_cast<float *>(smem + ds_off_gather(ROWS));
     DsMisc *misc = reinterpret_cast<DsMisc *>(smem + ds_off_misc(ROWS));
-    float *s_part = reinterpret_cast<float *>(s_w);  // accumulator rows, after the stream
     volatile int *abort_flag = &misc->abort;
     const uint32_t spin = a.spin ? (uint32_t)a.spin : TC_SPIN;
 
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int tile = blockIdx.x, s = blockIdx.y;
     const int B = a.B, S = a.S, K = a.K;
-    const int racc = NSPLIT * B;
-    const int G = tc_groups(B, NSPLIT);
-    const uint32_t LBO = G * 128, BLK = 2 * LBO, ASTG = 4 * BLK;
+    // activation operand: row r = part * ROWS + batch row, K-major core matrices of 8 rows x 16 bytes
+    constexpr uint32_t LBO = NSPLIT * ROWS * 16, BLK = 2 * LBO, ASTG = 4 * BLK;
     const XT *xg = reinterpret_cast<const XT *>(a.x);
     const int nblk64 = (K + 63) >> 6;
     const int nq = nblk64 > s ? (nblk64 - s + S - 1) / S : 0;  // 64-row blocks (= stages) of this rank
@@ -619,7 +624,7 @@ __global__ void __launch_bounds__(FC_THREADS, 2) fc_ds_kernel(const FcArgs a, co
         }
     }
     if (warp == 0) {
-        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&misc->tmem_base)), "r"(NACC * TNT) : "memory");
+        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&misc->tmem_base)), "r"(TCOLS) : "memory");
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
     }
     float bias0[2], bias1[2];
@@ -640,8 +645,8 @@ __global__ void __launch_bounds__(FC_THREADS, 2) fc_ds_kernel(const FcArgs a, co
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem = misc->tmem_base;
-    const uint32_t idesc = (1u << 4) | ((BF16 ? 1u : 0u) << 7) | ((BF16 ? 1u : 0u) << 10) | (0u << 15) | (1u << 16) |
-                           ((uint32_t)(TNT >> 3) << 17) | ((uint32_t)(128 >> 4) << 24);
+    const uint32_t idesc = (1u << 4) | ((BF16 ? 1u : 0u) << 7) | ((BF16 ? 1u : 0u) << 10) | (1u << 15) | (0u << 16) |
+                           ((uint32_t)(NCOLS >> 3) << 17) | ((uint32_t)(TNT >> 4) << 24);
 
     if (warp == 0) {
         // ---- TMA producer: two boxes per stage
@@ -676,12 +681,12 @@ __global__ void __launch_bounds__(FC_THREADS, 2) fc_ds_kernel(const FcArgs a, co
                 misc->issued = 1;
 #pragma unroll
                 for (uint32_t kb = 0; kb < 4; ++kb) {
-                    const uint64_t da = tc_desc(smem_u32(s_a) + st * ASTG + kb * BLK, LBO, 128, 0);
-                    const uint64_t db = tc_desc(smem_u32(s_w) + st * DS_STAGE_W + kb * 2048, DS_STAGE_W / 2, 1024, 2);
+                    const uint64_t dw = tc_desc(smem_u32(s_w) + st * DS_STAGE_W + kb * 2048, DS_STAGE_W / 2, 1024, 2);
+                    const uint64_t dx = tc_desc(smem_u32(s_a) + st * ASTG + kb * BLK, LBO, 128, 0);
                     // NACC = 2: stages alternate between two accumulators.  The tensor core truncates where it adds to one, so half
                     // the chain is half the error (K = 14336 in eight ranks: 9.5e-7 -> 4.2e-7); plain calls keep to one,
                     // which is 1 % faster.
-                    tc_mma(tmem + (uint32_t)(q & (NACC - 1)) * TNT, da, db, idesc, (q >= NACC || kb > 0) ? 1u : 0u);
+                    tc_mma(tmem + (uint32_t)(q & (NACC - 1)) * NCOLS, dw, dx, idesc, (q >= NACC || kb > 0) ? 1u : 0u);
                 }
                 tc_commit(&misc->empty[st]);
             }
@@ -689,7 +694,7 @@ __global__ void __launch_bounds__(FC_THREADS, 2) fc_ds_kernel(const FcArgs a, co
         }
         __syncwarp();
     } else {
-        // ---- A operand: chunk jc = stage 2 q + half h; element (row r = part * B + b, position pos of the stage): block
+        // ---- activations: chunk jc = stage 2 q + half h; element (row r = part * ROWS + b, position pos of the stage): block
         // pos / 16, K half (pos / 8) & 1, 8-row group r / 8, 16 bytes per row of the group, 2 bytes per position.
         // A lane takes ONE batch row and ROWS consecutive channels of the chunk (lane = channel group * ROWS + row): its
         // activations are one or two 16-byte loads, and the eight positions of a row inside a K half are one 16-byte
@@ -746,14 +751,14 @@ __global__ void __launch_bounds__(FC_THREADS, 2) fc_ds_kernel(const FcArgs a, co
                     mine |= kept ? (1u << i) : 0u;
                     ds_split<BF16, NACC>(kept ? dv : 0.0f, part[i]);
                 }
-                if (b < B) {
+                {  // (rows that the batch does not have: zeros)
 #pragma unroll
                     for (int v = 0; v < CPL / 8; ++v) {
                         const int pos = h * 32 + ch0 + 8 * v;   // first of eight consecutive positions: one K half of one block
                         unsigned char *dst = s_a + st * ASTG + (size_t)(pos >> 4) * BLK + ((pos >> 3) & 1) * LBO;
 #pragma unroll
                         for (int p = 0; p < NSPLIT; ++p) {
-                            const int r = p * B + b;
+                            const int r = p * ROWS + b;
                             uint4 w;
                             w.x = (uint32_t)part[8 * v + 0][p] | ((uint32_t)part[8 * v + 1][p] << 16);
                             w.y = (uint32_t)part[8 * v + 2][p] | ((uint32_t)part[8 * v + 3][p] << 16);
@@ -833,14 +838,14 @@ __global__ void __launch_bounds__(FC_THREADS, 2) fc_ds_kernel(const FcArgs a, co
                     const bool kept = b < B && k0 + i < K && fabsf(dv) >= tau;
                     ds_split<BF16, NACC>(kept ? dv : 0.0f, part[i]);
                 }
-                if (b < B) {
+                {
 #pragma unroll
                     for (int v = 0; v < CPL / 8; ++v) {
                         const int pos = h * 32 + chu + 8 * v;   // first of eight consecutive positions: one K half of one block
                         unsigned char *dst = s_a + st * ASTG + (size_t)(pos >> 4) * BLK + ((pos >> 3) & 1) * LBO;
 #pragma unroll
                         for (int p = 0; p < NSPLIT; ++p) {
-                            const int r = p * B + b;
+                            const int r = p * ROWS + b;
                             uint4 w;
                             w.x = (uint32_t)part[8 * v + 0][p] | ((uint32_t)part[8 * v + 1][p] << 16);
                             w.y = (uint32_t)part[8 * v + 2][p] | ((uint32_t)part[8 * v + 3][p] << 16);
@@ -872,36 +877,16 @@ __global__ void __launch_bounds__(FC_THREADS, 2) fc_ds_kernel(const FcArgs a, co
         mbar_wait(&misc->done, 0, 4, &drain_abort, TC_SPIN);
     }
     const bool have_acc = nq > 0 && !*abort_flag, two = NACC == 2 && nq > 1;
-    // Accumulator rows (part p of batch row b = row p B + b = TMEM lane) to shared memory.  A warp reaches the 32 lanes
-    // of its quarter (warp mod 4), so warps 0 and 4 share lanes 0-31, warps 1 and 5 lanes 32-63 (and so on), half the columns each.
-    if (have_acc && (warp & 3) * 32 < racc) {
-        const int lq = warp & 3;
-#pragma unroll 1
-        for (int c0 = (warp >> 2) * 64; c0 < (warp >> 2) * 64 + 64; c0 += 32) {
-            uint32_t v[32], w[32];
-            tc_ld32(v, tmem + ((uint32_t)(lq * 32) << 16) + (uint32_t)c0);
-            if (two) tc_ld32(w, tmem + ((uint32_t)(lq * 32) << 16) + (uint32_t)(TNT + c0));
-            asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-            const int r = lq * 32 + lane;
-            if (r < racc) {
-#pragma unroll
-                for (int j = 0; j < 32; ++j) s_part[r * TC_PART_LD + c0 + j] = two ? __uint_as_float(v[j]) + __uint_as_float(w[j]) : __uint_as_float(v[j]);
-            }
-        }
-    }
-    tc_fence_before();
-    __syncthreads();
-    tc_fence_after();
-    if (warp == 0) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(NACC * TNT) : "memory");
-    // ---- cluster exchange, push form: the parts of an element are added (smallest first) and the sum goes straight to
-    // the cluster rank that finishes its column - slot (this rank, row) of that rank's gather buffer - as an asynchronous
-    // store that counts down the owner's barrier.  No cluster-wide barrier after the prologue: a rank finishes its columns
-    // as soon as its own S partials are in, and may leave while its stores to the others are still under way.
+    // ---- cluster exchange, push form: a column of the tile is a TMEM lane, part p of batch row b its column p ROWS + b.  A warp
+    // reaches the 32 lanes of its quarter (warp mod 4), so warps w and w + 4 share 32 columns, half the rows each.  A thread adds the
+    // parts of an element (smallest first) and the sum goes straight to the cluster rank that finishes its column - slot (this
+    // rank, row) of that rank's gather buffer - as an asynchronous store that counts down the owner's barrier.  No
+    // cluster-wide barrier after the prologue: a rank finishes its columns as soon as its own S partials are in, and may
+    // leave while its stores to the others are still under way.
     if (S > 1) cluster_wait();  // every rank's barrier is initialised (all ranks arrived before their streams)
     {
-        // A thread keeps one column and walks the rows (two row phases per CTA), so owner, slot and the owner's
-        // addresses are computed once.
-        const int c = tid % TNT;
+        constexpr int RPW = ROWS / 2, RL = RPW < 8 ? RPW : 8;  // rows per warp, and at a time
+        const int c = (warp & 3) * 32 + lane;
         int r, slot0, bstride;
         if constexpr (EPI == EPI_GLU) {
             const int j = c % HALF, hf = c / HALF;
@@ -915,22 +900,50 @@ __global__ void __launch_bounds__(FC_THREADS, 2) fc_ds_kernel(const FcArgs a, co
         }
         const uint32_t dst0 = S > 1 ? cluster_addr(smem_addr(s_gather) + 4u * (uint32_t)slot0, (uint32_t)r) : 0u;
         const uint32_t dbar = S > 1 ? cluster_addr(recv_bar, (uint32_t)r) : 0u;
-        for (int b = tid / TNT; b < B; b += FC_THREADS / TNT) {
-            float v = 0.0f;
+        const uint32_t lanes = tmem + ((uint32_t)((warp & 3) * 32) << 16);
+#pragma unroll
+        for (int b0 = (warp >> 2) * RPW, i = 0; i < RPW / RL; ++i, b0 += RL) {
+            if (b0 >= B) break;  // (the same for the whole warp)
+            uint32_t v[NSPLIT][RL], w[NACC == 2 ? NSPLIT : 1][RL];
             if (have_acc) {
 #pragma unroll
-                for (int p = NSPLIT - 1; p >= 0; --p) v += s_part[(p * B + b) * TC_PART_LD + c];
+                for (int p = 0; p < NSPLIT; ++p) {
+                    tc_ldn(v[p], lanes + (uint32_t)(p * ROWS + b0));
+                    if constexpr (NACC == 2) {
+                        if (two) tc_ldn(w[p], lanes + (uint32_t)(NCOLS + p * ROWS + b0));
+                    }
+                }
+                asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
             }
-            if (S > 1) st_async_f32(dst0 + 4u * (uint32_t)(b * bstride), v, dbar);
-            else s_gather[slot0 + b * bstride] = v;
+#pragma unroll
+            for (int e = 0; e < RL; ++e) {
+                const int b = b0 + e;
+                float sum = 0.0f;
+                if (have_acc) {
+#pragma unroll
+                    for (int p = NSPLIT - 1; p >= 0; --p) {
+                        float t = __uint_as_float(v[p][e]);
+                        if constexpr (NACC == 2) {
+                            if (two) t += __uint_as_float(w[p][e]);
+                        }
+                        sum += t;
+                    }
+                }
+                if (b < B) {
+                    if (S > 1) st_async_f32(dst0 + 4u * (uint32_t)(b * bstride), sum, dbar);
+                    else s_gather[slot0 + b * bstride] = sum;
+                }
+            }
         }
     }
+    tc_fence_before();
+    __syncthreads();
+    tc_fence_after();
+    if (warp == 0) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(TCOLS) : "memory");
     if (S > 1) {
         bool landed = false;
         for (uint32_t it = 0; it < (1u << 22) && !landed; ++it) landed = mbarrier_try_wait(recv_bar, 0);
         if (!landed) atomicCAS(&g_tc_status, 0, 6);  // never in a correct run; the result is then incomplete
-    } else {
-        __syncthreads();
     }
     finish_columns<BF16, GR, EPI, TNT>(a, tile, s, per, s_gather, bias0, bias1);
 }
