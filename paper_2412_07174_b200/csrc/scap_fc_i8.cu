@@ -1,0 +1,603 @@
+// 8-bit weights as integers on the 5th-generation tensor cores: the sparse FC on signed 8-bit codes with tcgen05.mma kind::i8.
+//
+// The codes are integers, so they go into the tensor core as they lie in memory: the 128 columns of a tile are the M rows of the
+// MMA, and a TMA box of 128 channels with 128-byte swizzle is its operand (MN-major).  The activations become integers too: the
+// pruned and scaled values of a batch row are rounded to 31-bit fixed point under a common exponent, that of the largest one
+// among the rank's channels, and cut into four signed 8-bit digits, which are the N columns of the MMA (digit x BR + row).  Products
+// and sums are exact 32-bit integers in one accumulator, read once at the end.  So a weight costs no instruction at all, where the
+// mma.sync kernel (scap_fc_qm.cu) spends 1.5 on its conversion to bf16, and an activation is prepared once per CTA instead of once
+// per warp.
+//
+//   grid = (128-column tiles, S), cluster (1, S, 1), 384 threads, two CTAs per SM; a rank takes a contiguous range of blocks of
+//   128 channels; two blocks are a stage of the ring
+//   warp 0      boxes and MMAs (the whole warp runs the loop, one lane issues)
+//   warps 1-11  activations: a unit is a block's 128 channels of four batch rows, a lane has four channels of each row.  First the
+//               largest value of every row (the warp keeps the values of its first units in registers), then the digits
+//   warps 4-7   at the end: a thread per column reads the accumulator
+//
+// Precision: a value is off by at most 2^-31 of the largest of its row in the rank, the sum of a rank is put together from its digits
+// with three roundings to binary32: 5e-8 .. 7e-8 from 64 bits where the mma.sync kernel is 6e-8 .. 9e-8 off (128 x 128 to
+// 14336 x 11008, 1 - 16 rows).  A kept value that is not finite is left out of the digits and its row is marked; value x code of
+// those channels is then added one by one.
+//
+// What bounds it: K = 11008, N = 4096, half pruned, weights from DRAM, us per call, mma.sync kernel -> this one: 3 rows
+// 18.1 -> 11.4, 8 rows 24.0 -> 14.9, 16 rows 41.4 -> 20.3 (the 45 MB of codes take 6.9 at copy speed).  The first MMA starts 3 - 4 us
+// into the call: activations through L2 (1 us under the weight stream), the pass for the exponents, the digits - code that all 24
+// warps of an SM run at once, bound by instruction issue - while the ring has been full for two of them; the rest of the codes then
+// comes at 5.9 TB/s.  Tried and slower: an exponent per block and an accumulator per block or two, so that the first MMA does not
+// wait for a pass over all activations (8 rows 15.4 - 16.3, 16 rows 21.5 - 30.6: reading 11 accumulators costs more than the pass);
+// 256 threads (15.4); 4-bit codes the same way, the nibbles separated in shared memory (11008 x 4096, one row 15.4 - 27 against 13.0:
+// half the bytes per stage, and an accumulator read per scale group).
+// Every wait is bounded (as in scap_fc_tc.cu): one that runs out sets the status word, the CTA stops issuing work, still passes
+// its barriers, waits for the copies and MMAs under way and frees its TMEM.
+#include <string.h>
+
+#include <type_traits>
+
+#include "scap_qm.cuh"
+#include "scap_tc.cuh"
+
+namespace scap {
+
+constexpr int I8_TN = 128;        // columns per CTA
+constexpr int I8_KB = 128;        // channels per block (a box, a unit of activations)
+constexpr int I8_BPS = 2;         // blocks per stage: eight MMAs of 32 channels per round of waits
+constexpr int I8_THREADS = 384;
+constexpr int I8_PREP = I8_THREADS / 32 - 1;  // warps that prepare activations
+constexpr int I8_KEEP = 2;        // units whose values a warp keeps between the two passes
+static_assert(I8_KEEP == 2, "the first pass asks for two units at once");
+constexpr int I8_BOX = I8_KB * I8_TN;         // 16 KB
+// BR = batch rows of the instantiation (4, 8 or 16).
+// 16 channels of the activation operand: 4 BR rows of 16 bytes, and 16 bytes more, so that the chunks of a warp's stores start in different banks
+__host__ __device__ constexpr int i8_chunk(int BR) { return 4 * BR * 16 + 16; }
+__host__ __device__ constexpr int i8_xbytes(int BR) { return I8_BPS * I8_KB / 16 * i8_chunk(BR); }
+__host__ __device__ constexpr int i8_nw(int BR) { return BR == 16 ? 4 : 5; }  // blocks of weights in the ring
+// Stages of activations.  At least as many as lie between two units of a warp (11 units go round; one, two, or three and four per block):
+// a warp then meets every phase of a slot's barrier, which a parity only tells from its neighbours.
+__host__ __device__ constexpr int i8_nx(int BR) { return BR == 4 ? 6 : BR == 8 ? 3 : 2; }
+constexpr int i8_apart(int ups) { return ((I8_PREP + ups - 1) / ups + I8_BPS - 1) / I8_BPS; }  // stages between two units of a warp, at most
+static_assert(i8_apart(1) <= i8_nx(4) && i8_apart(2) <= i8_nx(8) && i8_apart(3) <= i8_nx(16) && i8_apart(4) <= i8_nx(16),
+              "units of a warp must not lie further apart than the slots of the activations reach");
+// What the host works out once instead of every warp of every CTA: the code before the first MMA runs on all warps of an SM at the same
+// moment and is bound by instruction issue (a division costs a warp as much as the activations of a row).
+struct I8Args {
+    FcArgs f;
+    int blocks, extra;  // blocks per rank; the first `extra` ranks have one more
+    int per;            // columns a rank finishes (the last rank may own fewer)
+    uint32_t per_inv;   // ceil(2^20 / per): (i * per_inv) >> 20 = i / per for i < 2048
+};
+struct I8Misc {
+    unsigned long long wfull[5], wempty[5];  // a block of weights has landed / has been multiplied
+    unsigned long long xfull[6], xempty[6];  // activations of a stage
+    unsigned long long done, recv;
+    uint32_t tmem_base;
+    int abort;
+    uint32_t top[16], fin[16];  // pattern of a row's largest magnitude; of the largest finite one
+};
+__host__ __device__ constexpr int i8_off_x(int BR) { return i8_nw(BR) * I8_BOX; }
+__host__ __device__ constexpr int i8_off_gather(int BR) { return i8_off_x(BR) + i8_nx(BR) * i8_xbytes(BR); }
+__host__ __device__ constexpr int i8_off_misc(int BR) { return i8_off_gather(BR) + BR * (I8_TN + 16) * 4; }
+__host__ __device__ constexpr int i8_smem(int BR) { return i8_off_misc(BR) + (int)sizeof(I8Misc) + 1024; }
+static_assert(2 * (i8_smem(4) + 1024) <= 233472 && 2 * (i8_smem(8) + 1024) <= 233472 && 2 * (i8_smem(16) + 1024) <= 233472,
+              "two CTAs must fit in the shared memory of an SM");
+
+__device__ __forceinline__ void tc_mma_i8(uint32_t d_tmem, uint64_t a_desc, uint64_t b_desc, uint32_t idesc, uint32_t accumulate) {
+    asm volatile(
+        "{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\t"
+        "tcgen05.mma.cta_group::1.kind::i8 [%0], %1, %2, %3, {%5, %5, %5, %5}, p;\n\t}\n" ::"r"(d_tmem),
+        "l"(a_desc), "l"(b_desc), "r"(idesc), "r"(accumulate), "r"(0u)
+        : "memory");
+}
+// Predicated 8-byte activation load through L2 (zeros where off).
+__device__ __forceinline__ uint2 ld_act8_if(const void *p, bool on) {
+    uint2 v;
+    asm volatile("{ .reg .pred q; setp.ne.u32 q, %3, 0; mov.u32 %0, 0; mov.u32 %1, 0; @q ld.global.cg.v2.u32 {%0,%1}, [%2]; }"
+                 : "=r"(v.x), "=r"(v.y) : "l"(p), "r"((unsigned)on) : "memory");
+    return v;
+}
+__device__ __forceinline__ uint2 ld_act8(const void *p) {
+    uint2 v;
+    asm volatile("ld.global.cg.v2.u32 {%0,%1}, [%2];" : "=r"(v.x), "=r"(v.y) : "l"(p) : "memory");
+    return v;
+}
+__device__ __forceinline__ uint4 ld_act16u(const void *p) {
+    uint4 v;
+    asm volatile("ld.global.cg.v4.u32 {%0,%1,%2,%3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "l"(p) : "memory");
+    return v;
+}
+// A bounded wait that sleeps in the barrier instead of polling (after a first look).
+__device__ __forceinline__ bool i8_wait(unsigned long long *bar, uint32_t parity, int code, volatile int *abort_flag, uint32_t limit, int *status) {
+    for (uint32_t i = 0; i < limit; ++i) {
+        if (i == 0 ? mbar_test(bar, parity) : mbarrier_try_wait(smem_u32(bar), parity)) return true;
+        if (*abort_flag) return false;
+    }
+    if (status) atomicCAS(status, 0, code);
+    *abort_flag = 1;
+    return false;
+}
+
+// Sum of value x code over the channels k0 .. k1 - 1 whose kept value is not finite, one batch row and one column.
+template <int MODE, typename XT>
+__device__ __noinline__ float i8_not_finite(const FcArgs *a, int k0, int k1, int b, int col) {
+    const float tau = MODE == MODE_GATHER ? ld_act(a->tau) : 0.0f;
+    float sum = 0.0f;
+    for (int k = k0; k < k1; ++k) {
+        float v = widen1(ld_act(static_cast<const XT *>(a->x) + (size_t)b * a->x_ld + k));
+        if (MODE == MODE_GATHER && a->m) v = __fsub_rn(v, ld_act(a->m + k));
+        if (MODE == MODE_GATHER && !(fabsf(v) >= tau)) continue;
+        v = __fmul_rn(v, ld_act(a->wscale + k));
+        if ((__float_as_uint(v) & 0x7f800000u) == 0x7f800000u) sum += v * (float)static_cast<const signed char *>(a->W)[(size_t)k * a->ldw + col];
+    }
+    return sum;
+}
+
+__device__ __forceinline__ uint32_t i8_bits(float v) { return __float_as_uint(v) & 0x7fffffffu; }
+__device__ __forceinline__ uint32_t i8_top(const float (&v)[4]) { return max(max(i8_bits(v[0]), i8_bits(v[1])), max(i8_bits(v[2]), i8_bits(v[3]))); }
+// Fixed point under the exponent of `top`: |v| < 2^(e - 126), so times 2^(156 - e) it is below 2^30 (where the largest value is under
+// 2^-96, bits below 2^-156 are lost).
+__device__ __forceinline__ int i8_shift(uint32_t top) { return min(156 - (int)(top >> 23), 126); }
+__device__ __forceinline__ float i8_pow2(int e) { return __uint_as_float((uint32_t)(127 + e) << 23); }
+
+template <int BR, int MODE, typename XT>
+__global__ void __launch_bounds__(I8_THREADS, 2) fc_i8_kernel(const __grid_constant__ I8Args ia, const __grid_constant__ CUtensorMap tmap) {
+    const FcArgs &a = ia.f;
+    constexpr int NC = 4 * BR, NW = i8_nw(BR), NX = i8_nx(BR);
+    constexpr uint32_t XB = i8_xbytes(BR), LBO = i8_chunk(BR), TCOLS = NC < 32 ? 32 : NC;
+    extern __shared__ unsigned char smem_raw[];
+    unsigned char *smem = reinterpret_cast<unsigned char *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
+    unsigned char *s_w = smem, *s_x = smem + i8_off_x(BR);
+    float *s_gather = reinterpret_cast<float *>(smem + i8_off_gather(BR));
+    I8Misc *misc = reinterpret_cast<I8Misc *>(smem + i8_off_misc(BR));
+    volatile int *abort_flag = &misc->abort;
+    const uint32_t spin = a.spin ? (uint32_t)a.spin : TC_SPIN;
+    int *const status = a.status;
+
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int tile = blockIdx.x, s = blockIdx.y;
+    const int B = a.B, S = a.S, K = a.K;
+    const int per = ia.per;
+    const uint32_t recv_bar = smem_addr(&misc->recv);
+    const int b_lo = s * ia.blocks + min(s, ia.extra), n = ia.blocks + (s < ia.extra ? 1 : 0);  // this rank's blocks
+    const int k_lo = b_lo * I8_KB, k_hi = min(K, k_lo + n * I8_KB), nst = (n + I8_BPS - 1) / I8_BPS;   // its channels and stages
+    const int ups = (B + 3) >> 2;  // units of a block: four batch rows each
+    if (tid == 0) {
+        for (int i = 0; i < NW; ++i) {
+            mbar_init(&misc->wfull[i], 1);
+            mbar_init(&misc->wempty[i], 1);
+        }
+        for (int i = 0; i < NX; ++i) {
+            mbar_init(&misc->xfull[i], I8_BPS * ups);
+            mbar_init(&misc->xempty[i], 1);
+        }
+        mbar_init(&misc->done, 1);
+        misc->abort = 0;
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+        if (S > 1) {
+            const int owned = max(0, min(per, I8_TN - s * per));
+            mbarrier_init(recv_bar, 1);
+            mbarrier_arrive_expect(recv_bar, (uint32_t)(S * B * owned * 4));
+        }
+    }
+    if (tid < 16) misc->top[tid] = misc->fin[tid] = 0;
+    if (S > 1) cluster_arrive_relaxed();
+    // m, x and the scales are asked into L2 ahead of the weight stream (hints, as in the dense-stream kernel)
+    if (warp == 1 && MODE == MODE_GATHER && a.m)
+        for (int k = k_lo + lane * 32; k < k_hi; k += 1024) prefetch_l2_keep(a.m + k);
+    if (warp == 2)
+        for (int k = k_lo + lane * 32; k < k_hi; k += 1024) prefetch_l2_keep(a.wscale + k);
+    if (warp >= 4)
+        for (int b = warp - 4; b < B; b += 8)
+            for (int k = k_lo + lane * 64; k < k_hi; k += 2048) prefetch_l2_keep(static_cast<const XT *>(a.x) + (size_t)b * a.x_ld + k);
+    // The codes are constants of the layer: the first ring is asked for before the wait for earlier work on the stream.
+    auto box = [&](int blk, uint32_t slot) {
+        mbar_arrive_expect_tx(&misc->wfull[slot], I8_BOX);
+        tma_box_2d(smem_u32(s_w) + slot * I8_BOX, &tmap, tile * I8_TN, (b_lo + blk) * I8_KB, &misc->wfull[slot]);
+    };
+    const int first = min(n, NW);
+    if (tid == 0) {
+        for (int i = 0; i < first; ++i) box(i, i);
+    }
+    if (warp == 0) {
+        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&misc->tmem_base)), "r"(TCOLS) : "memory");
+        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+    }
+    tc_fence_before();
+    __syncthreads();  // barriers and TMEM address
+    tc_fence_after();
+    griddep_wait();
+    griddep_launch_dependents();
+
+    struct Raw {
+        uint4 m, c;
+        uint2 x[4];
+    } raw, raw1;
+    // Units go round the preparing warps, (ub, uq) = block and quarter of the rows.
+    const uint32_t ups_inv = ups == 3 ? 86u : 256u >> (ups >> 1);  // ceil(256 / ups)
+    const int di = (I8_PREP * ups_inv) >> 8, dq = I8_PREP - di * ups;
+    int ub = ((warp - 1) * ups_inv) >> 8, uq = (warp - 1) - ub * ups;
+    auto step = [&](int &blk, int &rq) {
+        blk += di;
+        rq += dq;
+        if (rq >= ups) {
+            rq -= ups;
+            ++blk;
+        }
+    };
+    auto load = [&](Raw &raw, int blk, int rq) {
+        const int kb = k_lo + blk * I8_KB, k = kb + lane * 4, b0 = rq * 4;
+        const XT *xp = static_cast<const XT *>(a.x) + (size_t)b0 * a.x_ld + k;
+        if (kb + I8_KB <= k_hi && (MODE == MODE_DENSE || a.m)) {
+            // (a row that the batch does not have repeats the last one; its values are not used)
+#pragma unroll
+            for (int r = 0; r < 4; ++r) {
+                raw.x[r] = ld_act8(xp);
+                if (b0 + r + 1 < B) xp += a.x_ld;
+            }
+            if constexpr (MODE == MODE_GATHER) raw.m = ld_act16u(a.m + k);
+            raw.c = ld_act16u(a.wscale + k);
+        } else {
+            const bool in = k < k_hi;  // (K is a multiple of eight: four channels are inside the matrix or outside together)
+#pragma unroll
+            for (int r = 0; r < 4; ++r) raw.x[r] = ld_act8_if(xp + (size_t)r * a.x_ld, in && b0 + r < B);
+            if constexpr (MODE == MODE_GATHER) raw.m = ld_act16_if(a.m + k, in && a.m != nullptr);
+            raw.c = ld_act16_if(a.wscale + k, in);
+        }
+    };
+    float tau = 0.0f;
+    // Pruned and scaled values of row r of the unit: zeros for dropped channels.  Beyond the matrix everything is zero, kept or not.
+    auto value = [&](const Raw &raw, int r, float (&v)[4]) {
+        const XT *xe = reinterpret_cast<const XT *>(&raw.x[r]);
+        const float *me = reinterpret_cast<const float *>(&raw.m), *ce = reinterpret_cast<const float *>(&raw.c);
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+            float d = widen1(xe[e]);
+            if constexpr (MODE == MODE_GATHER) d = __fsub_rn(d, me[e]);  // (m == NULL: zeros)
+            const bool on = MODE == MODE_DENSE || fabsf(d) >= tau;
+            v[e] = on ? __fmul_rn(d, ce[e]) : 0.0f;  // (the scale of a dropped channel has no part in y, whatever it is)
+        }
+    };
+    float keep[I8_KEEP][4][4];
+    if (warp >= 1) {
+        if (ub < n) load(raw, ub, uq);
+        if constexpr (MODE == MODE_GATHER) tau = ld_act(a.tau);
+        int b1 = ub, q1 = uq;
+        step(b1, q1);
+        if (b1 < n) load(raw1, b1, q1);
+        // ---- first pass: the largest value of every row
+        int blk = ub, rq = uq;
+        auto largest = [&](const Raw &raw, float (&v)[4][4]) {
+            const int b0 = rq * 4;
+            uint32_t top[4];
+#pragma unroll
+            for (int r = 0; r < 4; ++r) {
+                if (b0 + r < B) {
+                    value(raw, r, v[r]);
+                    top[r] = i8_top(v[r]);
+                }
+            }
+            if (MODE == MODE_GATHER && BR == 4 && a.bits && tile == 0) {  // union mask (up to two rows), a word per 32 channels = eight lanes
+                const int k = k_lo + blk * I8_KB + lane * 4;
+                const float *me = reinterpret_cast<const float *>(&raw.m);
+                uint32_t w = 0;
+#pragma unroll
+                for (int e = 0; e < 4; ++e) {
+                    const bool k0 = fabsf(__fsub_rn(widen1(reinterpret_cast<const XT *>(&raw.x[0])[e]), me[e])) >= tau;
+                    const bool k1 = B > 1 && fabsf(__fsub_rn(widen1(reinterpret_cast<const XT *>(&raw.x[1])[e]), me[e])) >= tau;
+                    w |= k0 || k1 ? 1u << e : 0u;
+                }
+                w = k < k_hi ? w << (4 * (lane & 7)) : 0u;
+#pragma unroll
+                for (int o = 1; o < 8; o <<= 1) w |= __shfl_xor_sync(0xffffffffu, w, o);
+                if ((lane & 7) == 0 && k < k_hi) a.bits[k >> 5] = w;
+            }
+            step(blk, rq);
+#pragma unroll
+            for (int r = 0; r < 4; ++r) {
+                if (b0 + r < B) {
+                    const uint32_t t = __reduce_max_sync(0xffffffffu, top[r]);
+                    if (lane == 0) atomicMax(&misc->top[b0 + r], t);
+                }
+            }
+        };
+        if (blk < n) largest(raw, keep[0]);
+        int b2 = b1, q2 = q1;
+        step(b2, q2);
+        if (b2 < n) load(raw, b2, q2);  // asked for two units ahead
+        if (blk < n) largest(raw1, keep[1]);
+#pragma unroll 1
+        while (blk < n) {
+            float v[4][4];
+            raw1 = raw;
+            step(b2, q2);
+            if (b2 < n) load(raw, b2, q2);
+            largest(raw1, v);
+        }
+    }
+    __syncthreads();
+    uint32_t odd = 0;  // rows with a value that is not finite
+#pragma unroll
+    for (int b = 0; b < BR; ++b) odd |= misc->top[b] >= 0x7f800000u ? 1u << b : 0u;
+    if (odd) {  // the largest of the others (rare; the same for the whole CTA)
+        if (warp >= 1) {
+            for (int blk = ub, rq = uq; blk < n; step(blk, rq)) {
+                load(raw, blk, rq);
+#pragma unroll
+                for (int r = 0; r < 4; ++r) {
+                    float v[4];
+                    uint32_t t = 0;
+                    value(raw, r, v);
+#pragma unroll
+                    for (int e = 0; e < 4; ++e) t = max(t, i8_bits(v[e]) < 0x7f800000u ? i8_bits(v[e]) : 0u);
+                    atomicMax(&misc->fin[rq * 4 + r], t);
+                }
+            }
+        }
+        __syncthreads();
+        if (tid < BR && (odd >> tid & 1)) misc->top[tid] = misc->fin[tid];
+        __syncthreads();
+    }
+    const uint32_t tmem = misc->tmem_base;
+    // A wait by a whole warp; all lanes agree on the outcome.
+    auto warp_wait = [&](unsigned long long *bar, uint32_t parity, int code) -> bool {
+        const bool go = i8_wait(bar, parity, code, abort_flag, spin, status);
+        return __all_sync(0xffffffffu, go) != 0;
+    };
+
+    if (warp == 0) {
+        // ---- MMAs.  D: 32-bit integers; codes signed, MN-major; digits signed, K-major.  The whole warp runs the loop and one
+        // lane issues: descriptors and addresses then stay in uniform registers (with the loop inside `if (lane == 0)` 128 channels
+        // took 1600 cycles instead of 430).
+        uint32_t leader;
+        asm volatile("{ .reg .pred p; elect.sync _|p, 0xffffffff; selp.u32 %0, 1, 0, p; }" : "=r"(leader));
+        constexpr uint32_t idesc = (2u << 4) | (1u << 7) | (1u << 10) | (1u << 15) | ((uint32_t)(NC >> 3) << 17) | ((uint32_t)(I8_TN >> 4) << 24);
+        constexpr uint32_t WK = 32 * I8_TN >> 4, XK = (2 * LBO) >> 4;  // 32 channels further, in units of 16 bytes
+        const uint64_t dw0 = tc_desc(smem_u32(s_w), I8_BOX, 1024, 2), dx0 = tc_desc(smem_u32(s_x), LBO, 128, 0);
+        uint32_t ws = 0, wpar = 0, xs = 0, xpar = 0, rs = 0, rpar = 0;  // slots: weights, activations, weights to ask for
+        auto next = [&](uint32_t &slot, uint32_t &par) {
+            if (++slot == NW) { slot = 0; par ^= 1u; }
+        };
+        int asked = first;
+#pragma unroll 1
+        for (int i = 0; i < nst; ++i) {
+            // both operands, and the slots of the stage before, which take the next boxes: each is waited for by a lane of its own
+            const bool two = 2 * i + 1 < n;
+            const int refill = i >= 1 ? min(2, n - asked) : 0;
+            uint32_t ws1 = ws, wpar1 = wpar, rs1 = rs, rpar1 = rpar;
+            next(ws1, wpar1);
+            next(rs1, rpar1);
+            unsigned long long *bar = &misc->wfull[ws];
+            uint32_t bpar = wpar;
+            if (lane == 1) { bar = &misc->xfull[xs]; bpar = xpar; }
+            if (lane == 2 && two) { bar = &misc->wfull[ws1]; bpar = wpar1; }
+            if (lane == 3 && refill > 0) { bar = &misc->wempty[rs]; bpar = rpar; }
+            if (lane == 4 && refill > 1) { bar = &misc->wempty[rs1]; bpar = rpar1; }
+            if (!warp_wait(bar, bpar, 2)) break;
+            tc_fence_after();
+            const uint64_t da = dw0 + ws * (I8_BOX >> 4), db = dw0 + ws1 * (I8_BOX >> 4), dx = dx0 + xs * (XB >> 4);
+            const int left = (k_hi - k_lo - i * I8_BPS * I8_KB + 31) >> 5;  // steps of 32 channels
+            if (leader) {
+                if (left >= 8) {
+#pragma unroll
+                    for (uint32_t ks = 0; ks < 4; ++ks) tc_mma_i8(tmem, da + ks * WK, dx + ks * XK, idesc, (ks > 0 || i > 0) ? 1u : 0u);
+#pragma unroll
+                    for (uint32_t ks = 0; ks < 4; ++ks) tc_mma_i8(tmem, db + ks * WK, dx + (4 + ks) * XK, idesc, 1u);
+                } else {
+#pragma unroll 1
+                    for (int ks = 0; ks < left; ++ks) tc_mma_i8(tmem, (ks < 4 ? da : db) + (ks & 3) * WK, dx + ks * XK, idesc, (ks > 0 || i > 0) ? 1u : 0u);
+                }
+                tc_commit(&misc->wempty[ws]);
+                if (two) tc_commit(&misc->wempty[ws1]);
+                tc_commit(&misc->xempty[xs]);
+                if (refill > 0) box(asked, rs);
+                if (refill > 1) box(asked + 1, rs1);
+            }
+            if (refill > 0) next(rs, rpar);
+            if (refill > 1) next(rs, rpar);
+            asked += max(0, refill);
+            next(ws, wpar);
+            next(ws, wpar);
+            if (++xs == NX) { xs = 0; xpar ^= 1u; }
+        }
+        // all MMAs have finished, and no copy is under way, before anyone leaves
+        int own_abort = 0;
+        if (leader) tc_commit(&misc->done);
+        i8_wait(&misc->done, 0, 4, &own_abort, TC_SPIN, status);
+        if (*abort_flag)
+            for (int q = max(0, asked - NW); q < asked; ++q) i8_wait(&misc->wfull[q % NW], (uint32_t)(q / NW) & 1u, 5, &own_abort, TC_SPIN, status);
+    } else {
+        // ---- second pass: the digits
+        int blk = ub, rq = uq;
+        const uint32_t shifts = lane < BR ? (uint32_t)i8_shift(misc->top[lane]) : 0u;  // lane b: of row b
+        auto digits = [&](const float (&v)[4][4]) -> bool {
+            const int i = blk / I8_BPS;
+            const uint32_t xs = (uint32_t)i % NX;
+            if (i >= NX && !warp_wait(&misc->xempty[xs], ((uint32_t)(i / NX) & 1u) ^ 1u, 1)) return false;
+            unsigned char *dst = s_x + xs * XB + ((blk % I8_BPS) * (I8_KB / 16) + (lane >> 2)) * LBO + (lane & 3) * 4 + rq * 64;  // (rows of 16 bytes follow one another)
+#pragma unroll
+            for (int r = 0; r < 4; ++r) {
+                if (rq * 4 + r < B) {
+                    const float up = i8_pow2((int)__shfl_sync(0xffffffffu, shifts, rq * 4 + r));
+                    uint32_t q[4];  // four signed digits each
+#pragma unroll
+                    for (int e = 0; e < 4; ++e) q[e] = ((uint32_t)__float2int_rn((odd && i8_bits(v[r][e]) >= 0x7f800000u ? 0.0f : v[r][e]) * up) + 0x00808080u) ^ 0x00808080u;
+                    const uint32_t l01 = __byte_perm(q[0], q[1], 0x5140), h01 = __byte_perm(q[0], q[1], 0x7362);
+                    const uint32_t l23 = __byte_perm(q[2], q[3], 0x5140), h23 = __byte_perm(q[2], q[3], 0x7362);
+                    *reinterpret_cast<uint32_t *>(dst + (0 * BR + r) * 16) = __byte_perm(l01, l23, 0x5410);  // digit x BR + row: the lowest first
+                    *reinterpret_cast<uint32_t *>(dst + (1 * BR + r) * 16) = __byte_perm(l01, l23, 0x7632);
+                    *reinterpret_cast<uint32_t *>(dst + (2 * BR + r) * 16) = __byte_perm(h01, h23, 0x5410);
+                    *reinterpret_cast<uint32_t *>(dst + (3 * BR + r) * 16) = __byte_perm(h01, h23, 0x7632);
+                }
+            }
+            asm volatile("fence.proxy.async.shared::cta;" ::: "memory");  // generic-proxy writes -> visible to the tensor core
+            __syncwarp();
+            if (lane == 0) {
+                mbar_arrive(&misc->xfull[xs]);
+                if (blk + 1 == n && blk % I8_BPS == 0) mbar_arrive(&misc->xfull[xs]);  // the last stage has no second block
+            }
+            step(blk, rq);
+            return true;
+        };
+        bool ok = true;
+#pragma unroll
+        for (int j = 0; j < I8_KEEP; ++j) {
+            if (j + 1 == I8_KEEP) {  // the first unit that was not kept, asked for a unit ahead
+                int nb = blk, nq = rq;
+                step(nb, nq);
+                if (nb < n) load(raw, nb, nq);
+            }
+            if (ok && blk < n) ok = digits(keep[j]);
+        }
+        while (ok && blk < n) {
+            float v[4][4];
+#pragma unroll
+            for (int r = 0; r < 4; ++r) value(raw, r, v[r]);
+            int nb = blk, nq = rq;
+            step(nb, nq);
+            if (nb < n) load(raw, nb, nq);
+            ok = digits(v);
+        }
+    }
+    // ---- cluster exchange, push form: a column of the tile is a TMEM lane; every sum of the rank goes to the rank that finishes its
+    // column as a store that counts down its barrier
+    __syncwarp();
+    if (S > 1) cluster_wait();  // every rank's barrier is initialised (all ranks arrived before their streams)
+    if (warp >= 4 && warp < 8) {
+        const bool ok = warp_wait(&misc->done, 0, 4) && __all_sync(0xffffffffu, *abort_flag == 0);
+        tc_fence_after();
+        const int dc = (warp & 3) * 32 + lane, col = tile * I8_TN + dc;
+        const int r = (int)((uint32_t)dc * ia.per_inv >> 20), slot0 = s * BR * per + (dc - r * per);
+        const uint32_t dst0 = S > 1 ? cluster_addr(smem_addr(s_gather) + 4u * (uint32_t)slot0, (uint32_t)r) : 0u;
+        const uint32_t dbar = S > 1 ? cluster_addr(recv_bar, (uint32_t)r) : 0u;
+        const uint32_t lanes = tmem + ((uint32_t)((warp & 3) * 32) << 16);
+        constexpr int RL = BR < 8 ? BR : 8;
+        float *s_odd = reinterpret_cast<float *>(s_w) + dc;  // the ring is free: a thread's own column
+        if (odd) {
+#pragma unroll 1
+            for (int b = 0; b < B; ++b) s_odd[b * I8_TN] = (odd >> b & 1) && col < a.Nh ? i8_not_finite<MODE, XT>(&a, k_lo, k_hi, b, col) : 0.0f;
+        }
+#pragma unroll
+        for (int b0 = 0; b0 < BR; b0 += RL) {
+            uint32_t v[4][RL];
+            if (ok) {
+#pragma unroll
+                for (int d = 0; d < 4; ++d) tc_ldn(v[d], lanes + (uint32_t)(d * BR + b0));
+                asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+            }
+#pragma unroll
+            for (int e = 0; e < RL; ++e) {
+                const int b = b0 + e;
+                if (b < B) {
+                    float y = 0.0f;
+                    if (ok) {
+                        const float hi = fmaf((float)(int)v[3][e], 256.0f, (float)(int)v[2][e]), lo = fmaf((float)(int)v[1][e], 256.0f, (float)(int)v[0][e]);
+                        y = fmaf(hi, 65536.0f, lo) * i8_pow2(-i8_shift(misc->top[b]));
+                        if (odd) y += s_odd[b * I8_TN];
+                    }
+                    if (S > 1) st_async_f32(dst0 + 4u * (uint32_t)(b * per), y, dbar);
+                    else s_gather[slot0 + b * per] = y;
+                }
+            }
+        }
+    }
+    // the bias of this thread's first result, asked for ahead of the last wait
+    const int c0 = (int)((uint32_t)tid * ia.per_inv >> 20);  // batch row of result tid
+    const int mine = s * per + tid - c0 * per;               // its column in the tile
+    float bias = 0.0f;
+    if (tid < per * B && mine < I8_TN && tile * I8_TN + mine < a.Nh && a.bias) bias = __ldcg(a.bias + tile * I8_TN + mine);
+    tc_fence_before();
+    __syncthreads();
+    tc_fence_after();
+    if (warp == 0) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(TCOLS) : "memory");
+    if (warp * 32 >= per * B) return;
+    if (S > 1) {
+        bool landed = false;
+#pragma unroll 1
+        for (uint32_t it = 0; it < (1u << 22) && !landed; ++it) landed = mbarrier_try_wait(recv_bar, 0);
+        if (!landed && status) atomicCAS(status, 0, 6);  // never in a correct run; the result is then incomplete
+    }
+    // the S partials of a result in rank order, and the bias
+    for (int i = tid; i < per * B; i += I8_THREADS) {
+        const int b = (int)((uint32_t)i * ia.per_inv >> 20), c = s * per + i - b * per, col = tile * I8_TN + c;
+        if (c < I8_TN && col < a.Nh) {
+            float v = i == tid ? bias : a.bias ? __ldcg(a.bias + col) : 0.0f;
+#pragma unroll
+            for (int q = 0; q < MAX_CLUSTER; ++q)
+                if (q < S) v += s_gather[q * BR * per + i];
+            a.y[(size_t)b * a.y_ld + col] = v;
+        }
+    }
+}
+
+// ---- host side ------------------------------------------------------------------------------------------------
+
+// The codes as a 2-D tensor of bytes: boxes of 128 columns x 128 channels, 128-byte swizzle; rows and columns beyond the matrix read as
+// zeros.  The map covers this GPU's own W only, and every box goes to the one CTA that asked for it.
+static bool i8_tensor_map(CUtensorMap *map, const void *W, int K, int N) {
+    EncodeTiledFn fn = encode_tiled_fn();
+    if (!fn) return false;
+    const cuuint64_t dims[2] = {(cuuint64_t)N, (cuuint64_t)K};
+    const cuuint64_t strides[1] = {(cuuint64_t)N};
+    const cuuint32_t box[2] = {I8_TN, I8_KB};
+    const cuuint32_t estr[2] = {1, 1};
+    return fn(map, CU_TENSOR_MAP_DATA_TYPE_UINT8, 2, const_cast<void *>(W), dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
+              CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_128B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+}
+
+template <int BR, int MODE, typename XT>
+static cudaError_t launch_i8_b(const FcArgs &a, const CUtensorMap &map, cudaStream_t st) {
+    static SmemOptIn opt_in;
+    auto kern = fc_i8_kernel<BR, MODE, XT>;
+    cudaError_t e0 = ensure_dynamic_smem(kern, i8_smem(BR), opt_in);
+    if (e0 != cudaSuccess) return e0;
+    I8Args ia;
+    ia.f = a;
+    const int blocks = (a.K + I8_KB - 1) / I8_KB;
+    ia.blocks = blocks / a.S;
+    ia.extra = blocks % a.S;
+    ia.per = (I8_TN + a.S - 1) / a.S;
+    ia.per_inv = ((1u << 20) + ia.per - 1) / ia.per;
+    return launch_cluster(kern, dim3((a.ldw + I8_TN - 1) / I8_TN, a.S), dim3(I8_THREADS), i8_smem(BR), a.S, st, g_tune.pdl != 0, ia, map);
+}
+template <int MODE, typename XT>
+static cudaError_t launch_i8_x(const FcArgs &a, const CUtensorMap &map, cudaStream_t st) {
+    if (a.B <= 4) return launch_i8_b<4, MODE, XT>(a, map, st);
+    if (a.B <= 8) return launch_i8_b<8, MODE, XT>(a, map, st);
+    return launch_i8_b<16, MODE, XT>(a, map, st);
+}
+
+// Split-K factor: the most CTAs that are all resident (two per SM), at least one block per rank.
+static int i8_split(const FcArgs &a) {
+    const int tiles = (a.ldw + I8_TN - 1) / I8_TN, blocks = (a.K + I8_KB - 1) / I8_KB;
+    int best_S = 1;
+    long long best = -1;
+    for (int S = 1; S <= MAX_CLUSTER; ++S) {
+        if (g_tune.split_k > 0 && S > g_tune.split_k) continue;
+        const long long ctas = (long long)tiles * S;
+        if (S > blocks || (S > 1 && ctas > resident_ctas(S))) continue;
+        if (ctas >= best) { best = ctas; best_S = S; }
+    }
+    return best_S;
+}
+
+int i8_blocks_per_rank(const FcArgs &a) {
+    const int S = i8_split(a);
+    return ((a.K + I8_KB - 1) / I8_KB + S - 1) / S;
+}
+
+// Rows of x and of the codes must lie on 16-byte boundaries (vector loads, stride of the tensor map), and the 32-bit sums must hold a
+// rank's channels (2^14 per product).
+bool i8_applicable(const FcArgs &a) {
+    return a.K % 8 == 0 && a.ldw % 16 == 0 && a.B >= 1 && a.B <= 16 && !a.hold_dependents && aligned16(a.wscale) && i8_blocks_per_rank(a) <= 512;
+}
+
+cudaError_t launch_fc_i8(int mode, int xkind, FcArgs a, cudaStream_t st) {
+    CUtensorMap map;
+    if (!i8_tensor_map(&map, a.W, a.K, a.ldw)) return cudaErrorNotSupported;
+    a.S = i8_split(a);
+    a.status = tc_status_ptr();
+    a.spin = g_tune.tc_spin;
+    if (mode == MODE_DENSE) return xkind == 1 ? launch_i8_x<MODE_DENSE, __nv_bfloat16>(a, map, st) : launch_i8_x<MODE_DENSE, __half>(a, map, st);
+    return xkind == 1 ? launch_i8_x<MODE_GATHER, __nv_bfloat16>(a, map, st) : launch_i8_x<MODE_GATHER, __half>(a, map, st);
+}
+
+}  // namespace scap

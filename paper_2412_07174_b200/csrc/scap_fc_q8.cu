@@ -50,11 +50,18 @@ static cudaError_t launch_q8_t(const FcArgs &a, cudaStream_t st) {
     return launch_q8_pu<BT, MODE, XT, fc_pu(BT)>(a, st);
 }
 
-// Calls that take the tensor-core kernel (tune "dense_stream": 0 none, 2 all it can take).  From three rows on the FMA kernel
-// needs a second launch over the codes (figures in scap_fc_qm.cu).  Two launches over the kept rows only are the faster form for three
-// and four rows of a large layer that prune a lot, and the sparsity is not known here (11008 x 4096, us, FMA -> this one at
-// 50 / 80 / 85 / 90 / 95 %: three rows 21.7 / 16.8 / 15.1 / 13.9 / 12.7 -> 18.0, four rows 24.9 / 18.9 / 16.5 / 14.7 / 12.0 -> 18.1;
-// five rows 33.1 / 26.1 / 24.0 / 22.0 / 19.5 -> 23.7): a caller who knows sets "dense_stream" 0.
+// Calls that take the integer kernel (scap_fc_i8.cu; tune "dense_stream": 0 none, 2 all it can take): three and more rows, of a layer
+// that is long enough for its longer start.  us, half pruned, scap_fc_qm.cu -> integers: four blocks of 128 channels per rank (K = N =
+// 4096) three rows 9.3 -> 7.2, eight 10.5 -> 8.2, sixteen 17.2 -> 10.5; two blocks (2048 x 4096) 7.0 -> 6.3, 6.6 -> 7.2, 9.9 -> 8.6; one
+// (1024 x 4096) 5.9 -> 6.3, 4.7 -> 7.0, 6.3 -> 8.2.  With one and two rows the FMA kernel below reads the kept rows only (11008 x 4096,
+// one row 10.0 against 10.8, two rows 12.7 against 11.1 at 50 % but 9.5 at 80 %); at three it no longer wins at any sparsity (95 %: 12.7 against 11.4).
+static bool q8_in_integers(const FcArgs &a) {
+    if (g_tune.dense_stream == 0 || !i8_applicable(a)) return false;
+    return g_tune.dense_stream >= 2 || (a.B >= 3 && i8_blocks_per_rank(a) >= (a.B <= 4 ? 2 : 4));
+}
+
+// Calls that take the mma.sync kernel (scap_fc_qm.cu, same tune key): what is left of three and more rows - short layers, and K not a
+// multiple of eight - where the FMA kernel needs a second launch over the codes.
 // One and two rows: the FMA kernel reads the kept rows only, this one all of them, but its prologue is shorter.  It wins
 // whatever the sparsity only while a warp has a single block (K = N = 1024, one row: 2.7 us against 3.3 - 3.4, two rows 3.1 against
 // 3.9 - 4.2; at two blocks, K = 2048, N = 4096: 5.2 against 4.2 - 5.3).
@@ -70,6 +77,7 @@ static cudaError_t launch_q8(int mode, int xkind, FcArgs a, cudaStream_t st) {
     QmArgs qm;
     memset(&qm, 0, sizeof(qm));
     qm.f = a;
+    if (xkind != 2 && q8_in_integers(a)) return launch_fc_i8(mode, xkind, a, st);
     if (xkind != 2 && q8_on_tensor_cores(qm)) return launch_fc_qm(8, mode, xkind, qm, st);
     const size_t xsz = xkind == 2 ? 4 : 2;
     const unsigned char *x0 = static_cast<const unsigned char *>(a.x);

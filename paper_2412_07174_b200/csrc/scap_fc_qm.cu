@@ -12,6 +12,8 @@
 //   copy, convert, threshold, issue and promote - took 43 us for 8-bit 11008 x 4096 at one row: six different
 //   instruction streams on every scheduler and a dozen hand-overs per stage cost more than the tensor core saves.)
 //
+// (8-bit calls of three and more rows of a long layer take the integer kernel of scap_fc_i8.cu.)
+//
 // Why it is here: beyond two rows the fp32-FMA kernels run two rows per launch, so the codes cross the chip B / 2 times.
 // K = 11008, N = 4096, half of the entries pruned, weights from DRAM, FMA kernel -> this one, device us per call:
 //   8-bit            4 rows 24.6 -> 18.3   8 rows 48.0 -> 23.9   16 rows  94.6 -> 41.2

@@ -22,12 +22,12 @@
 // first and was no faster on this access pattern.)
 // Every wait on an mbarrier is bounded; a wait that runs out sets a device status word, the CTA stops issuing work,
 // still passes every cluster barrier and frees its TMEM.
-#include <cuda.h>
 #include <string.h>
 
 #include <atomic>
 
 #include "scap_ds.cuh"
+#include "scap_tc.cuh"
 
 namespace scap {
 
@@ -40,7 +40,6 @@ constexpr int TC_CAP = 1408;                        // most kept channels per fi
 constexpr int TC_PLANE_DATA = TC_CAP * 32;          // A-operand bytes: 16 per channel and 8-row group, two groups at full capacity
 constexpr int TC_PLANE = TC_PLANE_DATA + 2048;      // + slack for the rows of M that nobody uses
 constexpr int TC_PART_LD = TC_TN + 1;               // row pitch of the accumulator copy (conflict-free)
-constexpr uint32_t TC_SPIN = 1u << 20;              // polls before a wait gives up (tens of milliseconds); scap_tune("tc_spin") overrides
 __host__ __device__ constexpr int tc_pu(int ROWS) { return ROWS == 8 ? 6 : 3; }  // chunks per warp per fill, at most
 // 8-row groups of the A operand for B batch rows (parts stacked densely: row = part * B + b), and the chunks of 32
 // channels that fit in the A-operand region with that many groups
@@ -72,50 +71,9 @@ struct TcMisc {
     int rows[16];
 };
 
-__device__ __forceinline__ uint32_t smem_u32(const void *p) { return (uint32_t)__cvta_generic_to_shared(p); }
-
-__device__ __forceinline__ void mbar_init(unsigned long long *bar, int count) {
-    asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_u32(bar)), "r"(count) : "memory");
-}
-__device__ __forceinline__ void mbar_arrive(unsigned long long *bar) {
-    asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(bar)) : "memory");
-}
-__device__ __forceinline__ bool mbar_test(unsigned long long *bar, uint32_t parity) {
-    uint32_t ok;
-    asm volatile("{ .reg .pred p; mbarrier.test_wait.parity.shared::cta.b64 p, [%1], %2; selp.u32 %0, 1, 0, p; }"
-                 : "=r"(ok) : "r"(smem_u32(bar)), "r"(parity) : "memory");
-    return ok != 0;
-}
 // Bounded wait: false (and the status word set) when the phase did not complete within `limit` polls.
-__device__ __forceinline__ bool mbar_wait(unsigned long long *bar, uint32_t parity, int code, volatile int *abort_flag,
-                                          uint32_t limit) {
-    for (uint32_t i = 0; i < limit; ++i) {
-        if (mbar_test(bar, parity)) return true;
-        if (*abort_flag) return false;
-        if (i > 64) __nanosleep(32);
-    }
-    atomicCAS(&g_tc_status, 0, code);
-    *abort_flag = 1;
-    return false;
-}
-
-__device__ __forceinline__ void tc_mma(uint32_t d_tmem, uint64_t a_desc, uint64_t b_desc, uint32_t idesc, uint32_t accumulate) {
-    asm volatile(
-        "{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\t"
-        "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, {%5, %5, %5, %5}, p;\n\t}\n" ::"r"(d_tmem),
-        "l"(a_desc), "l"(b_desc), "r"(idesc), "r"(accumulate), "r"(0u)
-        : "memory");
-}
-__device__ __forceinline__ void tc_commit(unsigned long long *bar) {
-    asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(smem_u32(bar)) : "memory");
-}
-__device__ __forceinline__ void tc_fence_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
-__device__ __forceinline__ void tc_fence_after() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
-
-// Shared-memory matrix descriptor (start address, leading / stride byte offsets in 16-byte units, version 1, swizzle).
-__device__ __forceinline__ uint64_t tc_desc(uint32_t addr, uint32_t lbo, uint32_t sbo, uint32_t layout) {
-    return (uint64_t)((addr >> 4) & 0x3fffu) | ((uint64_t)((lbo >> 4) & 0x3fffu) << 16) |
-           ((uint64_t)((sbo >> 4) & 0x3fffu) << 32) | (1ull << 46) | ((uint64_t)layout << 61);
+__device__ __forceinline__ bool mbar_wait(unsigned long long *bar, uint32_t parity, int code, volatile int *abort_flag, uint32_t limit) {
+    return mbar_wait(bar, parity, code, abort_flag, limit, &g_tc_status);
 }
 
 template <bool BF16, int ROWS, int MODE, typename XT, int EPI>
@@ -498,24 +456,6 @@ struct DsMisc {
     int rows[16];
 };
 
-__device__ __forceinline__ void mbar_arrive_expect_tx(unsigned long long *bar, uint32_t bytes) {
-    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_u32(bar)), "r"(bytes) : "memory");
-}
-// One box of the tensor map (64 columns x 64 rows) to shared memory; completion counts bytes on `bar`.  The copy goes to this CTA only.
-__device__ __forceinline__ void tma_box_2d(uint32_t dst, const CUtensorMap *map, int x, int y, unsigned long long *bar) {
-    asm volatile("cp.async.bulk.tensor.2d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3}], [%4];" ::"r"(dst),
-                 "l"(map), "r"(x), "r"(y), "r"(smem_u32(bar))
-                 : "memory");
-}
-
-// 4 or 8 accumulator columns of this warp's 32 lanes (complete after tcgen05.wait::ld).
-__device__ __forceinline__ void tc_ldn(uint32_t (&v)[4], uint32_t addr) {
-    asm volatile("tcgen05.ld.sync.aligned.32x32b.x4.b32 {%0, %1, %2, %3}, [%4];" : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]) : "r"(addr));
-}
-__device__ __forceinline__ void tc_ldn(uint32_t (&v)[8], uint32_t addr) {
-    asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
-                 : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]), "=r"(v[7]) : "r"(addr));
-}
 // Parts of an activation.  fp16 rows of a grouped call (NACC = 2) take three parts of 4, 9 and 11 bits instead of two of 11: the
 // products with the leading part are 15 bits, so its accumulator has bits to spare and truncates next to nothing, and what the
 // others lose is small.  The gather, whose chains are shorter, is the measure: of 240 fp16 calls of 1024 .. 14336 channels the
@@ -1022,11 +962,7 @@ int tc_choose_split(int K, int Nh, int epi, int B, bool bf16) {
 
 
 // ---- dense-stream kernel: tensor map and launch ----------------------------------------------------------------
-typedef CUresult (*EncodeTiledFn)(CUtensorMap *, CUtensorMapDataType, cuuint32_t, void *, const cuuint64_t *, const cuuint64_t *,
-                                  const cuuint32_t *, const cuuint32_t *, CUtensorMapInterleave, CUtensorMapSwizzle,
-                                  CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
-
-static EncodeTiledFn encode_tiled_fn() {
+EncodeTiledFn encode_tiled_fn() {
     static std::atomic<EncodeTiledFn> cached{nullptr};
     EncodeTiledFn fn = cached.load(std::memory_order_acquire);
     if (fn) return fn;

@@ -20,4 +20,9 @@ int qm_blocks_per_warp(const QmArgs &a);
 // wbits: 8 or 4; xkind: 0 fp16, 1 bf16.  Chooses the split-K factor itself.
 cudaError_t launch_fc_qm(int wbits, int mode, int xkind, QmArgs a, cudaStream_t st);
 
+// 8-bit weights on the 5th-generation tensor cores in integers (scap_fc_i8.cu).
+bool i8_applicable(const FcArgs &a);
+int i8_blocks_per_rank(const FcArgs &a);  // blocks of 128 channels
+cudaError_t launch_fc_i8(int mode, int xkind, FcArgs a, cudaStream_t st);
+
 }  // namespace scap
