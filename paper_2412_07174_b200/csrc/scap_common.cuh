@@ -208,6 +208,13 @@ __device__ __forceinline__ uint4 ld_act16_if(const void *p, bool on, uint64_t po
     return v;
 }
 
+__device__ __forceinline__ uint4 ld_act16(const void *p, uint64_t pol) {
+    uint4 v;
+    asm volatile("ld.global.cg.L2::cache_hint.v4.u32 {%0,%1,%2,%3}, [%4], %5;"
+                 : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "l"(p), "l"(pol) : "memory");
+    return v;
+}
+
 // L2 eviction policies for loads that carry a cache hint.  keep: small data every column tile of a call reads again
 // (activations, modes); stream: weight rows, read once.
 __device__ __forceinline__ uint64_t l2_policy_keep() {

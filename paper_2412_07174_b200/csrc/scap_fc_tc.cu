@@ -424,6 +424,9 @@ __global__ void __launch_bounds__(FC_THREADS, 2) fc_tc_kernel(const FcArgs a) {
 // results in its own lane and sends them on without a pass through shared memory.  Us per call, back to back for 0.3 s, before -> now:
 // 14336 x 4096, 16 rows 27.3 - 29.3 -> 23.7; 11008 x 4096 dense, 8 rows 19.1 -> 17.6; 4096 x 4096 fp16, 5 rows 10.7 -> 10.2;
 // GELU block of MPT-7B, fp16, 8 rows 57 - 62 -> 48.5; 32 grouped rows of 11008 x 4096 33.3 -> 31.3.
+// The operand warps are bound by instruction issue: chunks inside the matrix are requested without a check per request, nothing is
+// checked per channel (beyond the matrix x and m are zero), the mask word is formed only where it is asked for, and what runs before
+// the first request has no division: 32 grouped rows 31.3 -> 28.2, 14336 x 4096 16 rows 23.7 -> 23.2, the GELU block 48.5 -> 48.2.
 // ------------------------------------------------------------------------------------------------
 // ROWS = 8 or 16: most batch rows of a call; 32: the rows of a grouped call (scap_grouped.cu), whose operand takes more of the
 // shared memory, so the ring is shorter.
@@ -530,19 +533,18 @@ __global__ void __launch_bounds__(FC_THREADS, 2) fc_ds_kernel(const FcArgs a, co
     // earlier work on the stream rewrites after the hint is rewritten there, and the loads proper - after the wait,
     // through L2 - see the final contents.  One line per thread and turn; every tile of the call asks for the same
     // lines, L2 merges them.
-    if (warp >= 2) {
-        const int t = tid - 64;
-        if (MODE == MODE_GATHER && a.m) {
-            for (int i = t; i < 2 * nq; i += FC_THREADS - 64) {
-                const int k = ((i >> 1) * S + s) * 64 + (i & 1) * 32;
-                if (k < K) prefetch_l2_keep(a.m + k);
-            }
+    // (No division and few instructions: this code runs on all warps of the SM at once and delays the first request of the activations.)
+    if (warp == 2 && MODE == MODE_GATHER && a.m) {
+        for (int i = lane; i < 2 * nq; i += 32) {
+            const int k = ((i >> 1) * S + s) * 64 + (i & 1) * 32;
+            if (k < K) prefetch_l2_keep(a.m + k);
         }
-        if (ROWS > 16 || !a.in_rows) {  // (with a row map the rows are not known yet)
-            constexpr int XL = (64 * (int)sizeof(XT) + 127) / 128;  // lines per row and block
-            for (int i = t; i < nq * B * XL; i += FC_THREADS - 64) {
-                const int l = i % XL, rb = i / XL, b = rb % B, q = rb / B;
-                const int k = (q * S + s) * 64 + l * (128 / (int)sizeof(XT));
+    }
+    if (warp >= 2 && (ROWS > 16 || !a.in_rows)) {  // (with a row map the rows are not known yet)
+        constexpr int XL = (64 * (int)sizeof(XT) + 127) / 128;  // lines per row and block
+        for (int b = warp - 2; b < B; b += FC_WARPS - 2) {
+            for (int i = lane; i < nq * XL; i += 32) {
+                const int k = ((i / XL) * S + s) * 64 + (i % XL) * (128 / (int)sizeof(XT));
                 if (k < K) prefetch_l2_keep(xg + (size_t)b * a.x_ld + k);
             }
         }
@@ -568,6 +570,9 @@ __global__ void __launch_bounds__(FC_THREADS, 2) fc_ds_kernel(const FcArgs a, co
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
     }
     float bias0[2], bias1[2];
+    tc_fence_before();
+    __syncthreads();  // barriers and TMEM address; before the wait, so that the operand warps do not have to meet anybody after it
+    tc_fence_after();
 
     griddep_wait();  // x, m, tau, the biases and the row maps may be outputs of the work just before this call
     griddep_launch_dependents();
@@ -579,11 +584,10 @@ __global__ void __launch_bounds__(FC_THREADS, 2) fc_ds_kernel(const FcArgs a, co
     if constexpr (MODE == MODE_GATHER) {
         if (warp >= 2) tau = ld_act(a.tau);
     }
-    prefetch_bias<BF16, EPI, TNT>(a, tile, s, per, bias0, bias1);
-    if (ROWS <= 16 && a.in_rows && tid < 16) misc->rows[tid] = __ldcg(a.in_rows + (tid < B ? tid : 0));
-    tc_fence_before();
-    __syncthreads();
-    tc_fence_after();
+    if (ROWS <= 16 && a.in_rows) {
+        if (tid < 16) misc->rows[tid] = __ldcg(a.in_rows + (tid < B ? tid : 0));
+        __syncthreads();
+    }
     const uint32_t tmem = misc->tmem_base;
     const uint32_t idesc = (1u << 4) | ((BF16 ? 1u : 0u) << 7) | ((BF16 ? 1u : 0u) << 10) | (1u << 15) | (0u << 16) |
                            ((uint32_t)(NCOLS >> 3) << 17) | ((uint32_t)(TNT >> 4) << 24);
@@ -611,27 +615,32 @@ __global__ void __launch_bounds__(FC_THREADS, 2) fc_ds_kernel(const FcArgs a, co
         }
         __syncwarp();
     } else if (warp == 1) {
-        // ---- MMA issuer: per stage four MMAs of 16 rows
-        if (lane == 0) {
-            for (int q = 0; q < nq; ++q) {
-                const uint32_t st = (uint32_t)q % NST, par = ((uint32_t)q / NST) & 1u;
-                if (!mbar_wait(&misc->afull[st], par, 2, abort_flag, spin)) break;
-                if (!mbar_wait(&misc->wfull[st], par, 2, abort_flag, spin)) break;
-                tc_fence_after();
+        // ---- MMA issuer: per stage four MMAs of 16 rows.  The whole warp runs the loop and one lane issues: descriptors and addresses
+        // then stay in uniform registers (inside `if (lane == 0)` an MMA takes several times as long to issue), and both
+        // operands are waited for at once, each by its own lanes.
+        const bool leader = lane == 0;  // (the one that commits again below, should a wait run out)
+        const uint64_t dw0 = tc_desc(smem_u32(s_w), DS_STAGE_W / 2, 1024, 2), dx0 = tc_desc(smem_u32(s_a), LBO, 128, 0);
+        uint32_t st = 0, par = 0;
+        bool ok = true;
+#pragma unroll 1
+        for (int q = 0; q < nq; ++q) {
+            ok = __all_sync(0xffffffffu, mbar_wait(lane == 0 ? &misc->afull[st] : &misc->wfull[st], par, 2, abort_flag, spin)) != 0;
+            if (!ok) break;
+            tc_fence_after();
+            const uint64_t dw = dw0 + st * (DS_STAGE_W >> 4), dx = dx0 + st * (ASTG >> 4);
+            const uint32_t acc = tmem + (uint32_t)(q & (NACC - 1)) * NCOLS;
+            if (leader) {
                 misc->issued = 1;
+                // NACC = 2: stages alternate between two accumulators.  The tensor core truncates where it adds to one, so half
+                // the chain is half the error (K = 14336 in eight ranks: 9.5e-7 -> 4.2e-7); plain calls keep to one,
+                // which is 1 % faster.
 #pragma unroll
-                for (uint32_t kb = 0; kb < 4; ++kb) {
-                    const uint64_t dw = tc_desc(smem_u32(s_w) + st * DS_STAGE_W + kb * 2048, DS_STAGE_W / 2, 1024, 2);
-                    const uint64_t dx = tc_desc(smem_u32(s_a) + st * ASTG + kb * BLK, LBO, 128, 0);
-                    // NACC = 2: stages alternate between two accumulators.  The tensor core truncates where it adds to one, so half
-                    // the chain is half the error (K = 14336 in eight ranks: 9.5e-7 -> 4.2e-7); plain calls keep to one,
-                    // which is 1 % faster.
-                    tc_mma(tmem + (uint32_t)(q & (NACC - 1)) * NCOLS, dw, dx, idesc, (q >= NACC || kb > 0) ? 1u : 0u);
-                }
+                for (uint32_t kb = 0; kb < 4; ++kb) tc_mma(acc, dw + kb * (2048 >> 4), dx + kb * (BLK >> 4), idesc, (q >= NACC || kb > 0) ? 1u : 0u);
                 tc_commit(&misc->empty[st]);
             }
-            if (nq > 0 && !*abort_flag) tc_commit(&misc->done);
+            if (++st == NST) { st = 0; par ^= 1u; }
         }
+        if (leader && nq > 0 && ok) tc_commit(&misc->done);
         __syncwarp();
     } else {
         // ---- activations: chunk jc = stage 2 q + half h; element (row r = part * ROWS + b, position pos of the stage): block
@@ -652,46 +661,51 @@ __global__ void __launch_bounds__(FC_THREADS, 2) fc_ds_kernel(const FcArgs a, co
                 const int c = 2 * (q * S + s) + h;  // global 32-channel chunk
                 const int k0 = c * 32 + ch0;        // this lane's first channel
                 float xv[CPL], mv[CPL];
-                if (vec_ok) {
-                    uint4 raw[XV];
+                const bool modes = MODE == MODE_GATHER && a.m != nullptr;
+                const unsigned char *xp = reinterpret_cast<const unsigned char *>(xg + (size_t)xrow * a.x_ld + k0);
+                if (vec_ok && K % 4 == 0) {
+                    uint4 raw[XV], r4[CPL / 4];
+                    if (c * 32 + 32 <= K) {  // the whole chunk is inside the matrix: no check per request
 #pragma unroll
-                    for (int v = 0; v < XV; ++v) {
-                        const int kk = k0 + v * (16 / (int)sizeof(XT));
-                        raw[v] = ld_act16_if(reinterpret_cast<const unsigned char *>(xg + (size_t)xrow * a.x_ld + kk), b < B && kk < K, pol_keep);
+                        for (int v = 0; v < XV; ++v) raw[v] = ld_act16(xp + 16 * v, pol_keep);
+#pragma unroll
+                        for (int v = 0; v < CPL / 4; ++v) r4[v] = modes ? ld_act16(a.m + k0 + 4 * v, pol_keep) : make_uint4(0, 0, 0, 0);
+                    } else {
+#pragma unroll
+                        for (int v = 0; v < XV; ++v) raw[v] = ld_act16_if(xp + 16 * v, k0 + v * (16 / (int)sizeof(XT)) < K, pol_keep);
+#pragma unroll
+                        for (int v = 0; v < CPL / 4; ++v) r4[v] = ld_act16_if(a.m + k0 + 4 * v, modes && k0 + 4 * v < K, pol_keep);
                     }
                     const XT *xe = reinterpret_cast<const XT *>(raw);
+                    const float *me = reinterpret_cast<const float *>(r4);
 #pragma unroll
-                    for (int i = 0; i < CPL; ++i) xv[i] = widen1(xe[i]);
+                    for (int i = 0; i < CPL; ++i) { xv[i] = widen1(xe[i]); mv[i] = me[i]; }
                 } else {
 #pragma unroll
-                    for (int i = 0; i < CPL; ++i) xv[i] = widen1(ld_act_if(xg + (size_t)xrow * a.x_ld + k0 + i, b < B && k0 + i < K));
-                }
-                if (K % 4 == 0) {
+                    for (int i = 0; i < CPL; ++i) xv[i] = widen1(ld_act_if(xg + (size_t)xrow * a.x_ld + k0 + i, k0 + i < K));
 #pragma unroll
-                    for (int v = 0; v < CPL / 4; ++v) {
-                        uint4 r4 = make_uint4(0, 0, 0, 0);
-                        if (MODE == MODE_GATHER && a.m) r4 = ld_act16_if(reinterpret_cast<const unsigned char *>(a.m + k0 + 4 * v), b < B && k0 + 4 * v < K, pol_keep);
-                        mv[4 * v] = __uint_as_float(r4.x); mv[4 * v + 1] = __uint_as_float(r4.y);
-                        mv[4 * v + 2] = __uint_as_float(r4.z); mv[4 * v + 3] = __uint_as_float(r4.w);
-                    }
-                } else {
-#pragma unroll
-                    for (int i = 0; i < CPL; ++i) mv[i] = (MODE == MODE_GATHER && a.m) ? ld_act_if(a.m + k0 + i, b < B && k0 + i < K) : 0.0f;
+                    for (int i = 0; i < CPL; ++i) mv[i] = ld_act_if(a.m + k0 + i, modes && k0 + i < K);
                 }
                 bool go = true;
                 if (lane == 0) go = mbar_wait(&misc->empty[st], (((uint32_t)q / NST) & 1u) ^ 1u, 1, abort_flag, spin);
                 go = __shfl_sync(0xffffffffu, go ? 1 : 0, 0) != 0;
                 if (!go) break;
-                uint32_t mine = 0;
+                // Beyond the matrix x and m are zero, so what is kept there does not matter; a row that the batch does not have
+                // repeats row 0, and its results are not used.
+                if (MODE == MODE_GATHER && a.bits && tile == 0) {  // the chunk's word of the union mask
+                    uint32_t mine = 0;
+#pragma unroll
+                    for (int i = 0; i < CPL; ++i) mine |= b < B && k0 + i < K && fabsf(__fsub_rn(xv[i], mv[i])) >= tau ? (1u << i) : 0u;
+                    const unsigned bal = __reduce_or_sync(0xffffffffu, mine << ch0);  // union over the rows, all 32 channels
+                    if (lane == 0 && c * 32 < K) a.bits[c] = bal;
+                }
                 unsigned short part[CPL][3];
 #pragma unroll
                 for (int i = 0; i < CPL; ++i) {
-                    const float dv = (MODE == MODE_GATHER && a.m) ? __fsub_rn(xv[i], mv[i]) : xv[i];
-                    const bool kept = b < B && k0 + i < K && (MODE == MODE_DENSE || fabsf(dv) >= tau);
-                    mine |= kept ? (1u << i) : 0u;
-                    ds_split<BF16, NACC>(kept ? dv : 0.0f, part[i]);
+                    const float dv = MODE == MODE_GATHER ? __fsub_rn(xv[i], mv[i]) : xv[i];  // (m == NULL: zeros)
+                    ds_split<BF16, NACC>(MODE == MODE_DENSE || fabsf(dv) >= tau ? dv : 0.0f, part[i]);
                 }
-                {  // (rows that the batch does not have: zeros)
+                {
 #pragma unroll
                     for (int v = 0; v < CPL / 8; ++v) {
                         const int pos = h * 32 + ch0 + 8 * v;   // first of eight consecutive positions: one K half of one block
@@ -708,8 +722,6 @@ __global__ void __launch_bounds__(FC_THREADS, 2) fc_ds_kernel(const FcArgs a, co
                         }
                     }
                 }
-                const unsigned bal = __reduce_or_sync(0xffffffffu, mine << ch0);   // union over the rows, all 32 channels
-                if (MODE == MODE_GATHER && a.bits && tile == 0 && lane == 0 && c * 32 < K) a.bits[c] = bal;
                 asm volatile("fence.proxy.async.shared::cta;" ::: "memory");  // generic-proxy writes -> visible to the tensor core
                 __syncwarp();
                 if (lane == 0) mbar_arrive(&misc->afull[st]);
@@ -726,30 +738,35 @@ __global__ void __launch_bounds__(FC_THREADS, 2) fc_ds_kernel(const FcArgs a, co
                 uint4 raw[XV];
                 float m[CPL];
             };
+            const bool vec = vec_ok && K % 4 == 0;
             auto load_piece = [&](Piece &pc, int jc, int u) {
-                const int k0 = (2 * ((jc >> 1) * S + s) + (jc & 1)) * 32 + u * CPL;
-                if (vec_ok) {
+                const int c0 = (2 * ((jc >> 1) * S + s) + (jc & 1)) * 32, k0 = c0 + u * CPL;
+                const unsigned char *xp = reinterpret_cast<const unsigned char *>(xg + (size_t)xrow * a.x_ld + k0);
+                if (vec && c0 + 32 <= K && a.m) {  // the whole chunk is inside the matrix: no check per request
 #pragma unroll
-                    for (int v = 0; v < XV; ++v) {
-                        const int kk = k0 + v * (16 / (int)sizeof(XT));
-                        pc.raw[v] = ld_act16_if(reinterpret_cast<const unsigned char *>(xg + (size_t)xrow * a.x_ld + kk), b < B && kk < K, pol_keep);
-                    }
-                } else {
-                    XT e[CPL];
-#pragma unroll
-                    for (int i = 0; i < CPL; ++i) e[i] = ld_act_if(xg + (size_t)xrow * a.x_ld + k0 + i, b < B && k0 + i < K);
-                    memcpy(pc.raw, e, sizeof(e));
-                }
-                if (K % 4 == 0) {
+                    for (int v = 0; v < XV; ++v) pc.raw[v] = ld_act16(xp + 16 * v, pol_keep);
 #pragma unroll
                     for (int v = 0; v < CPL / 4; ++v) {
-                        const uint4 r4 = ld_act16_if(reinterpret_cast<const unsigned char *>(a.m + k0 + 4 * v), a.m != nullptr && b < B && k0 + 4 * v < K, pol_keep);
+                        const uint4 r4 = ld_act16(a.m + k0 + 4 * v, pol_keep);
+                        pc.m[4 * v] = __uint_as_float(r4.x); pc.m[4 * v + 1] = __uint_as_float(r4.y);
+                        pc.m[4 * v + 2] = __uint_as_float(r4.z); pc.m[4 * v + 3] = __uint_as_float(r4.w);
+                    }
+                } else if (vec) {
+#pragma unroll
+                    for (int v = 0; v < XV; ++v) pc.raw[v] = ld_act16_if(xp + 16 * v, k0 + v * (16 / (int)sizeof(XT)) < K, pol_keep);
+#pragma unroll
+                    for (int v = 0; v < CPL / 4; ++v) {
+                        const uint4 r4 = ld_act16_if(a.m + k0 + 4 * v, a.m != nullptr && k0 + 4 * v < K, pol_keep);
                         pc.m[4 * v] = __uint_as_float(r4.x); pc.m[4 * v + 1] = __uint_as_float(r4.y);
                         pc.m[4 * v + 2] = __uint_as_float(r4.z); pc.m[4 * v + 3] = __uint_as_float(r4.w);
                     }
                 } else {
+                    XT e[CPL];
 #pragma unroll
-                    for (int i = 0; i < CPL; ++i) pc.m[i] = a.m ? ld_act_if(a.m + k0 + i, b < B && k0 + i < K) : 0.0f;
+                    for (int i = 0; i < CPL; ++i) e[i] = ld_act_if(xg + (size_t)xrow * a.x_ld + k0 + i, k0 + i < K);
+                    memcpy(pc.raw, e, sizeof(e));
+#pragma unroll
+                    for (int i = 0; i < CPL; ++i) pc.m[i] = ld_act_if(a.m + k0 + i, a.m != nullptr && k0 + i < K);
                 }
             };
             Piece cur, next;
@@ -758,7 +775,6 @@ __global__ void __launch_bounds__(FC_THREADS, 2) fc_ds_kernel(const FcArgs a, co
             for (int jc = pw, u = 0; jc < 2 * nq;) {
                 const int q = jc >> 1, h = jc & 1;
                 const uint32_t st = (uint32_t)q % NST;
-                const int c = 2 * (q * S + s) + h;  // global 32-channel chunk
                 const int nu = u + 1 == SUB ? 0 : u + 1, nj = u + 1 == SUB ? jc + FC_WARPS - 2 : jc;
                 cur = next;  // asked for a piece ahead: a request takes 1 - 2 us under the weight stream
                 if (nj < 2 * nq) load_piece(next, nj, nu);
@@ -768,15 +784,14 @@ __global__ void __launch_bounds__(FC_THREADS, 2) fc_ds_kernel(const FcArgs a, co
                     go = __shfl_sync(0xffffffffu, go ? 1 : 0, 0) != 0;
                     if (!go) break;
                 }
-                const int chu = u * CPL, k0 = c * 32 + chu;  // this lane's first channel of the piece
+                const int chu = u * CPL;  // first channel of the piece in its chunk
                 const XT *xe = reinterpret_cast<const XT *>(cur.raw);
                 unsigned short part[CPL][3];
 #pragma unroll
                 for (int i = 0; i < CPL; ++i) {
                     const float xv = widen1(xe[i]);
                     const float dv = __fsub_rn(xv, cur.m[i]);  // (m == NULL: zeros)
-                    const bool kept = b < B && k0 + i < K && fabsf(dv) >= tau;
-                    ds_split<BF16, NACC>(kept ? dv : 0.0f, part[i]);
+                    ds_split<BF16, NACC>(fabsf(dv) >= tau ? dv : 0.0f, part[i]);  // (beyond the matrix x and m are zero)
                 }
                 {
 #pragma unroll
@@ -805,6 +820,9 @@ __global__ void __launch_bounds__(FC_THREADS, 2) fc_ds_kernel(const FcArgs a, co
             }
         }
     }
+    // The bias of the columns this rank finishes, asked for here: a thread waits for its request (the value is used on the spot), which
+    // ahead of the stream would hold up the first activations by a microsecond.
+    prefetch_bias<BF16, EPI, TNT>(a, tile, s, per, bias0, bias1);
     // ---- all threads: wait until the last MMA has finished
     if (nq > 0) mbar_wait(&misc->done, 0, 3, abort_flag, spin);
     tc_fence_before();
