@@ -31,7 +31,7 @@ __host__ __device__ constexpr int fc_min_blocks(int BT) { return 2; }
 __host__ __device__ constexpr int fc_pu(int BT) { return BT <= 2 ? 8 : BT <= 4 ? 6 : BT <= 8 ? 2 : 1; }
 __host__ __device__ constexpr int fc_cap(int BT) { return FC_WARPS * fc_pu(BT) * 32; }  // channels staged per fill
 __host__ __device__ constexpr int fc_rb(int BT) { return BT < 4 ? BT : 4; }              // batch rows per cross-warp round
-__host__ __device__ constexpr int fc_unroll(int BT) { return BT <= 1 ? 16 : BT <= 4 ? 8 : 4; }  // row loads in flight per thread
+__host__ __device__ constexpr int fc_unroll(int BT) { return BT <= 1 ? 16 : BT == 3 ? 10 : BT <= 4 ? 8 : 4; }  // row loads in flight per thread
 
 __host__ __device__ constexpr int fc_main_bytes(int BT) {
     const int stage = fc_cap(BT) * 4 * (1 + BT);
@@ -1026,7 +1026,11 @@ __global__ void __launch_bounds__(FC_THREADS, fc_min_blocks(BT)) fc_kernel(const
 
 inline int batch_tile(int B) { return B <= 1 ? 1 : B <= 2 ? 2 : B <= 8 ? 8 : 16; }  // 3..16 rows: tensor-core variants
 // Batch tile of the plain FC and FFN calls: batches up to the tuned limit stay on the fp32-FMA body.
-inline int fc_batch_tile(int B) { return (B > 2 && B <= g_tune.fma_rows) ? 4 : batch_tile(B); }
+// (Three rows are their own tile: as four they paid for a row of zeros in every multiply and in the staging, and had registers
+// for eight loads in flight instead of ten.  Three rows, us, as four -> as three: 2560 x 10576 at 30 % x 4 layers 55.7 -> 52.0,
+// 11008 x 4096 at 60 % x 4 70.7 -> 65.8, 4096 x 4096 fp16 at 90 % x 4 26.9 -> 24.1, dense 4096 x 11008 x 2 37.2 -> 35.6, SwiGLU
+// 4096 / 11008 x 2 96.7 -> 91.0.)
+inline int fc_batch_tile(int B) { return (B > 2 && B <= g_tune.fma_rows) ? B : batch_tile(B); }
 inline int fc_tiles(int Nh, int epi, int tn) { return epi == EPI_GLU ? (Nh + tn / 2 - 1) / (tn / 2) : (Nh + tn - 1) / tn; }
 
 // Tile width (256 or 128 columns) and split-K factor (cluster size) for an FC with Nh columns per half and
