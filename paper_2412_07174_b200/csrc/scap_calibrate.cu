@@ -1,8 +1,11 @@
 // Offline calibration (Section 3; Eq. 2): per-channel mode by histogram arg-max, then the pooled
-// quantile of |x - m| by a three-pass radix select on the binary32 bit pattern (non-negative floats
-// order like their unsigned bit patterns).  All value arithmetic uses the *_rn intrinsics so that no
+// quantile of |x - m| by a radix select on the binary32 bit pattern (non-negative floats order like their unsigned bit
+// patterns): 13 bits counted by the strip kernel, the other 18 by one more pass over the tensor.  All value arithmetic uses the *_rn intrinsics so that no
 // multiply-add is contracted and results are bit-reproducible.
 #include <math.h>
+
+#include <atomic>
+#include <type_traits>
 
 #include "scap_common.cuh"
 
@@ -11,11 +14,23 @@ namespace scap {
 constexpr int CW = 32;             // channels per CTA strip: 4 threads x 8 channels (16 B) per row
 constexpr int CAL_THREADS = 512;   // 128 rows per sweep
 constexpr int CAL_ROWS = CAL_THREADS / 4;
-constexpr int RADIX_BINS = 2048;   // 11 bits per pass; passes take bits 30..20, 19..9, 8..0
+// The threshold is an order statistic of the keys |x - m|, found digit by digit from the top.  Two forms:
+// in passes (radix_pass_kernel): bits 30..20, 19..9 and 8..0;
+constexpr int RADIX_BINS = 2048;
+// in one launch (tau_kernel): 13 bits (exponent and five bits of the significand), 10 bits, 8 bits.
+constexpr int RADIX_A = 8192, RADIX_B = 1024, RADIX_C = 256;
+constexpr int SHIFT_A = 18, SHIFT_B = 8;
+// The one launch reads the tensor once where the passes read it twice, but it is cooperative, so it starts only when the mode
+// kernel has left the chip, and its barrier and the 8192 counters that every CTA searches cost as much at every size.  Whole
+// call, us, passes -> one launch: 512 x 4096 24.6 -> 36.9, 2048 x 4096 38.2 -> 46.5, 700 x 14336 (10.0 million) 63.2 -> 62.8,
+// 2048 x 8192 72.4 -> 66.4, 2048 x 14336 115.1 -> 100.1.
+constexpr long long TAU_ONE_LAUNCH_FROM = 10ll << 20;  // elements
 
 struct SelState {
     uint32_t prefix[2];  // key bits decided so far for order statistics j and j+1
     uint32_t rank[2];    // rank of each within the keys that share its prefix
+    uint32_t arrived;    // CTAs of tau_kernel that have counted their middle digits
+    uint32_t finished;   // and their last ones
 };
 
 template <bool BF16>
@@ -50,10 +65,9 @@ __device__ __forceinline__ int load_rows(const uint16_t *xp, int K, int T, int t
 __device__ __forceinline__ uint4 rotate_channels(const uint4 &v, int r) {
     uint32_t w0 = v.x, w1 = v.y, w2 = v.z, w3 = v.w;
     {
-        const bool on = (r & 1) != 0;  // one channel = 16 bits
-        const uint32_t t0 = __funnelshift_r(w0, w1, 16), t1 = __funnelshift_r(w1, w2, 16);
-        const uint32_t t2 = __funnelshift_r(w2, w3, 16), t3 = __funnelshift_r(w3, w0, 16);
-        w0 = on ? t0 : w0; w1 = on ? t1 : w1; w2 = on ? t2 : w2; w3 = on ? t3 : w3;
+        const uint32_t sel = (r & 1) ? 0x5432u : 0x3210u;  // one channel = 16 bits
+        const uint32_t t0 = __byte_perm(w0, w1, sel), t1 = __byte_perm(w1, w2, sel), t2 = __byte_perm(w2, w3, sel), t3 = __byte_perm(w3, w0, sel);
+        w0 = t0; w1 = t1; w2 = t2; w3 = t3;
     }
     {
         const bool on = (r & 2) != 0;  // two channels = one word
@@ -69,8 +83,13 @@ __device__ __forceinline__ uint4 rotate_channels(const uint4 &v, int r) {
 }
 
 // One CTA per strip of CWT channels (32: 512 threads, one CTA per SM; 16: 256 threads, two CTAs per SM, finer
-// strips that spread better over the SMs): min/max, histogram, arg-max -> m; then the first radix histogram
-// (bits 30..20 of |x - m|) of the strip is added to hist_a.
+// strips that spread better over the SMs): min/max, histogram, arg-max -> m; then the histogram of the top digits
+// of |x - m| of the strip is added to hist_a.
+//
+// Bound by instruction issue (a strip is read once, into registers).  So the extremes are taken of two channels at a time in
+// the storage type, the channels are rotated by byte permutes and selects rather than one by one, and a counter's address is
+// one multiply-add on the biased bin number; a `red` to shared memory returns nothing.  512 x 4096: whole call 31.5 -> 24.3 us;
+// 2048 x 14336: this kernel 74 -> 66 us.
 //
 // Histogram layout: the two 16-bit counters of bins 2h and 2h+1 of channel c share word h * CW + c, so the bank of
 // a counter is its channel (CWT = 32; with 16 channels two bin pairs share a row of banks).  A warp holds 8 rows x 4
@@ -85,7 +104,7 @@ __device__ __forceinline__ uint4 rotate_channels(const uint4 &v, int r) {
 template <bool BF16, int CWT, int U>
 __global__ void __launch_bounds__(CWT * 16, CWT == 16 ? 2 : 1) mode_kernel(const uint16_t *__restrict__ x, int T, int K, int nbins,
                                                            float *__restrict__ m_out, uint32_t *__restrict__ hist_a,
-                                                           int want_hist, const float *__restrict__ m_given) {
+                                                           int want_hist, bool one_launch, const float *__restrict__ m_given) {
     griddep_wait();               // m_given and the cleared counters come from earlier work on the stream
     griddep_launch_dependents();  // the next pass may become resident early; it waits for this grid itself
     constexpr int QN = CWT / 8;        // 16-byte pieces per row of the strip
@@ -112,22 +131,34 @@ __global__ void __launch_bounds__(CWT * 16, CWT == 16 ? 2 : 1) mode_kernel(const
         __syncthreads();
     } else if (nbins > 0) {
         // ---- pass 1: per-channel min / max (thread -> 8 rows of the warp by shuffles -> warps through shared memory)
-        float lo[8], hi[8];
+        // (two channels per instruction in the storage type: the extremes of a channel are values of it)
+        using P2 = typename std::conditional<BF16, __nv_bfloat162, __half2>::type;
+        const uint32_t plus = BF16 ? 0x7f807f80u : 0x7c007c00u;  // +infinity, twice
+        uint32_t lo2[4], hi2[4];
 #pragma unroll
-        for (int j = 0; j < 8; ++j) { lo[j] = INFINITY; hi[j] = -INFINITY; }
+        for (int j = 0; j < 4; ++j) { lo2[j] = plus; hi2[j] = plus | 0x80008000u; }
         if (ok)
             for (int t0 = rl; t0 < T; t0 += CAL_ROWS * U) {
                 if (!resident) nv = load_rows(xp, K, T, t0, v);
 #pragma unroll
                 for (int u = 0; u < U; ++u) {
                     if (u < nv) {
-                        float f[8];
-                        widen8<BF16>(v[u], f);
+                        const uint32_t w[4] = {v[u].x, v[u].y, v[u].z, v[u].w};
 #pragma unroll
-                        for (int j = 0; j < 8; ++j) { lo[j] = fminf(lo[j], f[j]); hi[j] = fmaxf(hi[j], f[j]); }
+                        for (int j = 0; j < 4; ++j) {
+                            const P2 e = *reinterpret_cast<const P2 *>(&w[j]);
+                            *reinterpret_cast<P2 *>(&lo2[j]) = __hmin2(*reinterpret_cast<P2 *>(&lo2[j]), e);
+                            *reinterpret_cast<P2 *>(&hi2[j]) = __hmax2(*reinterpret_cast<P2 *>(&hi2[j]), e);
+                        }
                     }
                 }
             }
+        float lo[8], hi[8];
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+            widen2<BF16>(lo2[j], lo[2 * j], lo[2 * j + 1]);
+            widen2<BF16>(hi2[j], hi[2 * j], hi[2 * j + 1]);
+        }
 #pragma unroll
         for (int o = QN; o < 32; o <<= 1)
 #pragma unroll
@@ -156,13 +187,16 @@ __global__ void __launch_bounds__(CWT * 16, CWT == 16 ? 2 : 1) mode_kernel(const
         __syncthreads();
         // this lane's channels in rotated order: slot i holds channel q * 8 + (i + r) mod 8
         float scale[8];
-        int cidx[8];
+        uint32_t at[8];  // byte offset of the channel's counters, less what the biased bin number below contributes
+        const uint32_t smem0 = smem_addr(smem);
+        const uint32_t last = 0x4b000000u + (uint32_t)nbins - 1u;
 #pragma unroll
         for (int i = 0; i < 8; ++i) {
-            cidx[i] = q * 8 + ((i + r) & 7);
-            lo[i] = s_lo[cidx[i]];
-            hi[i] = s_hi[cidx[i]];
+            const int c = q * 8 + ((i + r) & 7);
+            lo[i] = s_lo[c];
+            hi[i] = s_hi[c];
             scale[i] = hi[i] != lo[i] ? __fdiv_rn((float)nbins, __fsub_rn(hi[i], lo[i])) : 0.0f;
+            at[i] = smem0 + (uint32_t)c * 4u - 0x4b000000u * (uint32_t)(CWT * 2);
         }
         if (ok)
             for (int t0 = rl; t0 < T; t0 += CAL_ROWS * U) {
@@ -175,12 +209,13 @@ __global__ void __launch_bounds__(CWT * 16, CWT == 16 ? 2 : 1) mode_kernel(const
 #pragma unroll
                         for (int i = 0; i < 8; ++i) {
                             // floor of the non-negative product without a conversion instruction: adding 2^23
-                            // rounding down leaves floor(v) in the mantissa (exact for 0 <= v < 2^23).  A constant
-                            // channel has scale 0 and counts into bin 0; its mode is set from lo below.
+                            // rounding down leaves 0x4b000000 + floor(v) as the pattern (exact for 0 <= v < 2^23).  A
+                            // constant channel has scale 0 and counts into bin 0; its mode is set from lo below.  The two
+                            // bins of a word are CWT words apart from the next two: (b & ~1) * 2 CWT bytes.
                             const float vb = __fmul_rn(__fsub_rn(f[i], lo[i]), scale[i]);
-                            int b = __float_as_int(__fadd_rd(vb, 8388608.0f)) & 0x7fffff;
-                            b = min(b, nbins - 1);
-                            atomicAdd(&smem[(b >> 1) * CWT + cidx[i]], 1u << ((b & 1) * 16));
+                            const uint32_t b = min(__float_as_uint(__fadd_rd(vb, 8388608.0f)), last);  // (NaN: the last bin)
+                            const uint32_t word = (b & ~1u) * (uint32_t)(CWT * 2) + at[i];
+                            asm volatile("red.shared.add.u32 [%0], %1;" ::"r"(word), "r"((b & 1u) * 0xffffu + 1u) : "memory");
                         }
                     }
                 }
@@ -244,63 +279,76 @@ __global__ void __launch_bounds__(CWT * 16, CWT == 16 ? 2 : 1) mode_kernel(const
         __syncthreads();
     }
     if (!want_hist) return;
-    // ---- pass 3: first radix histogram of the importance |x - m|.  The keys crowd into a few dozen buckets (the
-    // top 11 bits are the exponent and three mantissa bits), so groups of four neighbouring lanes count into four
-    // copies of the histogram, each shifted by 8 banks against the previous one.
-    for (int i = tid; i < 4 * RADIX_BINS; i += NTH) smem[i] = 0;
+    // ---- pass 3: top digits of the importance |x - m|.  The keys crowd into a few dozen buckets of 11 bits (the exponent and
+    // three bits of the significand), so groups of four neighbouring lanes count into four copies of the histogram, each
+    // shifted by 8 banks against the previous one; 13 bits spread the keys over four times as many counters, in one copy.
+    constexpr uint32_t COPY = RADIX_BINS + 8;
+    for (int i = tid; i < (one_launch ? RADIX_A : 4 * (int)COPY); i += NTH) smem[i] = 0;
     float mk[8];
 #pragma unroll
     for (int j = 0; j < 8; ++j) mk[j] = s_m[q * 8 + j];
+    const uint32_t smem0 = smem_addr(smem) + (one_launch ? 0u : (lane & 3) * (COPY * 4));
     __syncthreads();
-    const int cp = lane & 3;  // copy of this lane
-    uint32_t *hq = smem + cp * RADIX_BINS;
-    if (ok)
-        for (int t0 = rl; t0 < T; t0 += CAL_ROWS * U) {
-            if (!resident) nv = load_rows(xp, K, T, t0, v);
+    auto count = [&](auto nb_tag) {
+        constexpr int NB = decltype(nb_tag)::value, COPIES = NB == RADIX_A ? 1 : 4, SHIFT = NB == RADIX_A ? SHIFT_A : 20;
+        if (ok)
+            for (int t0 = rl; t0 < T; t0 += CAL_ROWS * U) {
+                if (!resident) nv = load_rows(xp, K, T, t0, v);
 #pragma unroll
-            for (int u = 0; u < U; ++u) {
-                if (u < nv) {
-                    float f[8];
-                    widen8<BF16>(v[u], f);
+                for (int u = 0; u < U; ++u) {
+                    if (u < nv) {
+                        float f[8];
+                        widen8<BF16>(v[u], f);
 #pragma unroll
-                    for (int j = 0; j < 8; ++j) {
-                        const uint32_t key = __float_as_uint(__fsub_rn(f[j], mk[j])) & 0x7fffffffu;
-                        atomicAdd(&hq[((key >> 20) + 8 * cp) & (RADIX_BINS - 1)], 1u);
+                        for (int j = 0; j < 8; ++j) {
+                            const uint32_t bits = __float_as_uint(__fsub_rn(f[j], mk[j]));
+                            asm volatile("red.shared.add.u32 [%0], 1;" ::"r"(smem0 + ((bits >> (SHIFT - 2)) & (4u * (NB - 1)))) : "memory");
+                        }
                     }
                 }
             }
-        }
-    __syncthreads();
-    for (int i = tid; i < RADIX_BINS; i += NTH) {
-        uint32_t c = 0;
+        __syncthreads();
+        for (int i = tid; i < NB; i += NTH) {
+            uint32_t c = 0;
 #pragma unroll
-        for (int qq = 0; qq < 4; ++qq) c += smem[qq * RADIX_BINS + ((i + 8 * qq) & (RADIX_BINS - 1))];
-        if (c) atomicAdd(&hist_a[i], c);
-    }
+            for (int cp = 0; cp < COPIES; ++cp) c += smem[cp * COPY + i];
+            if (c) atomicAdd(&hist_a[i], c);
+        }
+    };
+    if (one_launch) count(std::integral_constant<int, RADIX_A>{});
+    else count(std::integral_constant<int, RADIX_BINS>{});
 }
 
-// Block-wide bucket search (256 threads): for the order statistics w = 0, 1, finds in the nb counters h[w] (nb a
-// multiple of 256, at most 2048) the bucket that holds rank[w] (0-based among the counted keys) and rebases the rank
-// to that bucket.  Every thread returns both results.  Thread t adds its nb / 256 consecutive counters, the block
-// scans the 256 sums, and the one thread whose stretch contains the rank walks its own counters.
+// Block-wide bucket search (256 threads): for the order statistics w = 0, 1, finds in the NB counters h[w] (which may be the same)
+// the bucket that holds rank[w] (0-based among the counted keys) and rebases the rank to that bucket.  Every thread returns both results.
+// Thread t adds its NB / 256 consecutive counters, the block scans the 256 sums, and the one thread whose stretch contains
+// the rank walks its own counters.
 struct SelPick {
     uint32_t bucket[2], rank[2];
 };
-__device__ __forceinline__ SelPick block_select(const uint32_t *const (&h)[2], int nb, const uint32_t (&rank)[2]) {
+template <int NB, bool ONE>  // ONE: both order statistics look into h[0]
+__device__ __forceinline__ SelPick block_select(const uint32_t *const (&h)[2], const uint32_t (&rank)[2]) {
+    constexpr int PER = NB / 256, NH = ONE ? 1 : 2;
     __shared__ uint32_t s_wsum[2][8];
     __shared__ uint32_t s_pick[2][2];
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const int per = nb >> 8;  // 1 .. 8
-    uint32_t cnt[2][8], incl[2];
+    uint32_t cnt[NH][PER], incl[NH], sum[NH];
 #pragma unroll
-    for (int w = 0; w < 2; ++w) {
-        uint32_t sum = 0;
+    for (int w = 0; w < NH; ++w) {
+        if constexpr (PER >= 4) {
 #pragma unroll
-        for (int i = 0; i < 8; ++i) {
-            cnt[w][i] = i < per ? __ldcg(h[w] + tid * per + i) : 0u;
-            sum += cnt[w][i];
+            for (int i = 0; i < PER / 4; ++i) {
+                const uint4 c = __ldcg(reinterpret_cast<const uint4 *>(h[w]) + tid * (PER / 4) + i);
+                cnt[w][4 * i] = c.x; cnt[w][4 * i + 1] = c.y; cnt[w][4 * i + 2] = c.z; cnt[w][4 * i + 3] = c.w;
+            }
+        } else {
+#pragma unroll
+            for (int i = 0; i < PER; ++i) cnt[w][i] = __ldcg(h[w] + tid * PER + i);
         }
-        uint32_t v = sum;
+        sum[w] = 0;
+#pragma unroll
+        for (int i = 0; i < PER; ++i) sum[w] += cnt[w][i];
+        uint32_t v = sum[w];
 #pragma unroll
         for (int o = 1; o < 32; o <<= 1) {
             const uint32_t t = __shfl_up_sync(0xffffffffu, v, o);
@@ -312,21 +360,19 @@ __device__ __forceinline__ SelPick block_select(const uint32_t *const (&h)[2], i
     __syncthreads();
 #pragma unroll
     for (int w = 0; w < 2; ++w) {
+        const int hw = ONE ? 0 : w;
         uint32_t before = 0;
 #pragma unroll
-        for (int q = 0; q < 8; ++q) before += q < warp ? s_wsum[w][q] : 0u;
-        uint32_t sum = 0;
+        for (int q = 0; q < 8; ++q) before += q < warp ? s_wsum[hw][q] : 0u;
+        uint32_t lo = before + incl[hw] - sum[hw];  // keys in the buckets before this thread's stretch
+        if (rank[w] >= lo && rank[w] < lo + sum[hw]) {
 #pragma unroll
-        for (int i = 0; i < 8; ++i) sum += cnt[w][i];
-        uint32_t lo = before + incl[w] - sum;  // keys in the buckets before this thread's stretch
-        if (rank[w] >= lo && rank[w] < lo + sum) {
-#pragma unroll
-            for (int i = 0; i < 8; ++i) {
-                if (rank[w] >= lo && rank[w] < lo + cnt[w][i]) {
-                    s_pick[w][0] = (uint32_t)(tid * per + i);
+            for (int i = 0; i < PER; ++i) {
+                if (rank[w] >= lo && rank[w] < lo + cnt[hw][i]) {
+                    s_pick[w][0] = (uint32_t)(tid * PER + i);
                     s_pick[w][1] = rank[w] - lo;
                 }
-                lo += cnt[w][i];
+                lo += cnt[hw][i];
             }
         }
     }
@@ -334,6 +380,7 @@ __device__ __forceinline__ SelPick block_select(const uint32_t *const (&h)[2], i
     SelPick r;
     r.bucket[0] = s_pick[0][0]; r.rank[0] = s_pick[0][1];
     r.bucket[1] = s_pick[1][0]; r.rank[1] = s_pick[1][1];
+    __syncthreads();  // (the words are used again by the next search)
     return r;
 }
 
@@ -361,7 +408,7 @@ __global__ void __launch_bounds__(256) radix_pass_kernel(const uint16_t *__restr
     // previous pass: one shared histogram (the first pass) or one per order statistic
     const uint32_t *const ph[2] = {prev_hist, prev_two ? prev_hist + RADIX_BINS : prev_hist};
     const uint32_t rk[2] = {st_in ? st_in->rank[0] : j, st_in ? st_in->rank[1] : j1};
-    const SelPick pick = block_select(ph, RADIX_BINS, rk);
+    const SelPick pick = block_select<RADIX_BINS, false>(ph, rk);
     const uint32_t p0 = ((st_in ? st_in->prefix[0] : 0u) << prev_width) | pick.bucket[0];
     const uint32_t p1 = ((st_in ? st_in->prefix[1] : 0u) << prev_width) | pick.bucket[1];
     if (blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x == 0) {
@@ -376,7 +423,7 @@ __global__ void __launch_bounds__(256) radix_pass_kernel(const uint16_t *__restr
 #pragma unroll
     for (int jj = 0; jj < 8; ++jj) mk[jj] = 0.0f;
     if (kc < K) {
-        const float4 ma = __ldg(reinterpret_cast<const float4 *>(m + kc)), mb = __ldg(reinterpret_cast<const float4 *>(m + kc + 4));
+        const float4 ma = __ldcg(reinterpret_cast<const float4 *>(m + kc)), mb = __ldcg(reinterpret_cast<const float4 *>(m + kc + 4));
         mk[0] = ma.x; mk[1] = ma.y; mk[2] = ma.z; mk[3] = ma.w;
         mk[4] = mb.x; mk[5] = mb.y; mk[6] = mb.z; mk[7] = mb.w;
     }
@@ -421,18 +468,185 @@ __global__ void __launch_bounds__(256) radix_pass_kernel(const uint16_t *__restr
 }
 
 // One CTA of 256 threads, after the last pass: finds the last `width` key bits of both order statistics in
-// hist[0] / hist[1] (nb counters each) and interpolates
+// hist[0] / hist[1] (512 counters each) and interpolates
 // tau = v_j + frac * (v_j1 - v_j) in binary64, each operation rounded once, then rounded to binary32.
-__global__ void __launch_bounds__(256) select_kernel(const uint32_t *__restrict__ hist, int nb, int width,
+__global__ void __launch_bounds__(256) select_kernel(const uint32_t *__restrict__ hist, int width,
                                                      const SelState *__restrict__ st_in, double frac,
                                                      float *__restrict__ tau_out) {
     griddep_wait();
     const uint32_t *const ph[2] = {hist, hist + RADIX_BINS};
     const uint32_t rk[2] = {st_in->rank[0], st_in->rank[1]};
-    const SelPick pick = block_select(ph, nb, rk);
+    const SelPick pick = block_select<512, false>(ph, rk);
     if (threadIdx.x == 0) {
         const double vj = (double)__uint_as_float((st_in->prefix[0] << width) | pick.bucket[0]);
         const double vj1 = (double)__uint_as_float((st_in->prefix[1] << width) | pick.bucket[1]);
+        const double t64 = __dadd_rn(vj, __dmul_rn(frac, __dsub_rn(vj1, vj)));
+        *tau_out = (float)t64;
+    }
+}
+
+// The threshold from the top digits: one pass over the tensor, in one cooperative launch.  Every CTA finds the buckets of the two
+// order statistics j and j + 1 itself (all get the same answer), reads its part of the tensor once and keeps the keys in those
+// buckets (1 - 2 % of them) in shared memory, with which it counts the middle digits.  When all CTAs have
+// counted (a barrier over the grid, whose CTAs are all resident), the last digits are counted from the lists alone, and the CTA
+// that finishes last interpolates tau = v_j + frac * (v_j1 - v_j) in binary64, each operation rounded once, then to binary32.
+// A warp one of whose lists would overflow (a tensor with few distinct values) does not use them: it reads its part again instead.
+//
+// A CTA owns a block of 256 channels (32 lanes x 8 channels: a warp reads 512 contiguous bytes of a row) and the rows blockIdx.y * 8 + warp,
+// stepping by 8 * gridDim.y; the modes of a thread's 8 channels stay in registers.  The pass is bound by instruction issue, so a key costs
+// six: widen, subtract, t = 2 key - 2 base (the sign bit shifted out), t < 2 << SHIFT_A, and a store and an addition under that
+// predicate - every thread has a list of its own, [entry][thread], so there is no counter to share and no vote.  (One list and
+// one counter per CTA: 56 us for the kernel; a list per warp, placed by votes: 51.)
+// 2048 x 14336: 37 us, where two passes and the selection took 70; whole call 126.0 -> 100.1.
+constexpr int TAU_U = 8;         // 16-byte loads in flight per thread
+constexpr int TAU_LIST = 24;     // keys per thread (24 KB, four CTAs per SM); a row adds at most eight
+template <bool BF16>
+__global__ void __launch_bounds__(256, 4) tau_kernel(const uint16_t *__restrict__ x, const float *__restrict__ m, int T, int K,
+                                                     const uint32_t *__restrict__ hist_a, uint32_t *__restrict__ hist_b, uint32_t *__restrict__ hist_c,
+                                                     SelState *__restrict__ state, uint32_t j, uint32_t j1, double frac, float *__restrict__ tau_out) {
+    __shared__ uint32_t s_h[2][RADIX_B];
+    __shared__ uint32_t s_list[TAU_LIST][256];
+    __shared__ uint32_t s_last;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    for (int i = tid; i < 2 * RADIX_B; i += 256) (&s_h[0][0])[i] = 0;
+    const uint32_t *const ha[2] = {hist_a, hist_a};
+    const uint32_t rank_a[2] = {j, j1};
+    const SelPick a = block_select<RADIX_A, true>(ha, rank_a);  // (its barriers publish the cleared counters)
+    const bool same = a.bucket[0] == a.bucket[1];
+    const uint32_t base0 = a.bucket[0] << SHIFT_A, base1 = a.bucket[1] << SHIFT_A;
+    // Every row of this warp: row(values of this lane less their modes, width of the buckets or 0 where the lane has no channel).
+    auto scan = [&](auto row) {
+        const int step = 8 * gridDim.y;
+        const uint64_t pol = l2_policy_keep();
+#pragma unroll 1
+        for (int c0 = blockIdx.x * 256; c0 < K; c0 += gridDim.x * 256) {
+            const int kc = c0 + lane * 8;
+            const bool in = kc < K;
+            const uint32_t span = in ? 2u << SHIFT_A : 0u;
+            float mk[8];
+#pragma unroll
+            for (int jj = 0; jj < 8; ++jj) mk[jj] = 0.0f;
+            if (in) {
+                const float4 ma = __ldcg(reinterpret_cast<const float4 *>(m + kc)), mb = __ldcg(reinterpret_cast<const float4 *>(m + kc + 4));
+                mk[0] = ma.x; mk[1] = ma.y; mk[2] = ma.z; mk[3] = ma.w;
+                mk[4] = mb.x; mk[5] = mb.y; mk[6] = mb.z; mk[7] = mb.w;
+            }
+            const uint16_t *xp = x + kc;
+#pragma unroll 1
+            for (int t0 = blockIdx.y * 8 + warp; t0 < T; t0 += step * TAU_U) {
+                uint4 v[TAU_U];
+#pragma unroll
+                for (int u = 0; u < TAU_U; ++u) {
+                    const int t = t0 + step * u;
+                    v[u] = make_uint4(0, 0, 0, 0);
+                    if (in && t < T) v[u] = ld_keep16(xp + (size_t)t * K, pol);
+                }
+#pragma unroll
+                for (int u = 0; u < TAU_U; ++u) {
+                    if (t0 + step * u < T) {
+                        float f[8];
+                        widen8<BF16>(v[u], f);
+#pragma unroll
+                        for (int jj = 0; jj < 8; ++jj) f[jj] = __fsub_rn(f[jj], mk[jj]);
+                        row(f, span);
+                    }
+                }
+            }
+        }
+    };
+    auto count_b = [&](uint32_t key) {
+        if (key - base0 < (1u << SHIFT_A)) atomicAdd(&s_h[0][(key >> SHIFT_B) & (RADIX_B - 1)], 1u);
+        else atomicAdd(&s_h[1][(key >> SHIFT_B) & (RADIX_B - 1)], 1u);  // (only where the buckets differ)
+    };
+    // The keys of the buckets once more from the tensor, for a warp whose lists overflowed.
+    auto again = [&](auto take) {
+        scan([&](const float (&f)[8], uint32_t span) {
+#pragma unroll
+            for (int jj = 0; jj < 8; ++jj) {
+                const uint32_t bits = __float_as_uint(f[jj]);
+                if (bits * 2u - base0 * 2u < span || bits * 2u - base1 * 2u < span) take(bits & 0x7fffffffu);
+            }
+        });
+    };
+    const uint32_t list = smem_addr(&s_list[0][tid]);
+    constexpr uint32_t NEXT = 256 * 4, FULL = (TAU_LIST - 8) * NEXT;
+    uint32_t end = 0;  // bytes behind the thread's last entry
+    bool over = false;
+    auto collect = [&](auto two_tag) {
+        scan([&](const float (&f)[8], uint32_t span) {
+            over |= end > FULL;
+            end = end > FULL ? 0u : end;  // (the lists are not used then)
+#pragma unroll
+            for (int jj = 0; jj < 8; ++jj) {
+                const uint32_t bits = __float_as_uint(f[jj]);
+                bool hit = bits * 2u - base0 * 2u < span;
+                if constexpr (decltype(two_tag)::value) hit |= bits * 2u - base1 * 2u < span;
+                asm volatile("{ .reg .pred q; setp.ne.u32 q, %3, 0; @q st.shared.u32 [%1], %2; @q add.u32 %0, %0, %4; }"
+                             : "+r"(end) : "r"(list + end), "r"(bits), "r"((uint32_t)hit), "n"(NEXT) : "memory");
+            }
+        });
+    };
+    if (same) collect(std::false_type{});
+    else collect(std::true_type{});
+    const bool listed = !__any_sync(0xffffffffu, over);
+    const uint32_t n = end / NEXT;
+    if (listed) {
+        for (uint32_t i = 0; i < n; ++i) count_b(s_list[i][tid] & 0x7fffffffu);
+    } else {
+        again(count_b);
+    }
+    __syncthreads();
+    for (int i = tid; i < RADIX_B; i += 256) {
+        const uint32_t c0 = s_h[0][i], c1 = same ? 0u : s_h[1][i];
+        if (c0) atomicAdd(&hist_b[i], c0);
+        if (c1) atomicAdd(&hist_b[RADIX_B + i], c1);
+    }
+    // ---- barrier over the grid: the middle digits are complete
+    const uint32_t ctas = gridDim.x * gridDim.y;
+    __threadfence();
+    __syncthreads();
+    if (tid == 0) {
+        atomicAdd(&state->arrived, 1u);
+        // (bounded like every wait; all CTAs are resident, so it ends as soon as the slowest has counted)
+        for (uint32_t it = 0; it < (1u << 24); ++it) {
+            uint32_t seen;
+            asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(seen) : "l"(&state->arrived) : "memory");
+            if (seen >= ctas) break;
+            if (it > 256) __nanosleep(64);
+        }
+    }
+    for (int i = tid; i < 2 * RADIX_C; i += 256) (&s_h[0][0])[i] = 0;
+    __syncthreads();
+    __threadfence();
+    const uint32_t *const hb[2] = {hist_b, same ? hist_b : hist_b + RADIX_B};
+    const SelPick b = block_select<RADIX_B, false>(hb, a.rank);
+    const uint32_t p0 = (a.bucket[0] << (SHIFT_A - SHIFT_B)) | b.bucket[0], p1 = (a.bucket[1] << (SHIFT_A - SHIFT_B)) | b.bucket[1];
+    auto count_c = [&](uint32_t key) {
+        if ((key >> SHIFT_B) == p0) atomicAdd(&s_h[0][key & (RADIX_C - 1)], 1u);
+        if ((key >> SHIFT_B) == p1) atomicAdd(&s_h[0][RADIX_C + (key & (RADIX_C - 1))], 1u);
+    };
+    if (listed) {
+        for (uint32_t i = 0; i < n; ++i) count_c(s_list[i][tid] & 0x7fffffffu);
+    } else {
+        again(count_c);
+    }
+    __syncthreads();
+    for (int i = tid; i < 2 * RADIX_C; i += 256) {
+        const uint32_t c = s_h[0][i];
+        if (c) atomicAdd(&hist_c[i], c);
+    }
+    // ---- the CTA that finishes last has all counts
+    __threadfence();
+    __syncthreads();
+    if (tid == 0) s_last = atomicAdd(&state->finished, 1u) == ctas - 1 ? 1u : 0u;
+    __syncthreads();
+    if (!s_last) return;
+    __threadfence();
+    const uint32_t *const hc[2] = {hist_c, hist_c + RADIX_C};
+    const SelPick c = block_select<RADIX_C, false>(hc, b.rank);
+    if (tid == 0) {
+        const double vj = (double)__uint_as_float((p0 << SHIFT_B) | c.bucket[0]);
+        const double vj1 = (double)__uint_as_float((p1 << SHIFT_B) | c.bucket[1]);
         const double t64 = __dadd_rn(vj, __dmul_rn(frac, __dsub_rn(vj1, vj)));
         *tau_out = (float)t64;
     }
@@ -864,12 +1078,13 @@ __global__ void init_pool_state_kernel(PoolState *st) {
 }
 
 struct CalLayout {
-    size_t hist, state, pool, pool_hist, zeroed, col_sum, total;  // hist: 3 passes x 2 x RADIX_BINS counters
+    size_t hist, state, pool, pool_hist, zeroed, col_sum, total;  // hist: the counters of the digits, 12288 in both forms at most
 };
 static CalLayout cal_layout(int K) {
     CalLayout L;
     L.hist = 0;
-    L.state = align_up(sizeof(uint32_t) * 3 * 2 * RADIX_BINS, 256);
+    L.state = sizeof(uint32_t) * 12288;
+    static_assert(RADIX_A + 2 * RADIX_B + 2 * RADIX_C <= 12288 && 6 * RADIX_BINS <= 12288, "the counters fit in their part of the workspace");
     L.pool = L.state + 256;                                   // PoolState
     L.pool_hist = L.pool + 256;                               // 2048 bins, then 256 + 512 key counters
     L.zeroed = L.pool_hist + sizeof(uint32_t) * (2048 + 768);  // everything before this is cleared per call
@@ -933,7 +1148,7 @@ static cudaError_t estimate_mode(const uint16_t *x, int T, int K, int estimator,
 
 template <bool BF16>
 static scap_status calibrate_t(const uint16_t *x, int T, int K, double sparsity, int estimator, bool scalar, int nbins,
-                               float *m_out, float *tau_out, unsigned char *ws, cudaStream_t st) {
+                               float *m_out, float *tau_out, unsigned char *ws, cudaStream_t st, bool may_cooperate = true) {
     const CalLayout L = cal_layout(K);
     uint32_t *hist = reinterpret_cast<uint32_t *>(ws + L.hist);
     SelState *state = reinterpret_cast<SelState *>(ws + L.state);
@@ -951,24 +1166,27 @@ static scap_status calibrate_t(const uint16_t *x, int T, int K, double sparsity,
     const int HW = (nbins + 1) / 2;
     const int cw = g_tune.cal_strip;  // 16 or 32 channels per CTA
     size_t smem = (size_t)cw * HW * 4;
-    if (smem < (size_t)4 * RADIX_BINS * 4) smem = (size_t)4 * RADIX_BINS * 4;  // the four copies of the first radix histogram
+    const size_t digits = (size_t)4 * (4 * RADIX_BINS + 32);  // four copies of 2048, 8 words apart; or one of 8192
+    static_assert(RADIX_A <= 4 * RADIX_BINS, "the top digits fit in the same words");
+    if (smem < digits) smem = digits;
+    const bool one_launch = want_tau && may_cooperate && M >= TAU_ONE_LAUNCH_FROM;
     static SmemOptIn opt_in32, opt_in16, opt_in16s;
     const float *given = own_mode ? (const float *)nullptr : (const float *)m_out;
     if (cw == 16 && T <= CAL_ROWS * 8) {
         e = ensure_dynamic_smem(mode_kernel<BF16, 16, 8>, 2048 / 2 * 16 * 4, opt_in16s);
         if (e != cudaSuccess) return cuda_status(e);
         e = launch(mode_kernel<BF16, 16, 8>, dim3((K + 15) / 16), dim3(256), smem, st, pdl, x, T, K, nbins, m_out, hist,
-                   want_tau ? 1 : 0, given);
+                   want_tau ? 1 : 0, one_launch, given);
     } else if (cw == 16) {
         e = ensure_dynamic_smem(mode_kernel<BF16, 16, CAL_U>, 2048 / 2 * 16 * 4, opt_in16);
         if (e != cudaSuccess) return cuda_status(e);
         e = launch(mode_kernel<BF16, 16, CAL_U>, dim3((K + 15) / 16), dim3(256), smem, st, pdl, x, T, K, nbins, m_out, hist,
-                   want_tau ? 1 : 0, given);
+                   want_tau ? 1 : 0, one_launch, given);
     } else {
         e = ensure_dynamic_smem(mode_kernel<BF16, 32, CAL_U>, 2048 / 2 * 32 * 4, opt_in32);
         if (e != cudaSuccess) return cuda_status(e);
         e = launch(mode_kernel<BF16, 32, CAL_U>, dim3((K + 31) / 32), dim3(512), smem, st, pdl, x, T, K, nbins, m_out, hist,
-                   want_tau ? 1 : 0, given);
+                   want_tau ? 1 : 0, one_launch, given);
     }
     if (e != cudaSuccess) return cuda_status(e);
     if (!want_tau) return cuda_status(launch(set_float_kernel, dim3(1), dim3(1), 0, st, false, tau_out, 0.0f));
@@ -978,22 +1196,51 @@ static scap_status calibrate_t(const uint16_t *x, int T, int K, double sparsity,
     if (j > M - 1) j = M - 1;
     const double frac = pos - (double)j;
     const long long j1 = j + 1 < M ? j + 1 : M - 1;
-    // radix passes: 256 channels per CTA column, enough row slabs for about four CTAs per SM
     const int gx = (K + 255) / 256;
-    int gy = (sm_count() * 4 + gx - 1) / gx;
+    if (!one_launch) {
+        // radix passes: 256 channels per CTA column, enough row slabs for about four CTAs per SM
+        int gy = (sm_count() * 4 + gx - 1) / gx;
+        if (gy > (T + 7) / 8) gy = (T + 7) / 8;
+        const dim3 grid(gx, gy < 1 ? 1 : gy);
+        // pass A (bits 30..20) was accumulated by mode_kernel; each later pass first extends the prefixes from the
+        // counters of the pass before it
+        e = launch(radix_pass_kernel<BF16>, grid, dim3(256), 0, st, pdl, x, (const float *)m_out, T, K, (const uint32_t *)hist, 0,
+                   11, (const SelState *)nullptr, (uint32_t)j, (uint32_t)j1, state, 9, 11, hist + 2 * RADIX_BINS);
+        if (e != cudaSuccess) return cuda_status(e);
+        e = launch(radix_pass_kernel<BF16>, grid, dim3(256), 0, st, pdl, x, (const float *)m_out, T, K,
+                   (const uint32_t *)(hist + 2 * RADIX_BINS), 1, 11, (const SelState *)state, 0u, 0u, state + 1, 0, 9,
+                   hist + 4 * RADIX_BINS);
+        if (e != cudaSuccess) return cuda_status(e);
+        e = launch(select_kernel, dim3(1), dim3(256), 0, st, pdl, (const uint32_t *)(hist + 4 * RADIX_BINS), 9,
+                   (const SelState *)(state + 1), frac, tau_out);
+        return cuda_status(e);
+    }
+    // 256 channels per CTA column, row slabs for as many CTAs as are resident at once (the kernel has a barrier over the grid)
+    static std::atomic<int> per_sm{0};
+    int resident = per_sm.load(std::memory_order_relaxed);
+    if (resident == 0) {
+        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&resident, tau_kernel<BF16>, 256, 0);
+        if (e != cudaSuccess) return cuda_status(e);
+        per_sm.store(resident, std::memory_order_relaxed);
+    }
+    const int ctas = sm_count() * (resident < 4 ? resident : 4);
+    int gy = ctas / gx;
     if (gy > (T + 7) / 8) gy = (T + 7) / 8;
-    const dim3 grid(gx, gy < 1 ? 1 : gy);
-    // pass A (bits 30..20) was accumulated by mode_kernel; each later pass first extends the prefixes from the
-    // counters of the pass before it
-    e = launch(radix_pass_kernel<BF16>, grid, dim3(256), 0, st, pdl, x, (const float *)m_out, T, K, (const uint32_t *)hist, 0,
-               11, (const SelState *)nullptr, (uint32_t)j, (uint32_t)j1, state, 9, 11, hist + 2 * RADIX_BINS);
-    if (e != cudaSuccess) return cuda_status(e);
-    e = launch(radix_pass_kernel<BF16>, grid, dim3(256), 0, st, pdl, x, (const float *)m_out, T, K,
-               (const uint32_t *)(hist + 2 * RADIX_BINS), 1, 11, (const SelState *)state, 0u, 0u, state + 1, 0, 9,
-               hist + 4 * RADIX_BINS);
-    if (e != cudaSuccess) return cuda_status(e);
-    e = launch(select_kernel, dim3(1), dim3(256), 0, st, pdl, (const uint32_t *)(hist + 4 * RADIX_BINS), 512, 9,
-               (const SelState *)(state + 1), frac, tau_out);
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(gx < ctas ? gx : ctas, gy < 1 ? 1 : gy);  // (a CTA column takes every gridDim.x-th block of channels)
+    cfg.blockDim = dim3(256);
+    cfg.stream = st;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeCooperative;
+    attr[0].val.cooperative = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    e = cudaLaunchKernelEx(&cfg, tau_kernel<BF16>, x, (const float *)m_out, T, K, (const uint32_t *)hist, hist + RADIX_A, hist + RADIX_A + 2 * RADIX_B,
+                           state, (uint32_t)j, (uint32_t)j1, frac, tau_out);
+    if (e == cudaErrorCooperativeLaunchTooLarge) {  // a context that was given fewer SMs than the device has: in passes, from the start
+        cudaGetLastError();
+        return calibrate_t<BF16>(x, T, K, sparsity, estimator, scalar, nbins, m_out, tau_out, ws, st, false);
+    }
     return cuda_status(e);
 }
 
