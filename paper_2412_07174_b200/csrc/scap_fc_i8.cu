@@ -21,7 +21,7 @@
 // those channels is then added one by one.
 //
 // What bounds it: K = 11008, N = 4096, half pruned, weights from DRAM, us per call, mma.sync kernel -> this one: 3 rows
-// 18.1 -> 11.4, 8 rows 24.0 -> 14.9, 16 rows 41.4 -> 20.3 (the 45 MB of codes take 6.9 at copy speed).  The first MMA starts 3 - 4 us
+// 18.1 -> 12.8, 8 rows 24.0 -> 14.9, 16 rows 41.4 -> 20.5 (the 45 MB of codes take 6.9 at copy speed).  The first MMA starts 3 - 4 us
 // into the call: activations through L2 (1 us under the weight stream), the pass for the exponents, the digits - code that all 24
 // warps of an SM run at once, bound by instruction issue - while the ring has been full for two of them; the rest of the codes then
 // comes at 5.9 TB/s.  Tried and slower: an exponent per block and an accumulator per block or two, so that the first MMA does not

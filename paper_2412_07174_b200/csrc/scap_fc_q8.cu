@@ -54,7 +54,8 @@ static cudaError_t launch_q8_t(const FcArgs &a, cudaStream_t st) {
 // that is long enough for its longer start.  us, half pruned, scap_fc_qm.cu -> integers: four blocks of 128 channels per rank (K = N =
 // 4096) three rows 9.3 -> 7.2, eight 10.5 -> 8.2, sixteen 17.2 -> 10.5; two blocks (2048 x 4096) 7.0 -> 6.3, 6.6 -> 7.2, 9.9 -> 8.6; one
 // (1024 x 4096) 5.9 -> 6.3, 4.7 -> 7.0, 6.3 -> 8.2.  With one and two rows the FMA kernel below reads the kept rows only (11008 x 4096,
-// one row 10.0 against 10.8, two rows 12.7 against 11.1 at 50 % but 9.5 at 80 %); at three it no longer wins at any sparsity (95 %: 12.7 against 11.4).
+// one row 10.0 against 10.8, two rows 12.7 against 11.1 at 50 % but 9.5 at 80 %); with three it needs a second launch
+// over the codes.
 static bool q8_in_integers(const FcArgs &a) {
     if (g_tune.dense_stream == 0 || !i8_applicable(a)) return false;
     return g_tune.dense_stream >= 2 || (a.B >= 3 && i8_blocks_per_rank(a) >= (a.B <= 4 ? 2 : 4));
