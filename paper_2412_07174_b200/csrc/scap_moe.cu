@@ -75,12 +75,31 @@ __global__ void __launch_bounds__(64) moe_route_kernel(const float *__restrict__
     }
 }
 
+// One expert's FC, in a body that is chosen by the rows it got (cluster-uniform).  BT = 1, 2, 4: FMA bodies only, with exactly as
+// many accumulator rows; a row of zeros less in every multiply, and one row alone has twice as many loads in flight per
+// thread as two.  BT = 8, 16: up to four rows of a larger batch take the FMA body of two or four.
+template <bool BF16, int BT, typename XT, int EPI, int TNT>
+__device__ __forceinline__ void expert_fc(const FcArgs &g) {
+    const int tile = blockIdx.x, s = blockIdx.y;
+    if constexpr (is_mma(BT)) {
+        if (g.B <= 2) fc_body<BF16, 2, MODE_GATHER, XT, EPI, TNT>(g, tile, s, false);
+        else if (g.B <= 4) fc_body<BF16, 4, MODE_GATHER, XT, EPI, TNT>(g, tile, s, false);
+        else fc_body_mma<BF16, BT, MODE_GATHER, XT, EPI, TNT>(g, tile, s, false);
+    } else {
+        if (BT == 1 || g.B == 1) fc_body<BF16, 1, MODE_GATHER, XT, EPI, TNT>(g, tile, s, false);
+        else if (BT == 2 || g.B == 2) fc_body<BF16, BT < 2 ? 1 : 2, MODE_GATHER, XT, EPI, TNT>(g, tile, s, false);
+        else if (g.B == 3) fc_body<BF16, BT < 4 ? 1 : 3, MODE_GATHER, XT, EPI, TNT>(g, tile, s, false);
+        else fc_body<BF16, BT, MODE_GATHER, XT, EPI, TNT>(g, tile, s, false);
+    }
+}
+
 // grid (tiles, S, E).  STAGE 1: packed gate|up FC of the rows routed to expert blockIdx.z, writing that
 // expert's z; STAGE 2: down FC reading z and writing each row to its (row, selection position) slot.
 template <bool BF16, int BT, int STAGE, int TNT>
 __global__ void __launch_bounds__(FC_THREADS, fc_min_blocks(BT)) moe_fc_kernel(const MoeArgs a) {
     using ST = typename std::conditional<BF16, __nv_bfloat16, __half>::type;
-    static_assert(fc_smem_for(BT) >= fc_smem_bytes(BT <= 4 ? BT : 4), "the FMA bodies for small experts use the kernel's shared memory");
+    static_assert(fc_smem_bytes(1) <= fc_smem_bytes(2) && fc_smem_bytes(2) <= fc_smem_bytes(3) && fc_smem_bytes(3) <= fc_smem_bytes(4) &&
+                      fc_smem_for(BT) >= fc_smem_bytes(BT <= 4 ? BT : 4), "the bodies for fewer rows use the kernel's shared memory");
     griddep_wait();
     griddep_launch_dependents();
     const int e = blockIdx.z;
@@ -98,26 +117,13 @@ __global__ void __launch_bounds__(FC_THREADS, fc_min_blocks(BT)) moe_fc_kernel(c
         g.x = a.h; g.x_ld = a.D; g.in_rows = a.route->rows[e];
         g.m = a.ex[e].m1; g.tau = a.ex[e].tau1; g.bias = a.ex[e].bgu_fused;
         g.y = z; g.y_ld = a.F;
-        // an expert that got up to four rows of a larger batch takes the FMA body (cluster-uniform choice)
-        if constexpr (is_mma(BT)) {
-            if (nb <= 2) fc_body<BF16, 2, MODE_GATHER, ST, EPI_GLU, TNT>(g, blockIdx.x, blockIdx.y, false);
-            else if (nb <= 4) fc_body<BF16, 4, MODE_GATHER, ST, EPI_GLU, TNT>(g, blockIdx.x, blockIdx.y, false);
-            else fc_body_mma<BF16, BT, MODE_GATHER, ST, EPI_GLU, TNT>(g, blockIdx.x, blockIdx.y, false);
-        } else {
-            fc_body<BF16, BT, MODE_GATHER, ST, EPI_GLU, TNT>(g, blockIdx.x, blockIdx.y, false);
-        }
+        expert_fc<BF16, BT, ST, EPI_GLU, TNT>(g);
     } else {
         g.W = a.ex[e].Wd; g.K = a.F; g.ldw = a.D; g.Nh = a.D; g.S = a.S2;
         g.x = z; g.x_ld = a.F;
         g.m = a.ex[e].m2; g.tau = a.ex[e].tau2; g.bias = a.ex[e].bd_fused;
         g.y = a.yslot; g.y_ld = a.D; g.out_rows = a.route->slots[e];
-        if constexpr (is_mma(BT)) {
-            if (nb <= 2) fc_body<BF16, 2, MODE_GATHER, float, EPI_BIAS, TNT>(g, blockIdx.x, blockIdx.y, false);
-            else if (nb <= 4) fc_body<BF16, 4, MODE_GATHER, float, EPI_BIAS, TNT>(g, blockIdx.x, blockIdx.y, false);
-            else fc_body_mma<BF16, BT, MODE_GATHER, float, EPI_BIAS, TNT>(g, blockIdx.x, blockIdx.y, false);
-        } else {
-            fc_body<BF16, BT, MODE_GATHER, float, EPI_BIAS, TNT>(g, blockIdx.x, blockIdx.y, false);
-        }
+        expert_fc<BF16, BT, float, EPI_BIAS, TNT>(g);
     }
 }
 
@@ -162,11 +168,20 @@ static cudaError_t launch_moe_fc_t(const MoeArgs &a, int tiles, int S, cudaStrea
     return tn == 128 ? launch_moe_fc_tn<BF16, BT, STAGE, 128>(a, tiles, S, st) : launch_moe_fc_tn<BF16, BT, STAGE, 256>(a, tiles, S, st);
 }
 
+// Three and four tokens: the kernel with a body for each count of rows, from this many input channels per split-K rank; below, the
+// one with fewer bodies (that of five to eight tokens).  A CTA that streams few channels spends its time at the start, and two
+// CTAs of an SM in different bodies fetch their code twice.  Whole layer, top 2 of 8 experts, four tokens, us, fewer -> more bodies:
+// D = 1024, F = 2048 26.7 -> 28.2; D = 2048, F = 7168 (1792 and 2048 channels per rank) 80.8 -> 74.8; D = 4096, F = 14336 257.9 -> 247.2.
+// Two tokens, where the two-row body used to take single rows as well: 149.1 -> 138.2, D = 1024, F = 2048 20.5 -> 19.9.
+constexpr int EXACT_ROWS_FROM = 1536;
+
 template <bool BF16, int STAGE>
 static cudaError_t launch_moe_fc(const MoeArgs &a, int tiles, int S, cudaStream_t st) {
-    switch (batch_tile(a.B)) {
+    const bool exact = a.B >= 3 && a.B <= 4 && (STAGE == 1 ? a.D : a.F) >= EXACT_ROWS_FROM * S;
+    switch (exact ? 4 : batch_tile(a.B)) {
         case 1: return launch_moe_fc_t<BF16, 1, STAGE>(a, tiles, S, st);
         case 2: return launch_moe_fc_t<BF16, 2, STAGE>(a, tiles, S, st);
+        case 4: return launch_moe_fc_t<BF16, 4, STAGE>(a, tiles, S, st);
         case 8: return launch_moe_fc_t<BF16, 8, STAGE>(a, tiles, S, st);
         default: return launch_moe_fc_t<BF16, 16, STAGE>(a, tiles, S, st);
     }

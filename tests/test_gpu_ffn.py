@@ -196,6 +196,20 @@ def test_moe_small(S, D, F, E, B, top_k):
     assert rel_l2_rows(y, y64) <= REL_L2_TOL
 
 
+@pytest.mark.parametrize("rows", [(1, 1), (2, 0), (1, 2), (1, 3), (1, 2, 3, 0, 2), (1, 2, 3, 4, 5, 1)])
+@pytest.mark.parametrize("D,F", [(200, 264), (1024, 2568), (2056, 13000)])
+def test_moe_rows_per_expert(S, D, F, rows):
+    """An expert's body is chosen by the rows it got: one to four each, and more, in one call."""
+    B, E = sum(rows), len(rows)
+    mo = build_moe(D, F, E, B)
+    mo["logits"] = mo["logits"] * 0.01
+    mo["logits"][np.arange(B), np.repeat(np.arange(E), rows)] += 1.0
+    y, ex, _ = run_moe(S, mo, 1)
+    y64, ex_o, _ = oracle.moe_ffn(si.to_f32(mo["h"], mo["dt"]), mo["logits"], mo["experts"], mo["dt"], 1)
+    assert np.array_equal(ex, ex_o) and np.array_equal(np.bincount(ex_o[:, 0], minlength=E), rows)
+    assert rel_l2_rows(y, y64) <= REL_L2_TOL
+
+
 # ---------------------------------------------------------------- non-GLU FFN (up -> exact GELU -> centred sparse down)
 
 def gelu_block(D, F, B, dt=si.BF16, T=64):
