@@ -205,10 +205,13 @@ scap_status scap_dense_fc(const void *x, const void *W, const float *b, float *y
  * dtype xdt (fp16 or bf16); everything else as in scap_sparse_fc / scap_dense_fc / scap_fold_bias, with these
  * differences: N must be a multiple of 16; the bias b of the dense call and of the folding is fp32 [N] or
  * NULL; idx_out / nnz_out are only available for B <= 2, else SCAP_ERR_SHAPE.  Three and more rows (and small layers)
- * run on the tensor cores - the integers and an exact split of d * wscale into three bf16 parts, fp32 accumulation, every
- * row of Wq requested once, by 9..16 rows twice - where K is a multiple of four and wscale 16-byte aligned; else two rows
- * at a time (results per row as in scap_sparse_fc).  The scale of a channel that a row drops has no part in that row of y.
- * Workspace: scap_fc_workspace(B, K, N). */
+ * run on the tensor cores where K is a multiple of four and wscale 16-byte aligned, else two rows at a time (results per row as in
+ * scap_sparse_fc).  Both tensor-core forms hold all bits of d * wscale, a product rounded to binary32 as in the other calls.  Long
+ * layers with K a multiple of eight: as integers - the bits of a value down to 2^-20 of the largest of its row among a rank's channels
+ * as six 8-bit digits, smaller and non-finite ones added by themselves; products and sums in 32-bit integers, exact; the sums of
+ * the digits put together in fp32; every row of Wq requested once.  Else: an exact split into three bf16 parts, fp32
+ * accumulation, every row of Wq requested once, by 9..16 rows twice.  The scale of a channel that a row drops has no part in that
+ * row of y.  Workspace: scap_fc_workspace(B, K, N). */
 scap_status scap_sparse_fc_q8(const void *x, scap_dtype xdt, const signed char *Wq, const float *wscale, const float *m,
                               const float *tau, const float *b_fused, float *y, int B, int K, int N, uint32_t *idx_out,
                               int *nnz_out, void *ws, size_t ws_bytes, scap_stream_t stream);

@@ -2,29 +2,32 @@
 //
 // The codes are integers, so they go into the tensor core as they lie in memory: the 128 columns of a tile are the M rows of the
 // MMA, and a TMA box of 128 channels with 128-byte swizzle is its operand (MN-major).  The activations become integers too: the
-// pruned and scaled values of a batch row are rounded to 31-bit fixed point under a common exponent, that of the largest one
-// among the rank's channels, and cut into four signed 8-bit digits, which are the N columns of the MMA (digit x BR + row).  Products
-// and sums are exact 32-bit integers in one accumulator, read once at the end.  So a weight costs no instruction at all, where the
-// mma.sync kernel (scap_fc_qm.cu) spends 1.5 on its conversion to bf16, and an activation is prepared once per CTA instead of once
-// per warp.
+// pruned and scaled values of a batch row are written as 45-bit fixed point under a common exponent, that of the largest one
+// among the rank's channels - three limbs of 15 bits, each of them two signed 8-bit digits - and the six digits are the N columns of the
+// MMA (digit x BR + row).  Products and sums are exact 32-bit integers in one accumulator, read once at the end.  So a weight costs no
+// instruction at all, where the mma.sync kernel (scap_fc_qm.cu) spends 1.5 on its conversion to bf16, and an activation is prepared
+// once per CTA instead of once per warp.
 //
 //   grid = (128-column tiles, S), cluster (1, S, 1), 384 threads, two CTAs per SM; a rank takes a contiguous range of blocks of
-//   128 channels; two blocks are a stage of the ring
+//   128 channels; one or two blocks are a stage of the ring
 //   warp 0      boxes and MMAs (the whole warp runs the loop, one lane issues)
 //   warps 1-11  activations: a unit is a block's 128 channels of four batch rows, a lane has four channels of each row.  First the
 //               largest value of every row (the warp keeps the values of its first units in registers), then the digits
 //   warps 4-7   at the end: a thread per column reads the accumulator
 //
-// Precision: a value is off by at most 2^-31 of the largest of its row in the rank, the sum of a rank is put together from its digits
-// with three roundings to binary32: 5e-8 .. 7e-8 from 64 bits where the mma.sync kernel is 6e-8 .. 9e-8 off (128 x 128 to
-// 14336 x 11008, 1 - 16 rows).  A kept value that is not finite is left out of the digits and its row is marked; value x code of
-// those channels is then added one by one.
+// Precision: no bit of a value is rounded away.  The 24 bits of a value down to 2^-20 of its row's largest one in the rank all lie in its
+// digits.  A kept value below that, or one that is not finite, has no digits: its row is marked, and value x code of those channels is
+// added by itself at the end, in binary64.  (Four digits under the same exponent cut every value below 2^-6 of the largest: with one
+// activation 10^4 times the others the columns that do not use it were 5e-6 off.)  The sum of a rank is put together from its digits
+// in binary32, a rounding per limb and one between two limbs.
 //
 // What bounds it: K = 11008, N = 4096, half pruned, weights from DRAM, us per call, mma.sync kernel -> this one: 3 rows
-// 18.1 -> 12.8, 8 rows 24.0 -> 14.9, 16 rows 41.4 -> 20.5 (the 45 MB of codes take 6.9 at copy speed).  The first MMA starts 3 - 4 us
+// 18.1 -> 12.3, 8 rows 23.8 -> 14.5, 16 rows 41.0 -> 20.0 (the 45 MB of codes take 6.9 at copy speed).  The first MMA starts 3 - 4 us
 // into the call: activations through L2 (1 us under the weight stream), the pass for the exponents, the digits - code that all 24
-// warps of an SM run at once, bound by instruction issue - while the ring has been full for two of them; the rest of the codes then
-// comes at 5.9 TB/s.  Tried and slower: an exponent per block and an accumulator per block or two, so that the first MMA does not
+// warps of an SM run at once, bound by instruction issue - while the ring has been full for two of them.  So a limb comes off a value by
+// additions and multiply-adds, where a conversion to an integer takes four issue slots, and six digits cost what four by
+// conversion did (3 / 8 / 16 rows 12.4 / 14.9 / 20.0, K = 4096 with its four blocks per rank 7.0 / 8.0 / 10.1 against 7.3 / 8.3 / 10.9).
+// Tried and slower: an exponent per block and an accumulator per block or two, so that the first MMA does not
 // wait for a pass over all activations (8 rows 15.4 - 16.3, 16 rows 21.5 - 30.6: reading 11 accumulators costs more than the pass);
 // 256 threads (15.4); 4-bit codes the same way, the nibbles separated in shared memory (11008 x 4096, one row 15.4 - 27 against 13.0:
 // half the bytes per stage, and an accumulator read per scale group).
@@ -41,23 +44,30 @@ namespace scap {
 
 constexpr int I8_TN = 128;        // columns per CTA
 constexpr int I8_KB = 128;        // channels per block (a box, a unit of activations)
-constexpr int I8_BPS = 2;         // blocks per stage: eight MMAs of 32 channels per round of waits
 constexpr int I8_THREADS = 384;
-constexpr int I8_PREP = I8_THREADS / 32 - 1;  // warps that prepare activations
+constexpr int I8_WARPS = I8_THREADS / 32;
+constexpr int I8_PREP = I8_WARPS - 1;         // warps that prepare activations
 constexpr int I8_KEEP = 2;        // units whose values a warp keeps between the two passes
 static_assert(I8_KEEP == 2, "the first pass asks for two units at once");
 constexpr int I8_BOX = I8_KB * I8_TN;         // 16 KB
-// BR = batch rows of the instantiation (4, 8 or 16).
-// 16 channels of the activation operand: 4 BR rows of 16 bytes, and 16 bytes more, so that the chunks of a warp's stores start in different banks
-__host__ __device__ constexpr int i8_chunk(int BR) { return 4 * BR * 16 + 16; }
-__host__ __device__ constexpr int i8_xbytes(int BR) { return I8_BPS * I8_KB / 16 * i8_chunk(BR); }
+constexpr int I8_ND = 6;          // digits of an activation
+// BR = batch rows of the instantiation (4, 8 or 16).  Two blocks are a stage: eight MMAs of 32 channels per round of waits.  (One with
+// sixteen rows, whose activations take half of the shared memory otherwise.)
+__host__ __device__ constexpr int i8_bps(int BR) { return BR == 16 ? 1 : 2; }
+// 16 channels of the activation operand: 6 BR rows of 16 bytes, and 16 bytes more, so that the chunks of a warp's stores start in different banks
+__host__ __device__ constexpr int i8_chunk(int BR) { return I8_ND * BR * 16 + 16; }
+__host__ __device__ constexpr int i8_xbytes(int BR) { return i8_bps(BR) * I8_KB / 16 * i8_chunk(BR); }
+__host__ __device__ constexpr int i8_ncols(int BR) { return (I8_ND * BR + 15) / 16 * 16; }  // N of the MMA (four rows: eight more, whose sums nobody reads)
+__host__ __device__ constexpr int i8_tcols(int BR) { return i8_ncols(BR) <= 32 ? 32 : i8_ncols(BR) <= 64 ? 64 : 128; }
 __host__ __device__ constexpr int i8_nw(int BR) { return BR == 16 ? 4 : 5; }  // blocks of weights in the ring
-// Stages of activations.  At least as many as lie between two units of a warp (11 units go round; one, two, or three and four per block):
-// a warp then meets every phase of a slot's barrier, which a parity only tells from its neighbours.
-__host__ __device__ constexpr int i8_nx(int BR) { return BR == 4 ? 6 : BR == 8 ? 3 : 2; }
-constexpr int i8_apart(int ups) { return ((I8_PREP + ups - 1) / ups + I8_BPS - 1) / I8_BPS; }  // stages between two units of a warp, at most
-static_assert(i8_apart(1) <= i8_nx(4) && i8_apart(2) <= i8_nx(8) && i8_apart(3) <= i8_nx(16) && i8_apart(4) <= i8_nx(16),
-              "units of a warp must not lie further apart than the slots of the activations reach");
+__host__ __device__ constexpr int i8_nx(int BR) { return BR == 4 ? 4 : BR == 8 ? 2 : 3; }  // stages of activations
+// Barriers that say that a stage has been multiplied.  At least as many as there are slots, and as lie between two units of a warp (11
+// units go round; one, two, or three and four per block): a warp that waits for a stage then knows that the one before on the same
+// barrier is done, and the one after cannot be (it needs this warp's own unit) - a parity only tells neighbours apart.
+__host__ __device__ constexpr int i8_ne(int BR) { return BR == 4 ? 6 : BR == 8 ? 3 : 4; }
+constexpr int i8_apart(int ups, int bps) { return ((I8_PREP + ups - 1) / ups + bps - 1) / bps; }  // stages between two units of a warp, at most
+static_assert(i8_apart(1, i8_bps(4)) <= i8_ne(4) && i8_apart(2, i8_bps(8)) <= i8_ne(8) && i8_apart(3, i8_bps(16)) <= i8_ne(16) && i8_apart(4, i8_bps(16)) <= i8_ne(16) &&
+                  i8_nx(4) <= i8_ne(4) && i8_nx(8) <= i8_ne(8) && i8_nx(16) <= i8_ne(16), "barriers of the stages of activations");
 // What the host works out once instead of every warp of every CTA: the code before the first MMA runs on all warps of an SM at the same
 // moment and is bound by instruction issue (a division costs a warp as much as the activations of a row).
 struct I8Args {
@@ -68,12 +78,24 @@ struct I8Args {
 };
 struct I8Misc {
     unsigned long long wfull[5], wempty[5];  // a block of weights has landed / has been multiplied
-    unsigned long long xfull[6], xempty[6];  // activations of a stage
+    unsigned long long xfull[4], xempty[6];  // activations of a stage are written (per slot) / have been multiplied (stage modulo i8_ne)
     unsigned long long done, recv;
     uint32_t tmem_base;
     int abort;
     uint32_t top[16], fin[16];  // pattern of a row's largest magnitude; of the largest finite one
+    uint32_t apart;             // rows with a value too small for the digits
 };
+struct I8Entry {
+    float v;
+    int k;
+};
+struct I8Apart {  // in the ring, when the stream is done
+    float sum[16][I8_TN];             // per row and column: the channels without digits
+    double part[I8_THREADS / I8_TN][I8_TN];
+    int count[I8_WARPS];
+    I8Entry entry[I8_WARPS][I8_KB];   // a warp's list
+};
+static_assert(sizeof(I8Apart) <= i8_nw(16) * I8_BOX, "it must fit in the ring");
 __host__ __device__ constexpr int i8_off_x(int BR) { return i8_nw(BR) * I8_BOX; }
 __host__ __device__ constexpr int i8_off_gather(int BR) { return i8_off_x(BR) + i8_nx(BR) * i8_xbytes(BR); }
 __host__ __device__ constexpr int i8_off_misc(int BR) { return i8_off_gather(BR) + BR * (I8_TN + 16) * 4; }
@@ -116,33 +138,66 @@ __device__ __forceinline__ bool i8_wait(unsigned long long *bar, uint32_t parity
     return false;
 }
 
-// Sum of value x code over the channels k0 .. k1 - 1 whose kept value is not finite, one batch row and one column.
-template <int MODE, typename XT>
-__device__ __noinline__ float i8_not_finite(const FcArgs *a, int k0, int k1, int b, int col) {
-    const float tau = MODE == MODE_GATHER ? ld_act(a->tau) : 0.0f;
-    float sum = 0.0f;
-    for (int k = k0; k < k1; ++k) {
-        float v = widen1(ld_act(static_cast<const XT *>(a->x) + (size_t)b * a->x_ld + k));
-        if (MODE == MODE_GATHER && a->m) v = __fsub_rn(v, ld_act(a->m + k));
-        if (MODE == MODE_GATHER && !(fabsf(v) >= tau)) continue;
-        v = __fmul_rn(v, ld_act(a->wscale + k));
-        if ((__float_as_uint(v) & 0x7f800000u) == 0x7f800000u) sum += v * (float)static_cast<const signed char *>(a->W)[(size_t)k * a->ldw + col];
-    }
-    return sum;
-}
-
 __device__ __forceinline__ uint32_t i8_bits(float v) { return __float_as_uint(v) & 0x7fffffffu; }
 __device__ __forceinline__ uint32_t i8_top(const float (&v)[4]) { return max(max(i8_bits(v[0]), i8_bits(v[1])), max(i8_bits(v[2]), i8_bits(v[3]))); }
-// Fixed point under the exponent of `top`: |v| < 2^(e - 126), so times 2^(156 - e) it is below 2^30 (where the largest value is under
-// 2^-96, bits below 2^-156 are lost).
-__device__ __forceinline__ int i8_shift(uint32_t top) { return min(156 - (int)(top >> 23), 126); }
+// Fixed point under the exponent e of `top`: |v| < 2^(e - 126), so times 2^(140 - e) it is below 2^14, the most that the first limb
+// takes.  Three limbs then hold multiples of 2^(e - 170): all bits of a value from 2^(e - 147) on.
+__device__ __forceinline__ int i8_shift(uint32_t top) { return min(140 - (int)(top >> 23), 126); }
 __device__ __forceinline__ float i8_pow2(int e) { return __uint_as_float((uint32_t)(127 + e) << 23); }
+__device__ __forceinline__ float i8_least(int shift) { return i8_pow2(max(-7 - shift, -126)); }
+// A value that gets no digits (`least` of its row; dropped channels are zeros and have digits).
+__device__ __forceinline__ bool i8_is_apart(float v, float least) { return (fabsf(v) < least && v != 0.0f) || i8_bits(v) >= 0x7f800000u; }
+
+// Sums of value x code over the channels without digits, for the rows that have some, to `out`.  The whole CTA, when the ring is free.  A
+// warp lists the channels of 128 in their order, a third of the threads each takes a third of the lists, a thread per column.
+template <int MODE, typename XT>
+__device__ __noinline__ void i8_apart_sums(const FcArgs *a, I8Apart *out, const uint32_t *top, uint32_t rows, int k_lo, int k_hi, int tile) {
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, c = tid % I8_TN, third = tid / I8_TN, col = tile * I8_TN + c;
+    const float tau = MODE == MODE_GATHER ? ld_act(a->tau) : 0.0f;
+    const signed char *W = static_cast<const signed char *>(a->W) + col;
+    for (; rows; rows &= rows - 1) {
+        const int b = __ffs(rows) - 1;
+        const float least = i8_least(i8_shift(top[b]));
+        const XT *x = static_cast<const XT *>(a->x) + (size_t)b * a->x_ld;
+        double sum = 0.0;
+        for (int k0 = k_lo; k0 < k_hi; k0 += I8_WARPS * I8_KB) {
+            int n = 0;
+            for (int e = 0; e < I8_KB; e += 32) {
+                const int k = k0 + warp * I8_KB + e + lane;
+                float v = 0.0f;
+                if (k < k_hi) {
+                    v = widen1(ld_act(x + k));
+                    if (MODE == MODE_GATHER && a->m) v = __fsub_rn(v, ld_act(a->m + k));
+                    v = MODE == MODE_DENSE || fabsf(v) >= tau ? __fmul_rn(v, ld_act(a->wscale + k)) : 0.0f;
+                }
+                const bool on = i8_is_apart(v, least);
+                const uint32_t vote = __ballot_sync(0xffffffffu, on);
+                if (on) out->entry[warp][n + __popc(vote & ((1u << lane) - 1u))] = I8Entry{v, k};
+                n += __popc(vote);
+            }
+            if (lane == 0) out->count[warp] = n;
+            __syncthreads();
+            if (col < a->Nh) {
+                for (int w = third; w < I8_WARPS; w += I8_THREADS / I8_TN)
+                    for (int i = 0; i < out->count[w]; ++i) {
+                        const I8Entry q = out->entry[w][i];
+                        sum += (double)q.v * (double)W[(size_t)q.k * a->ldw];
+                    }
+            }
+            __syncthreads();
+        }
+        out->part[third][c] = sum;
+        __syncthreads();
+        if (third == 0) out->sum[b][c] = (float)(out->part[0][c] + out->part[1][c] + out->part[2][c]);
+    }
+    __syncthreads();
+}
 
 template <int BR, int MODE, typename XT>
 __global__ void __launch_bounds__(I8_THREADS, 2) fc_i8_kernel(const __grid_constant__ I8Args ia, const __grid_constant__ CUtensorMap tmap) {
     const FcArgs &a = ia.f;
-    constexpr int NC = 4 * BR, NW = i8_nw(BR), NX = i8_nx(BR);
-    constexpr uint32_t XB = i8_xbytes(BR), LBO = i8_chunk(BR), TCOLS = NC < 32 ? 32 : NC;
+    constexpr int NC = i8_ncols(BR), NW = i8_nw(BR), NX = i8_nx(BR), NE = i8_ne(BR), BPS = i8_bps(BR);
+    constexpr uint32_t XB = i8_xbytes(BR), LBO = i8_chunk(BR), TCOLS = i8_tcols(BR);
     extern __shared__ unsigned char smem_raw[];
     unsigned char *smem = reinterpret_cast<unsigned char *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
     unsigned char *s_w = smem, *s_x = smem + i8_off_x(BR);
@@ -158,19 +213,18 @@ __global__ void __launch_bounds__(I8_THREADS, 2) fc_i8_kernel(const __grid_const
     const int per = ia.per;
     const uint32_t recv_bar = smem_addr(&misc->recv);
     const int b_lo = s * ia.blocks + min(s, ia.extra), n = ia.blocks + (s < ia.extra ? 1 : 0);  // this rank's blocks
-    const int k_lo = b_lo * I8_KB, k_hi = min(K, k_lo + n * I8_KB), nst = (n + I8_BPS - 1) / I8_BPS;   // its channels and stages
+    const int k_lo = b_lo * I8_KB, k_hi = min(K, k_lo + n * I8_KB), nst = (n + BPS - 1) / BPS;   // its channels and stages
     const int ups = (B + 3) >> 2;  // units of a block: four batch rows each
     if (tid == 0) {
         for (int i = 0; i < NW; ++i) {
             mbar_init(&misc->wfull[i], 1);
             mbar_init(&misc->wempty[i], 1);
         }
-        for (int i = 0; i < NX; ++i) {
-            mbar_init(&misc->xfull[i], I8_BPS * ups);
-            mbar_init(&misc->xempty[i], 1);
-        }
+        for (int i = 0; i < NX; ++i) mbar_init(&misc->xfull[i], BPS * ups);
+        for (int i = 0; i < NE; ++i) mbar_init(&misc->xempty[i], 1);
         mbar_init(&misc->done, 1);
         misc->abort = 0;
+        misc->apart = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         if (S > 1) {
             const int owned = max(0, min(per, I8_TN - s * per));
@@ -352,7 +406,7 @@ __global__ void __launch_bounds__(I8_THREADS, 2) fc_i8_kernel(const __grid_const
         constexpr uint32_t idesc = (2u << 4) | (1u << 7) | (1u << 10) | (1u << 15) | ((uint32_t)(NC >> 3) << 17) | ((uint32_t)(I8_TN >> 4) << 24);
         constexpr uint32_t WK = 32 * I8_TN >> 4, XK = (2 * LBO) >> 4;  // 32 channels further, in units of 16 bytes
         const uint64_t dw0 = tc_desc(smem_u32(s_w), I8_BOX, 1024, 2), dx0 = tc_desc(smem_u32(s_x), LBO, 128, 0);
-        uint32_t ws = 0, wpar = 0, xs = 0, xpar = 0, rs = 0, rpar = 0;  // slots: weights, activations, weights to ask for
+        uint32_t ws = 0, wpar = 0, xs = 0, xpar = 0, xe = 0, rs = 0, rpar = 0;  // slots: weights, activations and their barrier, weights to ask for
         auto next = [&](uint32_t &slot, uint32_t &par) {
             if (++slot == NW) { slot = 0; par ^= 1u; }
         };
@@ -360,8 +414,8 @@ __global__ void __launch_bounds__(I8_THREADS, 2) fc_i8_kernel(const __grid_const
 #pragma unroll 1
         for (int i = 0; i < nst; ++i) {
             // both operands, and the slots of the stage before, which take the next boxes: each is waited for by a lane of its own
-            const bool two = 2 * i + 1 < n;
-            const int refill = i >= 1 ? min(2, n - asked) : 0;
+            const bool two = BPS == 2 && 2 * i + 1 < n;
+            const int refill = i >= 1 ? min(BPS, n - asked) : 0;
             uint32_t ws1 = ws, wpar1 = wpar, rs1 = rs, rpar1 = rpar;
             next(ws1, wpar1);
             next(rs1, rpar1);
@@ -374,20 +428,22 @@ __global__ void __launch_bounds__(I8_THREADS, 2) fc_i8_kernel(const __grid_const
             if (!warp_wait(bar, bpar, 2)) break;
             tc_fence_after();
             const uint64_t da = dw0 + ws * (I8_BOX >> 4), db = dw0 + ws1 * (I8_BOX >> 4), dx = dx0 + xs * (XB >> 4);
-            const int left = (k_hi - k_lo - i * I8_BPS * I8_KB + 31) >> 5;  // steps of 32 channels
+            const int left = (k_hi - k_lo - i * BPS * I8_KB + 31) >> 5;  // steps of 32 channels
             if (leader) {
-                if (left >= 8) {
+                if (left >= 4 * BPS) {
 #pragma unroll
                     for (uint32_t ks = 0; ks < 4; ++ks) tc_mma_i8(tmem, da + ks * WK, dx + ks * XK, idesc, (ks > 0 || i > 0) ? 1u : 0u);
+                    if constexpr (BPS == 2) {
 #pragma unroll
-                    for (uint32_t ks = 0; ks < 4; ++ks) tc_mma_i8(tmem, db + ks * WK, dx + (4 + ks) * XK, idesc, 1u);
+                        for (uint32_t ks = 0; ks < 4; ++ks) tc_mma_i8(tmem, db + ks * WK, dx + (4 + ks) * XK, idesc, 1u);
+                    }
                 } else {
 #pragma unroll 1
                     for (int ks = 0; ks < left; ++ks) tc_mma_i8(tmem, (ks < 4 ? da : db) + (ks & 3) * WK, dx + ks * XK, idesc, (ks > 0 || i > 0) ? 1u : 0u);
                 }
                 tc_commit(&misc->wempty[ws]);
                 if (two) tc_commit(&misc->wempty[ws1]);
-                tc_commit(&misc->xempty[xs]);
+                tc_commit(&misc->xempty[xe]);
                 if (refill > 0) box(asked, rs);
                 if (refill > 1) box(asked + 1, rs1);
             }
@@ -395,8 +451,9 @@ __global__ void __launch_bounds__(I8_THREADS, 2) fc_i8_kernel(const __grid_const
             if (refill > 1) next(rs, rpar);
             asked += max(0, refill);
             next(ws, wpar);
-            next(ws, wpar);
+            if constexpr (BPS == 2) next(ws, wpar);
             if (++xs == NX) { xs = 0; xpar ^= 1u; }
+            if (++xe == NE) xe = 0;
         }
         // all MMAs have finished, and no copy is under way, before anyone leaves
         int own_abort = 0;
@@ -407,32 +464,55 @@ __global__ void __launch_bounds__(I8_THREADS, 2) fc_i8_kernel(const __grid_const
     } else {
         // ---- second pass: the digits
         int blk = ub, rq = uq;
-        const uint32_t shifts = lane < BR ? (uint32_t)i8_shift(misc->top[lane]) : 0u;  // lane b: of row b
+        const int shifts = lane < BR ? i8_shift(misc->top[lane]) : 0;  // lane b: of row b
         auto digits = [&](const float (&v)[4][4]) -> bool {
-            const int i = blk / I8_BPS;
+            const int i = blk / BPS;
             const uint32_t xs = (uint32_t)i % NX;
-            if (i >= NX && !warp_wait(&misc->xempty[xs], ((uint32_t)(i / NX) & 1u) ^ 1u, 1)) return false;
-            unsigned char *dst = s_x + xs * XB + ((blk % I8_BPS) * (I8_KB / 16) + (lane >> 2)) * LBO + (lane & 3) * 4 + rq * 64;  // (rows of 16 bytes follow one another)
+            if (i >= NX && !warp_wait(&misc->xempty[(uint32_t)(i - NX) % NE], ((uint32_t)(i - NX) / NE) & 1u, 1)) return false;
+            unsigned char *dst = s_x + xs * XB + ((blk % BPS) * (I8_KB / 16) + (lane >> 2)) * LBO + (lane & 3) * 4 + rq * 64;  // (rows of 16 bytes follow one another)
 #pragma unroll
             for (int r = 0; r < 4; ++r) {
                 if (rq * 4 + r < B) {
-                    const float up = i8_pow2((int)__shfl_sync(0xffffffffu, shifts, rq * 4 + r));
-                    uint32_t q[4];  // four signed digits each
+                    const int shift = __shfl_sync(0xffffffffu, shifts, rq * 4 + r);
+                    const float up = i8_pow2(shift), least = i8_least(shift);
+                    float w[4] = {v[r][0], v[r][1], v[r][2], v[r][3]};
+                    bool some = odd != 0;
 #pragma unroll
-                    for (int e = 0; e < 4; ++e) q[e] = ((uint32_t)__float2int_rn((odd && i8_bits(v[r][e]) >= 0x7f800000u ? 0.0f : v[r][e]) * up) + 0x00808080u) ^ 0x00808080u;
-                    const uint32_t l01 = __byte_perm(q[0], q[1], 0x5140), h01 = __byte_perm(q[0], q[1], 0x7362);
-                    const uint32_t l23 = __byte_perm(q[2], q[3], 0x5140), h23 = __byte_perm(q[2], q[3], 0x7362);
-                    *reinterpret_cast<uint32_t *>(dst + (0 * BR + r) * 16) = __byte_perm(l01, l23, 0x5410);  // digit x BR + row: the lowest first
-                    *reinterpret_cast<uint32_t *>(dst + (1 * BR + r) * 16) = __byte_perm(l01, l23, 0x7632);
-                    *reinterpret_cast<uint32_t *>(dst + (2 * BR + r) * 16) = __byte_perm(h01, h23, 0x5410);
-                    *reinterpret_cast<uint32_t *>(dst + (3 * BR + r) * 16) = __byte_perm(h01, h23, 0x7632);
+                    for (int e = 0; e < 4; ++e) some |= fabsf(w[e]) < least && w[e] != 0.0f;
+                    if (some) {  // (rare)
+#pragma unroll
+                        for (int e = 0; e < 4; ++e) {
+                            if (i8_is_apart(w[e], least)) {
+                                w[e] = 0.0f;
+                                atomicOr(&misc->apart, 1u << (rq * 4 + r));
+                            }
+                        }
+                    }
+                    // Limbs from the top, rounded to the nearest integer by adding 1.5 x 2^23; 0x8080 more, and the lower 16 bits of the sum are
+                    // two signed digits with their signs turned round.  What is left of a value is exact at every step.
+                    constexpr float M = 12582912.0f + 32896.0f;
+                    uint32_t t[3][4];
+#pragma unroll
+                    for (int e = 0; e < 4; ++e) {
+                        const float t2 = __fmaf_rn(w[e], up, M), d1 = __fmaf_rn(w[e], up, -__fsub_rn(t2, M));
+                        const float t1 = __fmaf_rn(d1, 32768.0f, M), d0 = __fmaf_rn(d1, 32768.0f, -__fsub_rn(t1, M));
+                        t[0][e] = __float_as_uint(__fmaf_rn(d0, 32768.0f, M));
+                        t[1][e] = __float_as_uint(t1);
+                        t[2][e] = __float_as_uint(t2);
+                    }
+#pragma unroll
+                    for (int l = 0; l < 3; ++l) {  // digit x BR + row: the lowest first
+                        const uint32_t t01 = __byte_perm(t[l][0], t[l][1], 0x5140), t23 = __byte_perm(t[l][2], t[l][3], 0x5140);
+                        *reinterpret_cast<uint32_t *>(dst + (2 * l * BR + r) * 16) = __byte_perm(t01, t23, 0x5410) ^ 0x80808080u;
+                        *reinterpret_cast<uint32_t *>(dst + ((2 * l + 1) * BR + r) * 16) = __byte_perm(t01, t23, 0x7632) ^ 0x80808080u;
+                    }
                 }
             }
             asm volatile("fence.proxy.async.shared::cta;" ::: "memory");  // generic-proxy writes -> visible to the tensor core
             __syncwarp();
             if (lane == 0) {
                 mbar_arrive(&misc->xfull[xs]);
-                if (blk + 1 == n && blk % I8_BPS == 0) mbar_arrive(&misc->xfull[xs]);  // the last stage has no second block
+                if (BPS == 2 && blk + 1 == n && blk % 2 == 0) mbar_arrive(&misc->xfull[xs]);  // the last stage has no second block
             }
             step(blk, rq);
             return true;
@@ -459,28 +539,27 @@ __global__ void __launch_bounds__(I8_THREADS, 2) fc_i8_kernel(const __grid_const
     }
     // ---- cluster exchange, push form: a column of the tile is a TMEM lane; every sum of the rank goes to the rank that finishes its
     // column as a store that counts down its barrier
-    __syncwarp();
+    __syncthreads();  // (all MMAs have finished, and every row with a value without digits is marked)
+    const uint32_t apart = misc->apart | odd;
+    I8Apart *const s_apart = reinterpret_cast<I8Apart *>(s_w);
+    if (apart) i8_apart_sums<MODE, XT>(&a, s_apart, misc->top, apart, k_lo, k_hi, tile);
     if (S > 1) cluster_wait();  // every rank's barrier is initialised (all ranks arrived before their streams)
     if (warp >= 4 && warp < 8) {
         const bool ok = warp_wait(&misc->done, 0, 4) && __all_sync(0xffffffffu, *abort_flag == 0);
         tc_fence_after();
-        const int dc = (warp & 3) * 32 + lane, col = tile * I8_TN + dc;
+        const int dc = (warp & 3) * 32 + lane;
         const int r = (int)((uint32_t)dc * ia.per_inv >> 20), slot0 = s * BR * per + (dc - r * per);
         const uint32_t dst0 = S > 1 ? cluster_addr(smem_addr(s_gather) + 4u * (uint32_t)slot0, (uint32_t)r) : 0u;
         const uint32_t dbar = S > 1 ? cluster_addr(recv_bar, (uint32_t)r) : 0u;
         const uint32_t lanes = tmem + ((uint32_t)((warp & 3) * 32) << 16);
-        constexpr int RL = BR < 8 ? BR : 8;
-        float *s_odd = reinterpret_cast<float *>(s_w) + dc;  // the ring is free: a thread's own column
-        if (odd) {
-#pragma unroll 1
-            for (int b = 0; b < B; ++b) s_odd[b * I8_TN] = (odd >> b & 1) && col < a.Nh ? i8_not_finite<MODE, XT>(&a, k_lo, k_hi, b, col) : 0.0f;
-        }
+        constexpr int RL = 4;  // rows at a time
 #pragma unroll
         for (int b0 = 0; b0 < BR; b0 += RL) {
-            uint32_t v[4][RL];
+            if (b0 >= B) break;  // (the same for the whole warp)
+            uint32_t v[I8_ND][RL];
             if (ok) {
 #pragma unroll
-                for (int d = 0; d < 4; ++d) tc_ldn(v[d], lanes + (uint32_t)(d * BR + b0));
+                for (int d = 0; d < I8_ND; ++d) tc_ldn(v[d], lanes + (uint32_t)(d * BR + b0));
                 asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
             }
 #pragma unroll
@@ -489,9 +568,11 @@ __global__ void __launch_bounds__(I8_THREADS, 2) fc_i8_kernel(const __grid_const
                 if (b < B) {
                     float y = 0.0f;
                     if (ok) {
-                        const float hi = fmaf((float)(int)v[3][e], 256.0f, (float)(int)v[2][e]), lo = fmaf((float)(int)v[1][e], 256.0f, (float)(int)v[0][e]);
-                        y = fmaf(hi, 65536.0f, lo) * i8_pow2(-i8_shift(misc->top[b]));
-                        if (odd) y += s_odd[b * I8_TN];
+                        float limb[3];
+#pragma unroll
+                        for (int l = 0; l < 3; ++l) limb[l] = fmaf((float)(int)v[2 * l + 1][e], 256.0f, (float)(int)v[2 * l][e]);
+                        y = fmaf(fmaf(limb[0], 0x1p-15f, limb[1]), 0x1p-15f, limb[2]) * i8_pow2(-i8_shift(misc->top[b]));
+                        if (apart >> b & 1) y += s_apart->sum[b][dc];
                     }
                     if (S > 1) st_async_f32(dst0 + 4u * (uint32_t)(b * per), y, dbar);
                     else s_gather[slot0 + b * per] = y;

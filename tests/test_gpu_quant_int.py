@@ -1,8 +1,9 @@
 """The integer kernel of the 8-bit calls (scap_fc_i8.cu) at the edges of its blocks of 128 channels, its pairs of blocks, its ring and
 its column tiles, for every number of row quarters, sparse and dense - and which calls take it.
 
-Bound: the codes are integers, an activation is rounded to 2^-31 of the largest of its row, products and sums are exact.  What is left: the
-sum of a rank is put together from its digits (three roundings and one by the unit), at most eight ranks and the bias are added - at
+Bound: the codes are integers, all bits of an activation are in its digits or it is added by itself in binary64, products and sums are
+exact.  What is left: the sum of a rank is put together from its digits (three roundings and one for what was added by itself: the upper
+limb's sum or, where that is zero, the next one's; the rest is 2^-15 of it), at most eight ranks and the bias are added - at
 most 13 roundings of 2^-24, of sums that are on average smaller than the last one."""
 import numpy as np
 import pytest
@@ -92,6 +93,51 @@ def test_a_row_that_is_not_finite_leaves_the_others_as_they_are(S):
         want2, want7 = np.inf * q[5].astype(np.float64) + np.inf * q[3999].astype(np.float64), -np.inf * q[2000].astype(np.float64)
     assert np.array_equal(out[1][2].numpy(), want2.astype(np.float32), equal_nan=True)
     assert np.array_equal(out[1][7].numpy(), want7.astype(np.float32), equal_nan=True)
+
+
+@pytest.mark.parametrize("large", [1e3, 1e5, 1e10])
+@pytest.mark.parametrize("K,N,B,split", [(4096, 144, 3, 1), (4104, 272, 8, 3), (4096, 144, 16, 8)])
+def test_columns_that_do_not_use_a_large_activation_keep_their_bits(S, K, N, B, split, large):
+    """One activation far above the others of its row, whose code is zero in every other column: those columns are as exact as without it."""
+    d, xf, q, scale = layer(K, N, B, si.BF16)
+    at = 37 * np.arange(B) % K  # another channel in every row
+    x = xf.copy()
+    x[np.arange(B), at] = large
+    q[at, ::2] = 0
+    bits = si.to_bits(x, si.BF16)
+    args, ws = (torch.from_numpy(q).cuda(), f32(scale)), workspace(S.scap_fc_workspace(B, K, N))
+    y = torch.empty((B, N), dtype=torch.float32, device="cuda")
+    S.scap_tune("split_k", split)
+    for m, tau in ((d["m_true"], 0.2), (None, 0.0)):
+        S.scap_sparse_fc_q8(dev(bits, si.BF16), *args, None if m is None else f32(m), f32([tau]), None, y, ws.payload)
+        want = oracle.sparse_fc_q8(si.to_f32(bits, si.BF16), q, scale, m, tau, None)
+        got = y.cpu().numpy()
+        assert rel_l2_rows(got[:, ::2], want[:, ::2]) <= TOL
+        assert rel_l2_rows(got[:, 1::2], want[:, 1::2]) <= TOL
+
+
+@pytest.mark.parametrize("K,N,B,split", [(1544, 144, 3, 1), (4096, 272, 6, 2), (3080, 144, 16, 1)])
+@pytest.mark.parametrize("power,sizes", [(0, 48), (100, 48), (-115, 10)])
+def test_values_of_every_size_in_one_row(S, K, N, B, split, power, sizes):
+    """Channel k lies 2^(k mod sizes) below the largest, and a column uses the channels of one size only, from the window of the digits or
+    from below it: every column is right by itself.  (And with all of them near either end of the range of binary32.)"""
+    rng = np.random.default_rng(5)
+    size = np.arange(K) % sizes
+    q = np.where(size[:, None] == np.arange(N)[None, :] % sizes, rng.integers(-127, 128, (K, N)), 0).astype(np.int8)
+    scale = np.ldexp(rng.uniform(1, 2, K), power - size).astype(np.float32)
+    bits = si.to_bits(rng.uniform(1, 2, (B, K)) * rng.choice([-1, 1], (B, K)), si.BF16)
+    args, ws = (torch.from_numpy(q).cuda(), f32(scale)), workspace(S.scap_fc_workspace(B, K, N))
+    y = torch.empty((B, N), dtype=torch.float32, device="cuda")
+    S.scap_tune("split_k", split)
+    for tau, run in ((0.0, "dense"), (1.25, "sparse")):
+        if run == "dense":
+            S.scap_dense_fc_q8(dev(bits, si.BF16), *args, None, y, ws.payload)
+        else:
+            S.scap_sparse_fc_q8(dev(bits, si.BF16), *args, None, f32([tau]), None, y, ws.payload)
+        want = oracle.sparse_fc_q8(si.to_f32(bits, si.BF16), q, scale, None, tau, None)
+        got = y.cpu().numpy().astype(np.float64)
+        for s in range(sizes):
+            assert rel_l2_rows(got[:, s::sizes], want[:, s::sizes]) <= TOL, s
 
 
 def test_a_wait_that_runs_out_is_reported_and_the_next_call_is_right(S):
