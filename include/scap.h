@@ -100,7 +100,8 @@ int scap_version(void);
  *              Grouped calls: 0 = always one gather per group (better when the rows of a group keep the very same
  *              channels, and less than about a fifth of them); else see scap_sparse_fc_grouped
  *   "tc_spin"  tcgen05 kernels: how often a wait on one of its shared-memory barriers polls before it gives up
- *              (0 = the built-in limit of about a million polls, the default).  A limit of 1 makes the waits of
+ *              (0 = the built-in limits, the default: about a million polls, tens of milliseconds, or, where the wait
+ *              sleeps, 65536 tries of 4 us).  A limit of 1 makes the waits of
  *              the next call run out at once, which is how the error path of scap_device_status() is exercised
  *              without a fault; y of such a call is incomplete.
  *   "host_direct"  scap_sparse_fc_host: 1 = when x_host and y_host are page-locked and addressable by the

@@ -584,7 +584,7 @@ __device__ __forceinline__ void fc_body(const FcArgs &a, const int tile, const i
     if (S > 1) {
         reduce_send_round<BT, EPI, TNT, NRED, RB>(s_red, 0, B, s, per, smem_addr(s_gather), bar);
         bool landed = false;
-        for (uint32_t it = 0; it < (1u << 22) && !landed; ++it) landed = mbarrier_try_wait(bar, 0);
+        for (uint32_t it = 0; it < TRIES && !landed; ++it) landed = mbarrier_try_wait(bar, 0);
         if (!landed && a.status) atomicCAS(a.status, 0, 2);  // never in a correct run; the result is then incomplete
     } else {
         float *owner[MAX_CLUSTER];

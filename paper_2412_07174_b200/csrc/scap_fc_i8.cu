@@ -127,7 +127,7 @@ __device__ __forceinline__ uint4 ld_act16u(const void *p) {
     asm volatile("ld.global.cg.v4.u32 {%0,%1,%2,%3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "l"(p) : "memory");
     return v;
 }
-// A bounded wait that sleeps in the barrier instead of polling (after a first look).
+// A bounded wait that sleeps in the barrier instead of polling (after a first look); `limit` in tries.
 __device__ __forceinline__ bool i8_wait(unsigned long long *bar, uint32_t parity, int code, volatile int *abort_flag, uint32_t limit, int *status) {
     for (uint32_t i = 0; i < limit; ++i) {
         if (i == 0 ? mbar_test(bar, parity) : mbarrier_try_wait(smem_u32(bar), parity)) return true;
@@ -204,7 +204,7 @@ __global__ void __launch_bounds__(I8_THREADS, 2) fc_i8_kernel(const __grid_const
     float *s_gather = reinterpret_cast<float *>(smem + i8_off_gather(BR));
     I8Misc *misc = reinterpret_cast<I8Misc *>(smem + i8_off_misc(BR));
     volatile int *abort_flag = &misc->abort;
-    const uint32_t spin = a.spin ? (uint32_t)a.spin : TC_SPIN;
+    const uint32_t spin = a.spin ? (uint32_t)a.spin : TRIES;
     int *const status = a.status;
 
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -458,9 +458,9 @@ __global__ void __launch_bounds__(I8_THREADS, 2) fc_i8_kernel(const __grid_const
         // all MMAs have finished, and no copy is under way, before anyone leaves
         int own_abort = 0;
         if (leader) tc_commit(&misc->done);
-        i8_wait(&misc->done, 0, 4, &own_abort, TC_SPIN, status);
+        i8_wait(&misc->done, 0, 4, &own_abort, TRIES, status);
         if (*abort_flag)
-            for (int q = max(0, asked - NW); q < asked; ++q) i8_wait(&misc->wfull[q % NW], (uint32_t)(q / NW) & 1u, 5, &own_abort, TC_SPIN, status);
+            for (int q = max(0, asked - NW); q < asked; ++q) i8_wait(&misc->wfull[q % NW], (uint32_t)(q / NW) & 1u, 5, &own_abort, TRIES, status);
     } else {
         // ---- second pass: the digits
         int blk = ub, rq = uq;
@@ -593,7 +593,7 @@ __global__ void __launch_bounds__(I8_THREADS, 2) fc_i8_kernel(const __grid_const
     if (S > 1) {
         bool landed = false;
 #pragma unroll 1
-        for (uint32_t it = 0; it < (1u << 22) && !landed; ++it) landed = mbarrier_try_wait(recv_bar, 0);
+        for (uint32_t it = 0; it < TRIES && !landed; ++it) landed = mbarrier_try_wait(recv_bar, 0);
         if (!landed && status) atomicCAS(status, 0, 6);  // never in a correct run; the result is then incomplete
     }
     // the S partials of a result in rank order, and the bias

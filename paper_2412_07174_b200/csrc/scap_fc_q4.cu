@@ -338,7 +338,7 @@ __global__ void __launch_bounds__(FC_THREADS, 2) fc_q4_kernel(const Q4Args qa) {
     if (S > 1) {
         reduce_send_round<BT, EPI, TNT, NR, RB>(s_red, 0, B, s, per, smem_addr(s_gather), bar);
         bool landed = false;
-        for (uint32_t it = 0; it < (1u << 22) && !landed; ++it) landed = mbarrier_try_wait(bar, 0);
+        for (uint32_t it = 0; it < TRIES && !landed; ++it) landed = mbarrier_try_wait(bar, 0);
         if (!landed && a.status) atomicCAS(a.status, 0, 2);  // never in a correct run; the result is then incomplete
     } else {
         float *owner[MAX_CLUSTER];

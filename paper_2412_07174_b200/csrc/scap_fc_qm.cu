@@ -381,7 +381,7 @@ __global__ void __launch_bounds__(FC_THREADS, 2) fc_qm_kernel(const QmArgs qa) {
         reduce_send_round<BT, EPI_BIAS, QM_TN, NKG, BT>(s_red, 0, B, s, per, smem_addr(s_gather), bar);
         bool landed = false;
 #pragma unroll 1
-        for (uint32_t it = 0; it < (1u << 22) && !landed; ++it) landed = mbarrier_try_wait(bar, 0);
+        for (uint32_t it = 0; it < TRIES && !landed; ++it) landed = mbarrier_try_wait(bar, 0);
         if (!landed && a.status) atomicCAS(a.status, 0, 2);  // never in a correct run; the result is then incomplete
     } else {
         float *owner[MAX_CLUSTER];

@@ -900,7 +900,7 @@ __global__ void __launch_bounds__(FC_THREADS, 2) fc_ds_kernel(const FcArgs a, co
     if (warp == 0) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(TCOLS) : "memory");
     if (S > 1) {
         bool landed = false;
-        for (uint32_t it = 0; it < (1u << 22) && !landed; ++it) landed = mbarrier_try_wait(recv_bar, 0);
+        for (uint32_t it = 0; it < TRIES && !landed; ++it) landed = mbarrier_try_wait(recv_bar, 0);
         if (!landed) atomicCAS(&g_tc_status, 0, 6);  // never in a correct run; the result is then incomplete
     }
     finish_columns<BF16, GR, EPI, TNT>(a, tile, s, per, s_gather, bias0, bias1);
