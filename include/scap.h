@@ -103,7 +103,8 @@ int scap_version(void);
  *              (0 = the built-in limits, the default: about a million polls, tens of milliseconds, or, where the wait
  *              sleeps, 65536 tries of 4 us).  A limit of 1 makes the waits of
  *              the next call run out at once, which is how the error path of scap_device_status() is exercised
- *              without a fault; y of such a call is incomplete.
+ *              without a fault; y of such a call is incomplete.  It is also the limit of the barrier of a large
+ *              calibration, whose threshold is then a NaN.
  *   "host_direct"  scap_sparse_fc_host: 1 = when x_host and y_host are page-locked and addressable by the
  *              device, a kernel pulls x and the FC kernel writes y to host memory (default), 0 = always copies
  *   "cal_strip"  scap_calibrate: channels per CTA of the per-channel histogram kernel, 16 (default: 256 threads,
@@ -121,9 +122,9 @@ int scap_version(void);
  * after tuning.                                                                               */
 scap_status scap_tune(const char *key, int value);
 
-/* The tcgen05 kernel bounds every wait on a shared-memory barrier; a wait that runs out (which a
- * correct run never does) makes the CTA stop issuing work, so y is then incomplete.  This call
- * synchronises the device, returns SCAP_ERR_TIMEOUT if that happened since the last call (and
+/* Every wait of a kernel on a barrier is bounded; a wait that runs out (which a correct run never
+ * does) makes the CTA stop issuing work, so y is then incomplete (the threshold of a calibration:
+ * a NaN).  This call synchronises the device, returns SCAP_ERR_TIMEOUT if that happened since the last call (and
  * clears the record), SCAP_OK otherwise.  Not for use during stream capture.                   */
 scap_status scap_device_status(void);
 

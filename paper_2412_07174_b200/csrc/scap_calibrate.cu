@@ -31,6 +31,7 @@ struct SelState {
     uint32_t rank[2];    // rank of each within the keys that share its prefix
     uint32_t arrived;    // CTAs of tau_kernel that have counted their middle digits
     uint32_t finished;   // and their last ones
+    uint32_t gave_up;    // one of them did not wait to the end
 };
 
 template <bool BF16>
@@ -491,6 +492,7 @@ __global__ void __launch_bounds__(256) select_kernel(const uint32_t *__restrict_
 // counted (a barrier over the grid, whose CTAs are all resident), the last digits are counted from the lists alone, and the CTA
 // that finishes last interpolates tau = v_j + frac * (v_j1 - v_j) in binary64, each operation rounded once, then to binary32.
 // A warp one of whose lists would overflow (a tensor with few distinct values) does not use them: it reads its part again instead.
+// The barrier's wait is bounded; where it runs out the status word says so and tau is a NaN, which no sparse call takes for a threshold.
 //
 // A CTA owns a block of 256 channels (32 lanes x 8 channels: a warp reads 512 contiguous bytes of a row) and the rows blockIdx.y * 8 + warp,
 // stepping by 8 * gridDim.y; the modes of a thread's 8 channels stay in registers.  The pass is bound by instruction issue, so a key costs
@@ -500,10 +502,12 @@ __global__ void __launch_bounds__(256) select_kernel(const uint32_t *__restrict_
 // 2048 x 14336: 37 us, where two passes and the selection took 70; whole call 126.0 -> 100.1.
 constexpr int TAU_U = 8;         // 16-byte loads in flight per thread
 constexpr int TAU_LIST = 24;     // keys per thread (24 KB, four CTAs per SM); a row adds at most eight
+constexpr uint32_t TAU_POLLS = 1u << 18;  // of the barrier, most of a microsecond each; scap_tune("tc_spin") overrides
 template <bool BF16>
 __global__ void __launch_bounds__(256, 4) tau_kernel(const uint16_t *__restrict__ x, const float *__restrict__ m, int T, int K,
                                                      const uint32_t *__restrict__ hist_a, uint32_t *__restrict__ hist_b, uint32_t *__restrict__ hist_c,
-                                                     SelState *__restrict__ state, uint32_t j, uint32_t j1, double frac, float *__restrict__ tau_out) {
+                                                     SelState *__restrict__ state, uint32_t j, uint32_t j1, double frac, float *__restrict__ tau_out,
+                                                     uint32_t polls, int *status) {
     __shared__ uint32_t s_h[2][RADIX_B];
     __shared__ uint32_t s_list[TAU_LIST][256];
     __shared__ uint32_t s_last;
@@ -607,12 +611,17 @@ __global__ void __launch_bounds__(256, 4) tau_kernel(const uint16_t *__restrict_
     __syncthreads();
     if (tid == 0) {
         atomicAdd(&state->arrived, 1u);
-        // (bounded like every wait; all CTAs are resident, so it ends as soon as the slowest has counted)
-        for (uint32_t it = 0; it < (1u << 24); ++it) {
+        // (all CTAs are resident, so it ends as soon as the slowest has counted)
+        bool all = false;
+        for (uint32_t it = 0; it < polls && !all; ++it) {
             uint32_t seen;
             asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(seen) : "l"(&state->arrived) : "memory");
-            if (seen >= ctas) break;
-            if (it > 256) __nanosleep(64);
+            all = seen >= ctas;
+            if (!all && it > 256) __nanosleep(64);
+        }
+        if (!all) {  // never in a correct run; the counters are incomplete
+            atomicExch(&state->gave_up, 1u);
+            if (status) atomicCAS(status, 0, 7);
         }
     }
     for (int i = tid; i < 2 * RADIX_C; i += 256) (&s_h[0][0])[i] = 0;
@@ -648,7 +657,7 @@ __global__ void __launch_bounds__(256, 4) tau_kernel(const uint16_t *__restrict_
         const double vj = (double)__uint_as_float((p0 << SHIFT_B) | c.bucket[0]);
         const double vj1 = (double)__uint_as_float((p1 << SHIFT_B) | c.bucket[1]);
         const double t64 = __dadd_rn(vj, __dmul_rn(frac, __dsub_rn(vj1, vj)));
-        *tau_out = (float)t64;
+        *tau_out = __ldcg(&state->gave_up) ? __int_as_float(0x7fffffff) : (float)t64;
     }
 }
 
@@ -1236,7 +1245,7 @@ static scap_status calibrate_t(const uint16_t *x, int T, int K, double sparsity,
     cfg.attrs = attr;
     cfg.numAttrs = 1;
     e = cudaLaunchKernelEx(&cfg, tau_kernel<BF16>, x, (const float *)m_out, T, K, (const uint32_t *)hist, hist + RADIX_A, hist + RADIX_A + 2 * RADIX_B,
-                           state, (uint32_t)j, (uint32_t)j1, frac, tau_out);
+                           state, (uint32_t)j, (uint32_t)j1, frac, tau_out, g_tune.tc_spin ? (uint32_t)g_tune.tc_spin : TAU_POLLS, tc_status_ptr());
     if (e == cudaErrorCooperativeLaunchTooLarge) {  // a context that was given fewer SMs than the device has: in passes, from the start
         cudaGetLastError();
         return calibrate_t<BF16>(x, T, K, sparsity, estimator, scalar, nbins, m_out, tau_out, ws, st, false);

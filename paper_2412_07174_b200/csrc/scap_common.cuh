@@ -32,6 +32,7 @@ extern Tuning g_tune;
 // ---- status helpers -------------------------------------------------------------------------
 scap_status check_device();  // SCAP_OK on compute capability 10.x
 int sm_count();              // multiprocessors of the current device (148 when no device is present)
+int *tc_status_ptr();        // device address of the status word of the bounded waits on the current device (NULL if it cannot be had)
 
 inline bool aligned16(const void *p) { return (reinterpret_cast<uintptr_t>(p) & 15u) == 0; }
 inline size_t align_up(size_t v, size_t a) { return (v + a - 1) / a * a; }

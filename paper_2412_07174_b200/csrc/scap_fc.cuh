@@ -1048,7 +1048,6 @@ int tc_take_status();
 bool ds_applicable(const FcArgs &a, int epi, bool bf16);
 int ds_choose_split(int K, int Nh, int epi);
 cudaError_t launch_fc_ds(bool bf16, int mode, int xkind, int epi, const FcArgs &a, cudaStream_t st);
-int *tc_status_ptr();  // device address of that status word on the current device (NULL if it cannot be had)
 
 // Launch with cluster dimension (1, S, 1) and, if enabled, programmatic dependent launch.
 template <typename... KArgs, typename... Args>

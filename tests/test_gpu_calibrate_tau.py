@@ -65,3 +65,21 @@ def test_order_statistics_in_different_buckets(S, gap, T, K):
     """j and j + 1 fall on either side of a jump that separates their last, middle or first digits (no centring: the values are the keys)."""
     v = np.where(np.arange(T * K).reshape(T, K) < T * K // 2, 1.0, 1.0 + gap)
     check(S, v, si.BF16, (T * K // 2 - 0.75) / (T * K - 1), nbins=0)
+
+
+def test_a_barrier_that_runs_out_is_reported_and_the_next_call_is_right(S):
+    """With a limit of one poll most CTAs do not see the others arrive: the call returns, the status word is set, the threshold is no number."""
+    x = dev(si.to_bits(normal(2048, 5128), si.BF16), si.BF16)
+    ws, m, tau = workspace(S.scap_calibrate_workspace(2048, 5128, 64)), torch.empty(5128, device="cuda"), torch.zeros(1, device="cuda")
+    S.scap_device_status()
+    try:
+        S.scap_tune("tc_spin", 1)
+        S.scap_calibrate(x, 0.5, 64, m, tau, ws.payload)
+        with pytest.raises(S.ScapError) as err:
+            S.scap_device_status()
+        assert err.value.code == 7  # SCAP_ERR_TIMEOUT
+        assert ws.intact() and torch.isnan(tau).all()
+    finally:
+        S.scap_tune("tc_spin", 0)
+    check(S, normal(2048, 5128), si.BF16, 0.5)
+    S.scap_device_status()
