@@ -647,7 +647,7 @@ static cudaError_t launch_i8_x(const FcArgs &a, const CUtensorMap &map, cudaStre
 }
 
 // Split-K factor: the most CTAs that are all resident (two per SM), at least one block per rank.
-static int i8_split(const FcArgs &a) {
+int i8_split(const FcArgs &a) {
     const int tiles = (a.ldw + I8_TN - 1) / I8_TN, blocks = (a.K + I8_KB - 1) / I8_KB;
     int best_S = 1;
     long long best = -1;
@@ -660,21 +660,17 @@ static int i8_split(const FcArgs &a) {
     return best_S;
 }
 
-int i8_blocks_per_rank(const FcArgs &a) {
-    const int S = i8_split(a);
-    return ((a.K + I8_KB - 1) / I8_KB + S - 1) / S;
-}
+int i8_blocks_per_rank(const FcArgs &a, int S) { return ((a.K + I8_KB - 1) / I8_KB + S - 1) / S; }
 
 // Rows of x and of the codes must lie on 16-byte boundaries (vector loads, stride of the tensor map), and the 32-bit sums must hold a
 // rank's channels (2^14 per product).
-bool i8_applicable(const FcArgs &a) {
-    return a.K % 8 == 0 && a.ldw % 16 == 0 && a.B >= 1 && a.B <= 16 && !a.hold_dependents && aligned16(a.wscale) && i8_blocks_per_rank(a) <= 512;
+bool i8_applicable(const FcArgs &a, int blocks_per_rank) {
+    return a.K % 8 == 0 && a.ldw % 16 == 0 && a.B >= 1 && a.B <= 16 && !a.hold_dependents && aligned16(a.wscale) && blocks_per_rank <= 512;
 }
 
 cudaError_t launch_fc_i8(int mode, int xkind, FcArgs a, cudaStream_t st) {
     CUtensorMap map;
     if (!i8_tensor_map(&map, a.W, a.K, a.ldw)) return cudaErrorNotSupported;
-    a.S = i8_split(a);
     a.status = tc_status_ptr();
     a.spin = g_tune.tc_spin;
     if (mode == MODE_DENSE) return xkind == 1 ? launch_i8_x<MODE_DENSE, __nv_bfloat16>(a, map, st) : launch_i8_x<MODE_DENSE, __half>(a, map, st);

@@ -56,9 +56,13 @@ static cudaError_t launch_q8_t(const FcArgs &a, cudaStream_t st) {
 // (1024 x 4096) 5.9 -> 6.3, 4.7 -> 7.0, 6.3 -> 8.2.  With one and two rows the FMA kernel below reads the kept rows only (11008 x 4096,
 // one row 10.0 against 10.8, two rows 12.7 against 11.1 at 50 % but 9.5 at 80 %); with three it needs a second launch
 // over the codes.
-static bool q8_in_integers(const FcArgs &a) {
-    if (g_tune.dense_stream == 0 || !i8_applicable(a)) return false;
-    return g_tune.dense_stream >= 2 || (a.B >= 3 && i8_blocks_per_rank(a) >= (a.B <= 4 ? 2 : 4));
+// (The rows are looked at first: the split is a search that the calls of one and two rows, which are bound by the host, do without.)
+static bool q8_in_integers(FcArgs &a) {
+    if (g_tune.dense_stream == 0 || (a.B < 3 && g_tune.dense_stream < 2)) return false;
+    const int S = i8_split(a), blocks = i8_blocks_per_rank(a, S);
+    if (!i8_applicable(a, blocks) || (g_tune.dense_stream < 2 && blocks < (a.B <= 4 ? 2 : 4))) return false;
+    a.S = S;
+    return true;
 }
 
 // Calls that take the mma.sync kernel (scap_fc_qm.cu, same tune key): what is left of three and more rows - short layers, and K not a
@@ -78,7 +82,8 @@ static cudaError_t launch_q8(int mode, int xkind, FcArgs a, cudaStream_t st) {
     QmArgs qm;
     memset(&qm, 0, sizeof(qm));
     qm.f = a;
-    if (xkind != 2 && q8_in_integers(a)) return launch_fc_i8(mode, xkind, a, st);
+    FcArgs ai = a;
+    if (xkind != 2 && q8_in_integers(ai)) return launch_fc_i8(mode, xkind, ai, st);
     if (xkind != 2 && q8_on_tensor_cores(qm)) return launch_fc_qm(8, mode, xkind, qm, st);
     const size_t xsz = xkind == 2 ? 4 : 2;
     const unsigned char *x0 = static_cast<const unsigned char *>(a.x);

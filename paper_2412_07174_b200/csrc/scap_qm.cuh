@@ -21,8 +21,9 @@ int qm_blocks_per_warp(const QmArgs &a);
 cudaError_t launch_fc_qm(int wbits, int mode, int xkind, QmArgs a, cudaStream_t st);
 
 // 8-bit weights on the 5th-generation tensor cores in integers (scap_fc_i8.cu).
-bool i8_applicable(const FcArgs &a);
-int i8_blocks_per_rank(const FcArgs &a);  // blocks of 128 channels
-cudaError_t launch_fc_i8(int mode, int xkind, FcArgs a, cudaStream_t st);
+int i8_split(const FcArgs &a);                    // split-K factor
+int i8_blocks_per_rank(const FcArgs &a, int S);  // blocks of 128 channels
+bool i8_applicable(const FcArgs &a, int blocks_per_rank);
+cudaError_t launch_fc_i8(int mode, int xkind, FcArgs a, cudaStream_t st);  // a.S: the split-K factor
 
 }  // namespace scap
