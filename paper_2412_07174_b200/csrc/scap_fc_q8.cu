@@ -83,7 +83,10 @@ static cudaError_t launch_q8(int mode, int xkind, FcArgs a, cudaStream_t st) {
     memset(&qm, 0, sizeof(qm));
     qm.f = a;
     FcArgs ai = a;
-    if (xkind != 2 && q8_in_integers(ai)) return launch_fc_i8(mode, xkind, ai, st);
+    if (xkind != 2 && q8_in_integers(ai)) {
+        const cudaError_t e = launch_fc_i8(mode, xkind, ai, st);
+        if (e != cudaErrorNotSupported) return e;  // (no tensor map to be had, nothing launched: the kernels below need none)
+    }
     if (xkind != 2 && q8_on_tensor_cores(qm)) return launch_fc_qm(8, mode, xkind, qm, st);
     const size_t xsz = xkind == 2 ? 4 : 2;
     const unsigned char *x0 = static_cast<const unsigned char *>(a.x);
