@@ -95,7 +95,7 @@ int scap_version(void);
  *              2 = the dense-stream kernel from batch 3 on.
  *              8- and 4-bit weights: 1 = the tensor-core kernel, which reads every row of codes, from batch 3 on and for
  *              small layers at batch 1 and 2; 0 = the FMA kernels, which fetch kept rows only and take two rows at a time
- *              (better for 8-bit calls of three or four rows that prune more than about 80 %); 2 = the tensor-core
+ *              (better for 8-bit calls of four rows that prune more than about 95 %); 2 = the tensor-core
  *              kernel wherever it can run.
  *              Grouped calls: 0 = always one gather per group (better when the rows of a group keep the very same
  *              channels, and less than about a fifth of them); else see scap_sparse_fc_grouped

@@ -51,16 +51,21 @@ static cudaError_t launch_q8_t(const FcArgs &a, cudaStream_t st) {
 }
 
 // Calls that take the integer kernel (scap_fc_i8.cu; tune "dense_stream": 0 none, 2 all it can take): three and more rows, of a layer
-// that is long enough for its longer start.  us, half pruned, scap_fc_qm.cu -> integers: four blocks of 128 channels per rank (K = N =
-// 4096) three rows 9.3 -> 7.2, eight 10.5 -> 8.2, sixteen 17.2 -> 10.5; two blocks (2048 x 4096) 7.0 -> 6.3, 6.6 -> 7.2, 9.9 -> 8.6; one
-// (1024 x 4096) 5.9 -> 6.3, 4.7 -> 7.0, 6.3 -> 8.2.  With one and two rows the FMA kernel below reads the kept rows only (11008 x 4096,
-// one row 10.0 against 10.8, two rows 12.7 against 11.1 at 50 % but 9.5 at 80 %); with three it needs a second launch
-// over the codes.
+// that is long enough for its longer start - two blocks of 128 channels per rank, and three from five rows on.  us, half pruned,
+// scap_fc_qm.cu -> integers, N = 4096 and N = 1024 at one, two, three and four blocks per rank (K = 1024 .. 4096):
+//   three rows    5.7 -> 6.3    7.0 -> 6.5          -> 7.0     9.0 -> 7.3  |                  -> 4.6           -> 5.0
+//   eight rows    4.6 -> 6.9    6.3 -> 7.2    8.3 -> 8.0    10.2 -> 8.3  |       4.6 -> 5.0    6.5 -> 5.5
+//   nine rows     5.8 -> 7.2    9.2 -> 8.0   12.9 -> 8.5             |       5.0 -> 5.7    6.8 -> 6.1
+//   sixteen rows  6.2 -> 7.7    9.7 -> 8.6   13.4 -> 10.0   17.0 -> 10.9 |       5.3 -> 6.1    7.1 -> 7.4
+// (From nine rows on two blocks would do where there are many tiles, and not where there are few.)  With one and two rows the FMA
+// kernel below reads the kept rows only (11008 x 4096, 50 / 80 % pruned: one row 9.9 / 6.5 against 11.7, two rows 12.7 / 9.6 against
+// 12.1); with three it needs a second launch over the codes, which pays at 95 % pruned at most (three rows 21.6 / 16.9 / 14.3 /
+// 13.2 at 50 / 80 / 90 / 95 % against 12.4, four rows 24.7 / 18.7 / 14.6 / 12.1 against 12.8, five rows 33.3 / 25.7 / 22.6 / 20.1 against 13.7).
 // (The rows are looked at first: the split is a search that the calls of one and two rows, which are bound by the host, do without.)
 static bool q8_in_integers(FcArgs &a) {
     if (g_tune.dense_stream == 0 || (a.B < 3 && g_tune.dense_stream < 2)) return false;
     const int S = i8_split(a), blocks = i8_blocks_per_rank(a, S);
-    if (!i8_applicable(a, blocks) || (g_tune.dense_stream < 2 && blocks < (a.B <= 4 ? 2 : 4))) return false;
+    if (!i8_applicable(a, blocks) || (g_tune.dense_stream < 2 && blocks < (a.B <= 4 ? 2 : 3))) return false;
     a.S = S;
     return true;
 }

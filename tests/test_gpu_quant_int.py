@@ -159,9 +159,10 @@ def test_a_wait_that_runs_out_is_reported_and_the_next_call_is_right(S):
 
 
 @pytest.mark.parametrize("K,N,B,same", [(4096, 4096, 3, True), (4096, 4096, 16, True), (2048, 1024, 4, True), (2048, 1024, 5, False),
-                                        (4092, 4096, 8, False), (4096, 4096, 2, False)])
+                                        (4092, 4096, 8, False), (4096, 4096, 2, False), (3072, 1024, 5, True), (3072, 1024, 16, True),
+                                        (2048, 1024, 16, False), (1024, 1024, 3, False)])
 def test_which_calls_take_it(S, K, N, B, same):
-    """By default: three and more rows, four blocks of 128 channels per rank (two up to four rows), K a multiple of eight."""
+    """By default: three and more rows, three blocks of 128 channels per rank (two up to four rows), K a multiple of eight."""
     d, _, q, scale = layer(K, N, B, si.BF16)
     x, args, ws = dev(d["x"], si.BF16), (torch.from_numpy(q).cuda(), f32(scale)), workspace(S.scap_fc_workspace(B, K, N))
     out = []

@@ -1,6 +1,7 @@
 """The tensor-core kernel of the quantised calls (scap_fc_qm.cu) at the edges of its tiles: remainders of the 16-channel
 blocks, of the 128-column tiles and of the scale groups, every row layout, each activation type, sparse and dense, every cluster
-size - and the calls that it does not take, which run on the fp32-FMA kernels two rows at a time.
+size - and the calls that it does not take, which run on the fp32-FMA kernels two rows at a time.  (8-bit calls with K a multiple of eight run
+on the integer kernel here; this one has those of K a multiple of four only, which every test has too.)
 
 Bound: the codes and the three parts of an activation are exact and their products are too.  What is left: an accumulator takes at
 most K / 64 products of 16 channels (four or eight warps, at least one rank), each of which truncates it by at most 2^-23 of its
@@ -26,6 +27,11 @@ SHAPES = [  # K, N, B, group
     (516, 1040, 9, 256),    # two halves of the batch, five and four rows
     (1504, 272, 11, 32),
     (2304, 784, 16, 2048),  # a group longer than a rank's range
+    # the same places with K four short of a multiple of eight, for the 8-bit codes
+    (68, 144, 1, 32),
+    (1004, 144, 4, 96),
+    (1508, 272, 11, 32),
+    (2308, 784, 16, 2048),
 ]
 
 
@@ -82,11 +88,12 @@ def test_quantised_rows_match_the_oracle(S, bits, K, N, B, group, dt):
 @pytest.mark.parametrize("bits", [8, 4])
 @pytest.mark.parametrize("split", [1, 3, 5, 6, 7])
 @pytest.mark.parametrize("B", [1, 2, 3, 8, 13])
-def test_every_cluster_size(S, bits, split, B):
+@pytest.mark.parametrize("K", [1000, 1004])
+def test_every_cluster_size(S, bits, split, B, K):
     """One rank, and ranks whose slices of the columns together are longer than the tile."""
     try:
         S.scap_tune("split_k", split)
-        check(S, bits, 1000, 272, B, 32, si.BF16)
+        check(S, bits, K, 272, B, 32, si.BF16)
     finally:
         S.scap_tune("split_k", 0)
 
@@ -126,10 +133,11 @@ def test_either_side_of_the_limit_of_scale_groups(S, K):
 
 @pytest.mark.parametrize("bits", [8, 4])
 @pytest.mark.parametrize("B", [1, 4, 16])
-def test_a_few_large_activations_do_not_cost_the_others_their_bits(S, bits, B):
+@pytest.mark.parametrize("K", [14336, 14332])
+def test_a_few_large_activations_do_not_cost_the_others_their_bits(S, bits, B, K):
     """A truncating accumulator that holds a large value early loses up to 2^-23 of it with every further product, so its chain has to be
     short: eight products (8-bit) or a scale group of 128 channels (4-bit), and a handful of additions after it."""
-    K, N = 14336, 144
+    N = 144
     d = si.laplace_fc(4, K, N, si.BF16, 16, B)
     x = si.to_f32(d["x"], si.BF16).astype(np.float64)
     x[:, ::K // 8] = 300.0 * (1 + np.arange(B))[:, None]  # the first channel of every warp's stretch
@@ -154,9 +162,10 @@ def test_a_few_large_activations_do_not_cost_the_others_their_bits(S, bits, B):
 
 
 @pytest.mark.parametrize("bits", [8, 4])
-def test_an_infinite_activation_stays_in_its_row(S, bits):
+@pytest.mark.parametrize("K", [256, 260])
+def test_an_infinite_activation_stays_in_its_row(S, bits, K):
     """Row 0 holds an infinity, row 1 a NaN that the threshold drops: row 0 is non-finite, the others are as without them."""
-    K, N, B = 256, 144, 3
+    N, B = 144, 3
     d = si.laplace_fc(4, K, N, si.BF16, 16, B)
     if bits == 8:
         q, scale = si.quantise_q8(d["W"], si.BF16)
@@ -182,9 +191,10 @@ def test_an_infinite_activation_stays_in_its_row(S, bits):
 @pytest.mark.parametrize("bits", [8, 4])
 @pytest.mark.parametrize("B", [1, 2, 3, 5])
 @pytest.mark.parametrize("special", [float("inf"), float("nan")])
-def test_a_scale_that_no_kept_channel_uses_has_no_effect(S, bits, B, special):
+@pytest.mark.parametrize("K", [256, 260])
+def test_a_scale_that_no_kept_channel_uses_has_no_effect(S, bits, B, special, K):
     """Channels 64..95 (one scale group of 32) are dropped by every row: their scales are not part of any sum, whatever they hold."""
-    K, N = 256, 144
+    N = 144
     d = si.laplace_fc(4, K, N, si.BF16, 16, B)
     x = dev(d["x"], si.BF16)
     x[:, 64:96] = 0.0
