@@ -168,17 +168,28 @@ static cudaError_t launch_moe_fc_t(const MoeArgs &a, int tiles, int S, cudaStrea
     return tn == 128 ? launch_moe_fc_tn<BF16, BT, STAGE, 128>(a, tiles, S, st) : launch_moe_fc_tn<BF16, BT, STAGE, 256>(a, tiles, S, st);
 }
 
-// Three and four tokens: the kernel with a body for each count of rows, from this many input channels per split-K rank; below, the
-// one with fewer bodies (that of five to eight tokens).  A CTA that streams few channels spends its time at the start, and two
-// CTAs of an SM in different bodies fetch their code twice.  Whole layer, top 2 of 8 experts, four tokens, us, fewer -> more bodies:
-// D = 1024, F = 2048 26.7 -> 28.2; D = 2048, F = 7168 (1792 and 2048 channels per rank) 80.8 -> 74.8; D = 4096, F = 14336 257.9 -> 247.2.
-// Two tokens, where the two-row body used to take single rows as well: 149.1 -> 138.2, D = 1024, F = 2048 20.5 -> 19.9.
-constexpr int EXACT_ROWS_FROM = 1536;
+// Three and four tokens: both FCs in the kernel with a body for each count of rows, or both in the one with fewer bodies (that of five to
+// eight tokens).  In a small layer a CTA spends its time at the start, and two CTAs of an SM in different bodies fetch their code
+// twice; what the exact bodies save grows with the weights of an expert and with the share of single rows.  Whole layer, us, fewer
+// -> more bodies, means over six routings (three from D = 3072 on), three and four tokens:
+//   D x F           top 1 of 8                   top 2 of 8                     top 2 of 4
+//   1024 x 2048     - -> -       21.2 -> 21.9    - -> -         27.0 -> 28.4    22.0 -> 23.0    23.8 -> 24.8
+//   1024 x 3072     21.5 -> 21.1 24.8 -> 24.7    27.6 -> 29.4   34.4 -> 34.9    26.9 -> 28.1    30.3 -> 30.8
+//   1024 x 5120     26.0 -> 25.0 31.8 -> 30.6    36.7 -> 36.8   39.7 -> 40.4    34.9 -> 34.5    38.0 -> 37.0
+//   1536 x 4096     29.1 -> 27.5 30.9 -> 30.6    43.3 -> 42.6   47.5 -> 47.0    34.4 -> 34.8    37.8 -> 37.6
+//   1024 x 8192     33.2 -> 31.1 35.9 -> 35.0    47.9 -> 45.5   57.1 -> 52.8    39.8 -> 39.4    44.7 -> 43.3
+//   3072 x 6144     48.5 -> 45.5 71.2 -> 66.9    87.2 -> 82.5  106.3 -> 104.0   77.7 -> 74.1    89.7 -> 80.2
+//   4096 x 14336   135.7 -> 123.0 154.4 -> 141.0 224.0 -> 204.9 260.2 -> 248.2 184.2 -> 175.0 216.6 -> 206.0
+// One FC in each kind gained less, and lost at some sizes (3072 x 6144, four tokens, top 2 of 8: 109.6 with the first FC only).
+// Two tokens, where the two-row body used to take single rows as well, top 2 of 8: 4096 x 14336 150.1 -> 137.9, 1024 x 2048 21.7 -> 20.8.
+static bool exact_rows(const MoeArgs &a) {
+    const long long from = 2 * a.B * a.top_k <= a.E ? 3ll << 20 : 6ll << 20;
+    return a.B >= 3 && a.B <= 4 && (long long)a.D * a.F >= from;
+}
 
 template <bool BF16, int STAGE>
 static cudaError_t launch_moe_fc(const MoeArgs &a, int tiles, int S, cudaStream_t st) {
-    const bool exact = a.B >= 3 && a.B <= 4 && (STAGE == 1 ? a.D : a.F) >= EXACT_ROWS_FROM * S;
-    switch (exact ? 4 : batch_tile(a.B)) {
+    switch (exact_rows(a) ? 4 : batch_tile(a.B)) {
         case 1: return launch_moe_fc_t<BF16, 1, STAGE>(a, tiles, S, st);
         case 2: return launch_moe_fc_t<BF16, 2, STAGE>(a, tiles, S, st);
         case 4: return launch_moe_fc_t<BF16, 4, STAGE>(a, tiles, S, st);
