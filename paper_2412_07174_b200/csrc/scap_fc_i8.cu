@@ -22,11 +22,14 @@
 // in binary32, a rounding per limb and one between two limbs.
 //
 // What bounds it: K = 11008, N = 4096, half pruned, weights from DRAM, us per call, mma.sync kernel -> this one: 3 rows
-// 18.1 -> 12.3, 8 rows 23.8 -> 14.5, 16 rows 41.0 -> 20.0 (the 45 MB of codes take 6.9 at copy speed).  The first MMA starts 3 - 4 us
+// 18.1 -> 12.3, 8 rows 23.8 -> 14.6, 16 rows 41.0 -> 19.4 (the 45 MB of codes take 6.9 at copy speed).  The first MMA starts 3 - 4 us
 // into the call: activations through L2 (1 us under the weight stream), the pass for the exponents, the digits - code that all 24
 // warps of an SM run at once, bound by instruction issue - while the ring has been full for two of them.  So a limb comes off a value by
-// additions and multiply-adds, where a conversion to an integer takes four issue slots, and six digits cost what four by
-// conversion did (3 / 8 / 16 rows 12.4 / 14.9 / 20.0, K = 4096 with its four blocks per rank 7.0 / 8.0 / 10.1 against 7.3 / 8.3 / 10.9).
+// additions and multiply-adds, where a conversion to an integer takes four issue slots, and whether a value lies below the digits' window is
+// asked only where the threshold and the scales do not rule it out (16 rows 20.1 -> 19.4).  Six digits then cost what four by
+// conversion did in a long layer (3 / 8 / 11 / 16 rows 12.5 / 14.9 / 17.7 / 20.3 -> 12.3 / 14.6 / 15.7 / 19.4) and more in a short one (K = 4096, four
+// blocks per rank, 7.0 / 8.0 / 9.3 / 10.1 -> 7.2 / 8.2 / 9.7 / 10.7).  Values below the window cost time at the end (dense, 8 rows: none 14.6, one
+// in 10^5 17.5, a tenth 74, nearly all 330).
 // Tried and slower: an exponent per block and an accumulator per block or two, so that the first MMA does not
 // wait for a pass over all activations (8 rows 15.4 - 16.3, 16 rows 21.5 - 30.6: reading 11 accumulators costs more than the pass);
 // 256 threads (15.4); 4-bit codes the same way, the nibbles separated in shared memory (11008 x 4096, one row 15.4 - 27 against 13.0:
@@ -84,6 +87,7 @@ struct I8Misc {
     int abort;
     uint32_t top[16], fin[16];  // pattern of a row's largest magnitude; of the largest finite one
     uint32_t apart;             // rows with a value too small for the digits
+    uint32_t scale;             // pattern of the rank's smallest scale magnitude
 };
 struct I8Entry {
     float v;
@@ -225,6 +229,7 @@ __global__ void __launch_bounds__(I8_THREADS, 2) fc_i8_kernel(const __grid_const
         mbar_init(&misc->done, 1);
         misc->abort = 0;
         misc->apart = 0;
+        misc->scale = 0x7fffffffu;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         if (S > 1) {
             const int owned = max(0, min(per, I8_TN - s * per));
@@ -322,6 +327,12 @@ __global__ void __launch_bounds__(I8_THREADS, 2) fc_i8_kernel(const __grid_const
         auto largest = [&](const Raw &raw, float (&v)[4][4]) {
             const int b0 = rq * 4;
             uint32_t top[4];
+            if (MODE == MODE_GATHER && rq == 0) {  // the smallest scale (beyond the matrix there is none)
+                const float *ce = reinterpret_cast<const float *>(&raw.c);
+                const uint32_t t = min(min(i8_bits(ce[0]), i8_bits(ce[1])), min(i8_bits(ce[2]), i8_bits(ce[3])));
+                const uint32_t least = __reduce_min_sync(0xffffffffu, k_lo + blk * I8_KB + lane * 4 < k_hi ? t : 0x7fffffffu);
+                if (lane == 0) atomicMin(&misc->scale, least);
+            }
 #pragma unroll
             for (int r = 0; r < 4; ++r) {
                 if (b0 + r < B) {
@@ -465,7 +476,11 @@ __global__ void __launch_bounds__(I8_THREADS, 2) fc_i8_kernel(const __grid_const
         // ---- second pass: the digits
         int blk = ub, rq = uq;
         const int shifts = lane < BR ? i8_shift(misc->top[lane]) : 0;  // lane b: of row b
-        auto digits = [&](const float (&v)[4][4]) -> bool {
+        // Rows that can have a value without digits: a kept one is no smaller than the threshold times the smallest scale (products are
+        // rounded alike), which mostly settles it for the whole rank.
+        const bool can = lane < B && (MODE == MODE_DENSE || odd || !(__fmul_rn(tau, __uint_as_float(misc->scale)) >= i8_least(shifts)));
+        const uint32_t check = __ballot_sync(0xffffffffu, can);
+        auto digits = [&](float (&v)[4][4]) -> bool {
             const int i = blk / BPS;
             const uint32_t xs = (uint32_t)i % NX;
             if (i >= NX && !warp_wait(&misc->xempty[(uint32_t)(i - NX) % NE], ((uint32_t)(i - NX) / NE) & 1u, 1)) return false;
@@ -474,27 +489,29 @@ __global__ void __launch_bounds__(I8_THREADS, 2) fc_i8_kernel(const __grid_const
             for (int r = 0; r < 4; ++r) {
                 if (rq * 4 + r < B) {
                     const int shift = __shfl_sync(0xffffffffu, shifts, rq * 4 + r);
-                    const float up = i8_pow2(shift), least = i8_least(shift);
-                    float w[4] = {v[r][0], v[r][1], v[r][2], v[r][3]};
-                    bool some = odd != 0;
+                    const float up = i8_pow2(shift);
+                    if (check >> (rq * 4 + r) & 1u) {
+                        const float least = i8_least(shift);
+                        bool some = odd != 0;
 #pragma unroll
-                    for (int e = 0; e < 4; ++e) some |= fabsf(w[e]) < least && w[e] != 0.0f;
-                    if (some) {  // (rare)
+                        for (int e = 0; e < 4; ++e) some |= fabsf(v[r][e]) < least && v[r][e] != 0.0f;
+                        if (some) {  // (rare)
 #pragma unroll
-                        for (int e = 0; e < 4; ++e) {
-                            if (i8_is_apart(w[e], least)) {
-                                w[e] = 0.0f;
-                                atomicOr(&misc->apart, 1u << (rq * 4 + r));
+                            for (int e = 0; e < 4; ++e) {
+                                if (i8_is_apart(v[r][e], least)) {
+                                    v[r][e] = 0.0f;
+                                    atomicOr(&misc->apart, 1u << (rq * 4 + r));
+                                }
                             }
                         }
                     }
-                    // Limbs from the top, rounded to the nearest integer by adding 1.5 x 2^23; 0x8080 more, and the lower 16 bits of the sum are
-                    // two signed digits with their signs turned round.  What is left of a value is exact at every step.
-                    constexpr float M = 12582912.0f + 32896.0f;
+                    // Limbs from the top, rounded to the nearest integer by adding 1.5 x 2^23; 128 more, and the second byte of the sum is the upper
+                    // digit, the first one the lower digit with its sign turned round.  What is left of a value is exact at every step.
+                    constexpr float M = 12582912.0f + 128.0f;
                     uint32_t t[3][4];
 #pragma unroll
                     for (int e = 0; e < 4; ++e) {
-                        const float t2 = __fmaf_rn(w[e], up, M), d1 = __fmaf_rn(w[e], up, -__fsub_rn(t2, M));
+                        const float t2 = __fmaf_rn(v[r][e], up, M), d1 = __fmaf_rn(v[r][e], up, -__fsub_rn(t2, M));
                         const float t1 = __fmaf_rn(d1, 32768.0f, M), d0 = __fmaf_rn(d1, 32768.0f, -__fsub_rn(t1, M));
                         t[0][e] = __float_as_uint(__fmaf_rn(d0, 32768.0f, M));
                         t[1][e] = __float_as_uint(t1);
@@ -504,7 +521,7 @@ __global__ void __launch_bounds__(I8_THREADS, 2) fc_i8_kernel(const __grid_const
                     for (int l = 0; l < 3; ++l) {  // digit x BR + row: the lowest first
                         const uint32_t t01 = __byte_perm(t[l][0], t[l][1], 0x5140), t23 = __byte_perm(t[l][2], t[l][3], 0x5140);
                         *reinterpret_cast<uint32_t *>(dst + (2 * l * BR + r) * 16) = __byte_perm(t01, t23, 0x5410) ^ 0x80808080u;
-                        *reinterpret_cast<uint32_t *>(dst + ((2 * l + 1) * BR + r) * 16) = __byte_perm(t01, t23, 0x7632) ^ 0x80808080u;
+                        *reinterpret_cast<uint32_t *>(dst + ((2 * l + 1) * BR + r) * 16) = __byte_perm(t01, t23, 0x7632);
                     }
                 }
             }
