@@ -121,18 +121,21 @@ scap_status scap_sparse_fc_grouped(const void *x, const void *W, const float *m,
     // to four rows stays on the gather: such a group runs on the FMA bodies there, in binary32 and rounded to nearest, and
     // what a row gets does not depend on the size of another row's group.)  Device time, us, gather -> stream,
     // rows of a group with nine tenths of their pattern in common, 50 % / 80 % pruned | with all of it, 65 / 80 / 90 %:
-    //   11008 x 4096   2 x 6 rows  40 /  33 -> 22 | 27 / 21 / 17 -> 22
-    //                  4 x 8 rows  73 /  58 -> 35 | 46 / 36 / 28 -> 35
-    //                  8 x 8 rows 136 / 104 -> 67 | 79 / 61 / 48 -> 67
-    //    4096 x 4096   2 x 6 rows  23 /  20 -> 14 | 18 / 15 / 13 -> 13
-    //                  4 x 8 rows  33 /  28 -> 19 | 23 / 19 / 16 -> 19
-    //                  8 x 8 rows  58 /  47 -> 36 | 37 / 30 / 25 -> 36
-    //    2048 x 1024   2 x 6 rows  12 /  12 ->  7   4 x 8 rows 13 / 13 -> 10   8 x 8 rows 16 / 14 -> 19
-    //   14336 x 2048   2 x 6 rows  35 /  30 -> 24   4 x 8 rows 53 / 43 -> 40   8 x 8 rows 93 / 71 -> 78
+    //   11008 x 4096   2 x 6 rows  40 /  32 -> 19 | 26 / 21 / 17 -> 19
+    //                  4 x 8 rows  72 /  58 -> 28 | 45 / 35 / 28 -> 28
+    //                  8 x 8 rows 134 / 103 -> 54 | 79 / 61 / 47 -> 54
+    //    4096 x 4096   2 x 6 rows  22 /  19 -> 10 | 16 / 14 / 12 -> 10
+    //                  4 x 8 rows  33 /  27 -> 14 | 23 / 19 / 16 -> 14
+    //                  8 x 8 rows  56 /  45 -> 28 | 36 / 29 / 24 -> 28
+    //    2048 x 1024   2 x 6 rows  12 /  12 -> 5.5   4 x 8 rows 13 / 12 -> 7.5   8 x 8 rows 16 / 14 -> 15 | 13 / 12 / 11 -> 15
+    //   14336 x 2048   2 x 6 rows  35 /  30 -> 19   4 x 8 rows 52 / 42 -> 32 | 34 / 27 / 22 -> 32
+    //                  8 x 8 rows  92 /  71 -> 61 | 55 / 44 / 34 -> 61
     // The masks are not known here.  Rows that keep exactly the same channels, fewer than a fifth of them, are the one kind of
-    // call that loses by the stream (at 90 % pruned up to 1.4 times the time); a caller who has them sets "dense_stream" 0.
+    // call that loses by the stream (64 rows at 90 % pruned: up to 1.2 times the time); a caller who has them sets "dense_stream" 0.
     // Above 16 rows it is bound by the preparation of the activations, which takes two CTAs on most SMs to hide, while the
-    // groups of a gather fill an empty chip themselves: there it needs a full grid, or a short layer and one pass.
+    // groups of a gather fill an empty chip themselves: there it needs a full grid, or a short layer and one pass.  (Longer layers
+    // without a full grid win by the stream too where the rows of a group differ, and lose up to 1.8 times where they do not:
+    // the last lines of the table; they stay on the gather.)
     const int s_ds = ds_choose_split(K, N, EPI_BIAS);
     const bool full_grid = 2 * fc_tiles(N, EPI_BIAS, 128) * s_ds >= 3 * sm_count();
     if (min_nb > 4 && g_tune.dense_stream != 0 && K >= 64 && (B <= 16 || full_grid || (B <= 32 && K <= 4096))) {
