@@ -118,7 +118,7 @@ int scap_version(void);
  *              column tile of a call reads again, are kept (evict_last); weight rows, read once, go first
  *              (evict_first); 0 = no hints
  * Unknown keys return SCAP_ERR_INVALID_ARG.  Tuning never changes what is computed; split_k
- * changes the (fixed) summation order and therefore the last bits of y.  Query workspace sizes
+ * and the keys that choose a kernel change the (fixed) summation order and therefore the last bits of y.  Query workspace sizes
  * after tuning.                                                                               */
 scap_status scap_tune(const char *key, int value);
 
